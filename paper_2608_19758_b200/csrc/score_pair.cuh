@@ -250,42 +250,44 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     }
   } else if (warp == 9) {
     // ---------------- UMMA issuer: acc[chunk & 1] = kbar_hi Q^T + kbar_lo Q^T over the unit's one or two tiles ----------------
-    if (lane == 0) {
-      uint32_t pc = 0, ac0 = 0, ac1 = 0, gc0 = 0;   // gc0: chunks of all earlier units
-      for (int it = 0;; ++it) {
-        const int slot = it % kPairInfoSlots, qb = it % kPairQBufs;
-        mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 131);
-        const PairInfo& pi = info[slot];
-        if (!pi.valid) break;
-        const int nchunks = unit_chunks(pi);
-        const uint32_t idesc = make_idesc(128, 128 * pi.nt, 1, 1, 0, 0);
-        mbar_wait(&q_full[qb], (it / kPairQBufs) & 1, ctx, 132);
-        const uint32_t q_addr = smem_u32(sQ + qb * 65536);
-        for (int c = 0; c < nchunks; ++c) {
-          const int a = (gc0 + c) & 1;
-          uint32_t& ac = a ? ac1 : ac0;
-          if (ac >= 1) mbar_wait(&acc_empty[a], (ac - 1) & 1, ctx, 133);
-          ++ac;
+    // the whole warp walks the loop, one elected lane issues (see the attention kernel's issuer)
+    const bool leader = elect_one();
+    uint32_t pc = 0, ac0 = 0, ac1 = 0, gc0 = 0;   // gc0: chunks of all earlier units
+    for (int it = 0;; ++it) {
+      const int slot = it % kPairInfoSlots, qb = it % kPairQBufs;
+      mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 131);
+      const PairInfo& pi = info[slot];
+      if (!pi.valid) break;
+      const int nchunks = unit_chunks(pi);
+      const uint32_t idesc = make_idesc(128, 128 * pi.nt, 1, 1, 0, 0);
+      mbar_wait(&q_full[qb], (it / kPairQBufs) & 1, ctx, 132);
+      const uint64_t q_desc = make_smem_desc_sw128(smem_u32(sQ + qb * 65536), 16, 1024);
+      for (int c = 0; c < nchunks; ++c) {
+        const int a = (gc0 + c) & 1;
+        uint32_t& ac = a ? ac1 : ac0;
+        if (ac >= 1) mbar_wait(&acc_empty[a], (ac - 1) & 1, ctx, 133);
+        ++ac;
 #pragma unroll
-          for (int p = 0; p < 4; ++p, ++pc) {
-            const int s = pc % kPairPieces;
-            mbar_wait(&full[s], (pc / kPairPieces) & 1, ctx, 134);
-            tc_fence_after();
-            const uint32_t a_addr = smem_u32(sStage + s * kPairPieceBytes);
+        for (int p = 0; p < 4; ++p, ++pc) {
+          const int s = pc % kPairPieces;
+          mbar_wait(&full[s], (pc / kPairPieces) & 1, ctx, 134);
+          tc_fence_after();
+          const uint64_t a_desc = make_smem_desc_sw128(smem_u32(sStage + s * kPairPieceBytes), 16, 1024);
+          if (leader) {
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-              const uint64_t ad = make_smem_desc_sw128(a_addr + ks * 32, 16, 1024);
-              const uint64_t bd = make_smem_desc_sw128(q_addr + (p & 1) * 32768 + ks * 32, 16, 1024);
-              umma_f16_ss(tmem + a * 256, ad, bd, idesc, (p | ks) != 0);
-            }
+            for (int ks = 0; ks < 4; ++ks)
+              umma_f16_ss(tmem + a * 256, a_desc + ks * 2, q_desc + ((p & 1) * 2048 + ks * 2), idesc, (p | ks) != 0);
             umma_commit(&empty[s]);
+            if (p == 3) umma_commit(&acc_full[a]);
           }
-          umma_commit(&acc_full[a]);
         }
+      }
+      __syncwarp();   // no lane reads the descriptor any more
+      if (leader) {
         umma_commit(&q_empty[qb]);
         mbar_arrive(&info_empty[slot]);
-        gc0 += nchunks;
       }
+      gc0 += nchunks;
     }
   } else {
     // ---------------- consumers: per pooled key and tile, maximum and exponential sum over the tile's rows ----------------
@@ -366,7 +368,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     }
   }
   if (abort_flag) {   // MMAs and bulk copies may still be in flight: let them finish before tensor memory goes
-    if (warp == 9 && lane == 0) {
+    if (warp == 9 && elect_one()) {
       umma_commit(&drain_bar);
       mbar_wait_drain(&drain_bar, 0, 200000000ll);
     }

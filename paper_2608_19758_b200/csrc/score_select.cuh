@@ -474,42 +474,45 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
     }
   } else if (warp == 9) {
     // ---------------- UMMA issuer: acc[c & 1] = kbar_hi Q^T + kbar_lo Q^T ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = FP8 ? make_idesc(128, 128, 0, 0, 0, 0) : make_idesc(128, 128, 1, 1, 0, 0);
-      uint32_t pc = 0, ac0 = 0, ac1 = 0, gc0 = 0;   // gc0: chunks of all earlier tiles
-      for (int it = 0;; ++it) {
-        const int slot = it % kScoreInfoSlots, qb = it % kScoreQBufs;
-        mbar_wait(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 131);
-        if (!info_valid[slot]) break;
-        const int nchunks = (info[slot].J_hi + 128) >> 7;
-        mbar_wait(&q_full[qb], (it / kScoreQBufs) & 1, ctx, 132);
-        const uint32_t q_addr = smem_u32(sQ + qb * 32768);
-        for (int c = 0; c < nchunks; ++c) {
-          const int a = (gc0 + c) & 1;
-          uint32_t& ac = a ? ac1 : ac0;
-          if (ac >= 1) mbar_wait(&acc_empty[a], (ac - 1) & 1, ctx, 133);
-          ++ac;
+    // the whole warp walks the loop, one elected lane issues (see the attention kernel's issuer)
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = FP8 ? make_idesc(128, 128, 0, 0, 0, 0) : make_idesc(128, 128, 1, 1, 0, 0);
+    uint32_t pc = 0, ac0 = 0, ac1 = 0, gc0 = 0;   // gc0: chunks of all earlier tiles
+    for (int it = 0;; ++it) {
+      const int slot = it % kScoreInfoSlots, qb = it % kScoreQBufs;
+      mbar_wait(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 131);
+      if (!info_valid[slot]) break;
+      const int nchunks = (info[slot].J_hi + 128) >> 7;
+      mbar_wait(&q_full[qb], (it / kScoreQBufs) & 1, ctx, 132);
+      const uint64_t q_desc = make_smem_desc_sw128(smem_u32(sQ + qb * 32768), 16, 1024);
+      for (int c = 0; c < nchunks; ++c) {
+        const int a = (gc0 + c) & 1;
+        uint32_t& ac = a ? ac1 : ac0;
+        if (ac >= 1) mbar_wait(&acc_empty[a], (ac - 1) & 1, ctx, 133);
+        ++ac;
 #pragma unroll
-          for (int part = 0; part < 2; ++part, ++pc) {
-            const int s = pc % kScoreStages;
-            mbar_wait(&full[s], (pc / kScoreStages) & 1, ctx, 134);
-            tc_fence_after();
-            const uint32_t a_addr = smem_u32(sStage + s * 32768);
+        for (int part = 0; part < 2; ++part, ++pc) {
+          const int s = pc % kScoreStages;
+          mbar_wait(&full[s], (pc / kScoreStages) & 1, ctx, 134);
+          tc_fence_after();
+          const uint64_t a_desc = make_smem_desc_sw128(smem_u32(sStage + s * 32768), 16, 1024);
+          if (leader) {
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-              const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
-              const uint64_t ad = make_smem_desc_sw128(a_addr + off, 16, 1024);
-              const uint64_t bd = make_smem_desc_sw128(q_addr + off, 16, 1024);
-              umma_f16_ss(tmem + a * 128, ad, bd, idesc, (part | ks) != 0);
+              const uint64_t off = (ks >> 2) * 1024 + (ks & 3) * 2;
+              umma_f16_ss(tmem + a * 128, a_desc + off, q_desc + off, idesc, (part | ks) != 0);
             }
             umma_commit(&empty[s]);
+            if (part == 1) umma_commit(&acc_full[a]);
           }
-          umma_commit(&acc_full[a]);
         }
+      }
+      __syncwarp();   // no lane reads the descriptor any more
+      if (leader) {
         umma_commit(&q_empty[qb]);
         mbar_arrive(&info_empty[slot]);
-        gc0 += nchunks;
       }
+      gc0 += nchunks;
     }
   } else {
     // ---------------- consumers: per pooled key, max and exp-sum over the tile's rows; then selection ----------------
@@ -584,7 +587,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
     }
   }
   if (abort_flag) {   // MMAs and bulk copies may still be in flight: let them finish before tensor memory goes
-    if (warp == 9 && lane == 0) {
+    if (warp == 9 && elect_one()) {
       umma_commit(&drain_bar);
       mbar_wait_drain(&drain_bar, 0, 200000000ll);
     }
