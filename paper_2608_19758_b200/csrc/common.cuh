@@ -9,6 +9,13 @@ constexpr int kBlock = 128;       // B: KV tokens per selection block (Sec. 4.1)
 constexpr int kTileRows = 128;    // packed query rows per tile (kBlockM, Sec. 4.1)
 constexpr int kMaxBlocks = 4096;  // KV blocks per sequence the kernels are compiled for (512K tokens)
 constexpr int kMaxChunks = kMaxBlocks / 128;
+// Query tiles by TMA.  Under PackGQA (Eq. 13) the packed rows of a tile are consecutive (token, head) pairs of one KV head's
+// group, so the box [128 bytes, g heads, tokens] that starts at the tile's first token holds them all, in packed order, the
+// first one r0 % g rows into it.  Where g does not divide 128 the box lands that many rows in front of the tile's place in
+// shared memory (the 128-byte swizzle goes by the address, so the tile itself sits as the MMA reads it) and its overhang on
+// padding: at most kQLeadRows rows in front and kQTailRows behind.
+constexpr int kQLeadRows = 8;
+constexpr int kQTailRows = 16;
 constexpr int kCountBuckets = 1024;  // work-order histogram resolution (selected-block count, capped)
 
 // One (sequence, KV head, tile) segment; built on the host by the planner.
@@ -34,10 +41,9 @@ struct DevParams {
   int32_t sink_blocks, window_blocks, use_correction;
   int32_t num_seqs, nseg, nblk_tot, total_q;
   int32_t fp8;
-  int32_t q_tma;     // 1: the group size divides 128, so a packed query tile is a TMA box [128 bytes, g heads, 128 / g tokens]
-                     //    (x 2 for BF16); used by the attention kernel (both dtypes) and the BF16 scorer
-  int32_t q_box_tok; // tokens of the box that holds a packed tile's rows: 128 / g, or floor((g - 1 + 127) / g) + 1 when g does not
-                     // divide 128 (the tile then starts r0 % g rows into the box)
+  int32_t q_box;     // 1: the boxes around one packed tile (q_box_tok tokens) and around two adjacent ones (q_box2_tok) fit the
+                     //    padding: attention kernel (both dtypes) and BF16 scorer fetch query tiles by TMA
+  int32_t q_box_tok, q_box2_tok;   // 128 / g tokens where g divides 128, else floor((g - 1 + 127) / g) + 1; 256 rows likewise
   int32_t q_raw_tma; // 1: FP8 plans whose box fits the scorer's raw staging slot: the scorer fetches query tiles by TMA
   int32_t diag_mma;  // 1: a tile spans at most 32 positions (g >= 4), so the causal mask of a diagonal block can ride
                      //    on a K = 32 one-hot MMA step in the attention kernel

@@ -38,7 +38,7 @@ struct fp2_plan {
   int32_t* d_blk_off;
   int32_t* d_carry;                 // [3 x num_seqs]: pooled rows carried over from a previous chunk (fp2_pool_carry)
   int32_t* d_lk;                    // [num_seqs]: KV lengths as given to fp2_plan_create
-  int2* d_units;                    // scorer work units of BF16 plans with TMA query tiles: (segment, second segment or -1)
+  int2* d_units;                    // scorer work units of BF16 plans whose query tiles come by TMA: (segment, second segment or -1)
   int32_t nunits;
   std::vector<int32_t> h_blk_off, h_carry;
   bool carry_valid;
@@ -261,8 +261,11 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
   d.use_correction = p->use_correction ? 1 : 0;
   d.num_seqs = p->num_seqs; d.nseg = (int32_t)pl->nseg; d.nblk_tot = (int32_t)nblk_tot; d.total_q = p->total_q;
   d.fp8 = p->dtype == FP2_FP8_E4M3;
-  d.q_tma = (128 % g == 0) ? 1 : 0;
   d.q_box_tok = (128 % g == 0) ? 128 / g : (g - 1 + 127) / g + 1;
+  d.q_box2_tok = (256 % g == 0) ? 256 / g : (g - 1 + 255) / g + 1;
+  // tiles start at multiples of 128 rows, so at most g - gcd(g, 128) rows into their box (g & -g: the power of two in g)
+  d.q_box = (g <= 128 && g - (g & -g) <= kQLeadRows && d.q_box2_tok <= 256 &&
+             g * d.q_box_tok <= 128 + kQTailRows && g * d.q_box2_tok <= 256 + kQTailRows) ? 1 : 0;
   d.q_raw_tma = (d.fp8 && g <= 128 && d.q_box_tok <= 256 && g * d.q_box_tok * 128 <= kScoreRawBytes) ? 1 : 0;
   // positions spanned by a 128-row packed tile: 128 / g when g divides 128, else up to floor((g - 1 + 127) / g) + 1
   d.diag_mma = ((128 % g == 0) ? 128 / g : (g - 1 + 127) / g + 1) <= 32 ? 1 : 0;
@@ -321,15 +324,15 @@ static bool make_map(fp2_plan* pl, CUtensorMap* m, const void* base, int64_t row
   return r == CUDA_SUCCESS;
 }
 
-// Packed query tile as a TMA box (see DevParams::q_tma): [128 bytes, g heads, 128 / g tokens] of q [total_q, Hq, 128]
-// -- 64 BF16 elements (the tile takes two boxes) or 128 e4m3 bytes (one box).
-static bool make_q_map(fp2_plan* pl, CUtensorMap* m, const void* q, int box_tokens = 0) {
+// Packed query rows as a TMA box (see DevParams::q_box): [128 bytes, g heads, box_tokens tokens] of q [total_q, Hq, 128]
+// -- 64 BF16 elements (rows take two boxes) or 128 e4m3 bytes (one box).
+static bool make_q_map(fp2_plan* pl, CUtensorMap* m, const void* q, int box_tokens) {
   const int g = pl->dev.group;
   const bool fp8 = pl->dev.fp8;
   const cuuint64_t esz = fp8 ? 1 : 2;
   cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)pl->prm.num_q_heads, (cuuint64_t)pl->prm.total_q};
   cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * esz, (cuuint64_t)kHeadDim * esz * pl->prm.num_q_heads};
-  cuuint32_t box[3] = {fp8 ? 128u : 64u, (cuuint32_t)g, (cuuint32_t)(box_tokens > 0 ? box_tokens : 128 / g)};
+  cuuint32_t box[3] = {fp8 ? 128u : 64u, (cuuint32_t)g, (cuuint32_t)box_tokens};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = pl->encode(m, fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                           const_cast<void*>(q), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -451,19 +454,20 @@ extern "C" fp2_status fp2_select_blocks(fp2_plan* pl, const void* q, const void*
       !make_map(pl, &mlo, ws + pl->ws_klo, pl->nblk_tot, pl->prm.num_kv_heads, 128, false))
     return FP2_ERR_CUDA;
   CUtensorMap mq = mhi;   // unused unless the scorer takes its query tiles by TMA
+  CUtensorMap mq2 = mhi;
   if (pl->dev.fp8 ? (pl->dev.q_raw_tma && !make_q_map(pl, &mq, q, pl->dev.q_box_tok))
-                  : (pl->dev.q_tma && !make_q_map(pl, &mq, q)))
+                  : (pl->dev.q_box && (!make_q_map(pl, &mq, q, pl->dev.q_box_tok) || !make_q_map(pl, &mq2, q, pl->dev.q_box2_tok))))
     return FP2_ERR_CUDA;
   int* status = reinterpret_cast<int*>(ws + pl->ws_status);
   const unsigned grid = (unsigned)(pl->nseg < pl->num_sms ? pl->nseg : pl->num_sms);
   if (pl->dev.fp8)
     score_select_kernel<true><<<grid, kScoreThreads, kScoreSmemBytes, st>>>(
         mhi, mlo, mq, (const uint8_t*)q, pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
-  else if (pl->dev.q_tma) {
-    // BF16 tiles that are TMA boxes: pairs of adjacent tiles per pooled-key chunk.  The pair kernel takes the pooled
+  else if (pl->dev.q_box) {
+    // BF16 tiles that come as TMA boxes: pairs of adjacent tiles per pooled-key chunk.  The pair kernel takes the pooled
     // keys in pieces of 64 elements x 128 keys, which is the box of mhi / mlo already.
     const unsigned grid_pairs = (unsigned)(pl->nunits < pl->num_sms ? pl->nunits : pl->num_sms);
-    score_pair_kernel<<<grid_pairs, kPairThreads, kPairSmemBytes, st>>>(mhi, mlo, mq, pl->d_segs, pl->d_units, pl->nunits,
+    score_pair_kernel<<<grid_pairs, kPairThreads, kPairSmemBytes, st>>>(mhi, mlo, mq, mq2, pl->d_segs, pl->d_units, pl->nunits,
                                                                         pl->dev, seg_offset, seg_count, blk_idx, status);
   } else
     score_select_kernel<false><<<grid, kScoreThreads, kScoreSmemBytes, st>>>(
@@ -581,8 +585,8 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
     a.part_ml = reinterpret_cast<float2*>(ws + pl->ws_part_ml);
     max_units = pl->split_units_cap;
   }
-  CUtensorMap mq = mk;   // unused unless q_tma
-  if (pl->dev.q_tma && !make_q_map(pl, &mq, q)) return FP2_ERR_CUDA;
+  CUtensorMap mq = mk;   // unused unless q_box
+  if (pl->dev.q_box && !make_q_map(pl, &mq, q, pl->dev.q_box_tok)) return FP2_ERR_CUDA;
   launch_attn(pl, mk, mv, mkb, mkb_lo, mvb, mq, a, max_units, st);
   pl->last_launches += 1;
   if (split) {
@@ -693,8 +697,8 @@ extern "C" fp2_status fp2_dense_prefill_static(fp2_plan* pl, const void* q, cons
 #ifdef FP2_PROFILE
   a.prof = nullptr;
 #endif
-  CUtensorMap mq = mk;   // unused unless q_tma
-  if (pl->dev.q_tma && !make_q_map(pl, &mq, q)) return FP2_ERR_CUDA;
+  CUtensorMap mq = mk;   // unused unless q_box
+  if (pl->dev.q_box && !make_q_map(pl, &mq, q, pl->dev.q_box_tok)) return FP2_ERR_CUDA;
   launch_attn(pl, mk, mv, mk, mk, mv, mq, a, pl->nseg, st);
   pl->last_launches = 4;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;

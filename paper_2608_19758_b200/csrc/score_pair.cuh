@@ -1,5 +1,5 @@
-// Fused block scoring and selection (Eq. 19, Eq. 20; Algorithm 1 lines 3-5) for BF16 plans whose packed query tile
-// is a TMA box (group size divides 128): score_select_kernel with TWO adjacent query tiles of a KV head per unit.
+// Fused block scoring and selection (Eq. 19, Eq. 20; Algorithm 1 lines 3-5) for BF16 plans whose packed query tiles
+// come as TMA boxes (DevParams::q_box): score_select_kernel with TWO adjacent query tiles of a KV head per unit.
 //
 // At long sequences score_select_kernel is bound by the traffic of the pooled keys from L2 into shared memory: every
 // chunk of 128 pooled keys (hi + lo: 64 KB) is fetched once per query tile, 35 bytes per cycle and SM at 131072
@@ -19,7 +19,12 @@
 // Roles: warps 0-3 / 4-7 consumer warpgroups; warp 8 TMA producer of kbar pieces (16 KB: 128 keys x 64 elements, four
 // per chunk: hi | lo x the two halves of d); warp 9 UMMA issuer and TMEM owner; warp 10 unit set-up and query tiles by
 // TMA (two units in flight); warp 11 selection.
-// Shared memory: 2 x 64 KB query pairs + 4 x 16 KB pieces + 16 KB energies.  TMEM: 2 x 256 columns.
+// Shared memory: 2 x 64 KB query pairs (and 5 KB of padding each) + 4 x 16 KB pieces + 16 KB energies.  TMEM: 2 x 256
+// columns.
+//
+// Group sizes that do not divide 128 (7 and the like) used to stage every tile with 2048 cp.async pieces of 16 bytes, each
+// with its own divisions: 24 sequences of 60 to 1500 tokens, 28 query heads on 4 KV heads, 202 us for the index stage then,
+// 53 us with the boxes (and the attention call 174 -> 131 us by the same change).
 #pragma once
 #include "score_select.cuh"
 
@@ -31,7 +36,10 @@ constexpr int kPairQBufs = 2;            // 64 KB query-pair buffers
 constexpr int kPairPieces = 4;           // ring of 16 KB kbar pieces
 constexpr int kPairPieceBytes = 16384;
 constexpr int kPairMaxCand = 1024;       // a tile is paired only if it has at most this many candidate blocks
-constexpr int kPairSmemBytes = 1024 /*align*/ + kPairQBufs * 65536 + kPairPieces * kPairPieceBytes + kMaxBlocks * 4;
+constexpr int kPairQHalf = 32768 + kQTailRows * 128;                // 256 rows x 128 bytes and the overhang behind them
+constexpr int kPairQBytes = kQLeadRows * 128 + 2 * kPairQHalf;      // (the overhang in front of the second half falls there too)
+static_assert(kQLeadRows * 128 % 1024 == 0 && kPairQHalf % 1024 == 0, "query halves start on the swizzle's period");
+constexpr int kPairSmemBytes = 1024 /*align*/ + kPairQBufs * kPairQBytes + kPairPieces * kPairPieceBytes + kMaxBlocks * 4;
 
 struct PairInfo {
   SegInfo sg[2];
@@ -85,15 +93,15 @@ __device__ __forceinline__ void score_cols(uint32_t lane_addr, float cs, int nro
 
 __global__ void __launch_bounds__(kPairThreads, 1)
 score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_constant__ CUtensorMap map_klo,
-                  const __grid_constant__ CUtensorMap map_q, const SegInfo* __restrict__ segs,
-                  const int2* __restrict__ units, int nunits, DevParams P, int64_t* __restrict__ seg_offset,
+                  const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_q2,
+                  const SegInfo* __restrict__ segs, const int2* __restrict__ units, int nunits, DevParams P, int64_t* __restrict__ seg_offset,
                   int32_t* __restrict__ seg_count, int32_t* __restrict__ blk_idx, int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // query pair buffer: [half of d][tile][128 rows x 128 bytes] -- the two tiles of a half are 256 consecutive rows of
-  // one swizzled K-major operand
-  uint8_t* sQ = smem;
-  uint8_t* sStage = smem + kPairQBufs * 65536;                                  // ring of kbar pieces
+  // query pair buffer: [half of d][tile][128 rows x 128 bytes] -- the two tiles of a half are 256 consecutive packed rows,
+  // one swizzled K-major operand and one TMA box
+  uint8_t* sQ = smem + kQLeadRows * 128;
+  uint8_t* sStage = smem + kPairQBufs * kPairQBytes;                                  // ring of kbar pieces
   float* sE = reinterpret_cast<float*>(sStage + kPairPieces * kPairPieceBytes); // log2 energies: unit parity x 2048,
                                                                                 // second tile of a pair 1024 further
 
@@ -145,8 +153,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
 
   if (warp == 10) {
     // ---------------- set-up: unit k of this CTA is number blockIdx.x + k * gridDim.x of the planner's table
-    // (heaviest first; a static round-robin, no atomic on the critical path).  Query tiles by TMA: under PackGQA
-    // (Eq. 13) a tile is 128 / g consecutive tokens x g consecutive heads, one box per 64-element half.
+    // (heaviest first; a static round-robin, no atomic on the critical path).  Query tiles by TMA, one box per 64-element
+    // half (see kQLeadRows); rows of a short last tile get whatever follows and are not used.
     const uint64_t pol = l2_policy_evict_first();
     for (int k = 0;; ++k) {
       const int slot = k % kPairInfoSlots, qb = k % kPairQBufs;
@@ -171,14 +179,14 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       if (k >= kPairQBufs) mbar_wait(&q_empty[qb], ((k / kPairQBufs) - 1) & 1, ctx, 112);
       if (lane == 0) {
         const PairInfo& pi = info[slot];
-        uint8_t* dst = sQ + qb * 65536;
-        mbar_arrive_expect_tx(&q_full[qb], (uint32_t)pi.nt * 32768u);
-        for (int tt = 0; tt < pi.nt; ++tt) {
-          const SegInfo& sg = pi.sg[tt];
-          const int tok = sg.q_tok0 + sg.r0 / P.group;
-          tma_load_3d_hint(dst + tt * 16384, &map_q, &q_full[qb], 0, sg.h * P.group, tok, pol);
-          tma_load_3d_hint(dst + 32768 + tt * 16384, &map_q, &q_full[qb], 64, sg.h * P.group, tok, pol);
-        }
+        const SegInfo& sg = pi.sg[0];
+        const int tok0 = sg.r0 / P.group, lead = sg.r0 - tok0 * P.group;
+        uint8_t* dst = sQ + qb * kPairQBytes - lead * 128;
+        const CUtensorMap* mp = pi.nt > 1 ? &map_q2 : &map_q;
+        const uint32_t rows = (uint32_t)(P.group * (pi.nt > 1 ? P.q_box2_tok : P.q_box_tok));
+        mbar_arrive_expect_tx(&q_full[qb], rows * 256u);
+        tma_load_3d_hint(dst, mp, &q_full[qb], 0, sg.h * P.group, sg.q_tok0 + tok0, pol);
+        tma_load_3d_hint(dst + kPairQHalf, mp, &q_full[qb], 64, sg.h * P.group, sg.q_tok0 + tok0, pol);
       }
       __syncwarp();
     }
@@ -261,7 +269,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       const int nchunks = unit_chunks(pi);
       const uint32_t idesc = make_idesc(128, 128 * pi.nt, 1, 1, 0, 0);
       mbar_wait(&q_full[qb], (it / kPairQBufs) & 1, ctx, 132);
-      const uint64_t q_desc = make_smem_desc_sw128(smem_u32(sQ + qb * 65536), 16, 1024);
+      const uint64_t q_desc = make_smem_desc_sw128(smem_u32(sQ + qb * kPairQBytes), 16, 1024);
       for (int c = 0; c < nchunks; ++c) {
         const int a = (gc0 + c) & 1;
         uint32_t& ac = a ? ac1 : ac0;
@@ -276,7 +284,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
           if (leader) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-              umma_f16_ss(tmem + a * 256, a_desc + ks * 2, q_desc + ((p & 1) * 2048 + ks * 2), idesc, (p | ks) != 0);
+              umma_f16_ss(tmem + a * 256, a_desc + ks * 2, q_desc + ((p & 1) * (kPairQHalf >> 4) + ks * 2), idesc, (p | ks) != 0);
             umma_commit(&empty[s]);
             if (p == 3) umma_commit(&acc_full[a]);
           }

@@ -16,8 +16,7 @@
 //
 // Roles: warps 0-3 / 4-7 = two consumer warpgroups alternating over chunks (TMEM accumulators 0 / 1); warp 8 = TMA
 // producer of kbar pieces; warp 9 = UMMA issuer; warp 10 fetches the next segments and stages their query tiles into
-// free Q buffers (by TMA when the tile is a box -- BF16, group size divides 128 --, else with cp.async, widening FP8
-// to F16), so that the next tile's MMAs start while the current tile is still being exponentiated; warp 11 applies
+// free Q buffers (FP8: one raw TMA box, widened to F16; BF16 group sizes without a box, see DevParams::q_box: cp.async), so that the next tile's MMAs start while the current tile is still being exponentiated; warp 11 applies
 // threshold and forced sets and writes the ordered list of tile t beside the scoring of tile t+1.
 #pragma once
 #include <cuda_bf16.h>
@@ -200,6 +199,7 @@ __device__ __forceinline__ void score_chunk(uint32_t lane_addr, float cs, const 
 // register-staged variant above keeps only a few loads per thread in flight and was latency-bound at one tile
 // per ~12 us).  Same layout and zero fill as load_q_tile_bf16; with `wait` it returns after the copies have landed,
 // otherwise the caller closes a cp.async group and waits for it later.
+template <int HALF = 16384>   // bytes from one 64-element half of the tile to the other
 __device__ __forceinline__ void load_q_tile_async(uint8_t* sQ, const uint8_t* __restrict__ q, const SegInfo& sg,
                                                   const DevParams& P, int t, int nthr, bool wait = true) {
   const int g = P.group;
@@ -216,7 +216,7 @@ __device__ __forceinline__ void load_q_tile_async(uint8_t* sQ, const uint8_t* __
       src = q + ((tok * P.num_q_heads + head) * kHeadDim + ch * 8) * 2;
       nbytes = 16;
     }
-    cp_async16(base + (ch >> 3) * 16384 + sw128_offset(row, ch & 7), src, nbytes, pol);
+    cp_async16(base + (ch >> 3) * HALF + sw128_offset(row, ch & 7), src, nbytes, pol);
   }
   if (wait) cp_async_wait_all();
 }
@@ -250,13 +250,11 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   WaitCtx ctx{status, &abort_flag};
-  // When the query tiles come by TMA, one set-up warp is enough and the other (warp 11) takes the selection off
-  // the consumers: they only leave the tile's energies (and their maxima) in shared memory and go on with the next
-  // tile's chunks; threshold, forced blocks and the ordered compaction of tile t run beside the scoring of tile
-  // t+1.  The energy buffer is used in two halves by tile parity; a tile with more than kMaxBlocks / 2 candidates
-  // takes both and waits for its neighbours.  In this mode the two warpgroups also share the chunks by a count
-  // that runs across tiles, so a tile with an odd number of chunks leaves neither of them short.
-  const bool q_by_tma = !FP8 && P.q_tma;   // else warp 10 stages the tile with cp.async (and widens FP8 to F16)
+  // Warp 11 takes the selection off the consumers: they only leave the tile's energies (and their maxima) in shared memory
+  // and go on with the next tile's chunks; threshold, forced blocks and the ordered compaction of tile t run beside the
+  // scoring of tile t+1.  The energy buffer is used in two halves by tile parity; a tile with more than kMaxBlocks / 2
+  // candidates takes both and waits for its neighbours.  The two warpgroups share the chunks by a count that runs across
+  // tiles, so a tile with an odd number of chunks leaves neither of them short.
 
   if (tid == 0) {
     abort_flag = 0;
@@ -265,7 +263,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
       mbar_init(&info_empty[i], 2 + 256 + 1);   // producer, issuer, consumers, selection warp
     }
     for (int i = 0; i < kScoreQBufs; ++i) {
-      mbar_init(&q_full[i], q_by_tma ? 1 : 32);
+      mbar_init(&q_full[i], 32);
       mbar_init(&q_empty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -338,38 +336,6 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
       cp_async_commit();
       return true;
     };
-    if (q_by_tma) {
-      // Under PackGQA (Eq. 13) packed row r is (token r / g, head r % g): when g divides 128 a tile is 128 / g
-      // consecutive tokens x g consecutive heads, i.e. one TMA box per 64-element half, landing in exactly the
-      // swizzled layout the MMA reads.  No thread touches the data; the tile's barrier carries the byte count.
-      // Rows past the end of a short last tile read the tokens that follow (or zeros past the tensor's end) and are
-      // never used.  Three tiles in flight.
-      const uint64_t pol = l2_policy_evict_first();
-      for (int k = 0;; ++k) {
-        const int slot = k % kScoreInfoSlots, qb = k % kScoreQBufs;
-        if (k >= kScoreInfoSlots) mbar_wait(&info_empty[slot], ((k / kScoreInfoSlots) - 1) & 1, ctx, 111);
-        const int sgi = seg_of(k);
-        bool valid = sgi >= 0 && !*ctx.abort;   // after a wait has run out no further tile is started
-        valid = __shfl_sync(0xffffffffu, valid, 0);
-        if (t64 == 0) {
-          info_valid[slot] = valid;
-          if (valid) info[slot] = segs[sgi];
-          __threadfence_block();
-          mbar_arrive(&info_full[slot]);
-        }
-        __syncwarp();
-        if (!valid) break;
-        if (k >= kScoreQBufs) mbar_wait(&q_empty[qb], ((k / kScoreQBufs) - 1) & 1, ctx, 112);
-        if (t64 == 0) {
-          const SegInfo& sg = info[slot];
-          uint8_t* dst = sQ + qb * 32768;
-          mbar_arrive_expect_tx(&q_full[qb], 32768);
-          tma_load_3d_hint(dst, &map_q, &q_full[qb], 0, sg.h * P.group, sg.q_tok0 + sg.r0 / P.group, pol);
-          tma_load_3d_hint(dst + 16384, &map_q, &q_full[qb], 64, sg.h * P.group, sg.q_tok0 + sg.r0 / P.group, pol);
-        }
-        __syncwarp();
-      }
-    } else {
 #ifdef FP2_PROFILE
     long long sp[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     long long sa = clock64(), sb;
@@ -410,7 +376,6 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
       for (int i = 0; i < 8; ++i) g_score_prof[((size_t)gridDim.x * 2 + blockIdx.x) * 8 + i] = sp[i];
     }
 #endif
-    }
   } else if (warp == 11) {
     // ---------------- selection warp: threshold, forced blocks, ordered compaction of tile `it` ----------------
     for (int it = 0;; ++it) {

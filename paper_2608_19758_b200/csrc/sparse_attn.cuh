@@ -104,7 +104,11 @@ struct AttnCfg {
   static constexpr int kThreads = 256;
   static constexpr int kCtasPerSm = 2;
   static constexpr int kBiasBytes = 4096;                    // one 128 x 32 e5m2 operand without swizzle
-  static constexpr int kSmemBytes = 1024 + 3 * kTileBytes + 2 * kBiasBytes;   // both dtypes: 96 KB of tiles + the mask operands
+  // query tile: per 128 bytes of a row (two halves BF16, one FP8) 128 rows and the overhang of the box (see kQLeadRows)
+  static constexpr int kQHalf = 16384 + kQTailRows * 128;
+  static constexpr int kOffK = kQLeadRows * 128 + (FP8 ? 1 : 2) * kQHalf;
+  static constexpr int kOffHot = kOffK + 2 * kTileBytes + (FP8 ? kRawBytes : 0);
+  static constexpr int kSmemBytes = 1024 + kOffHot + 2 * kBiasBytes;   // 98 to 101 KB of tiles + the mask operands
   // Registers: two CTAs share the file, 128 per thread at launch; setmaxnreg moves them from the service warps
   // to the softmax warps.  The move waits without bound for registers the CTA does not own, so the sum is
   // checked here and the compiled register count is checked on the host before the first launch.
@@ -192,7 +196,7 @@ __device__ __forceinline__ float row_exp(const uint32_t (&x)[128], uint32_t p_ad
 }
 
 // map_kbar / map_kbar_lo: pooled keys of the correction chunks -- BF16: one BF16 array (map_kbar_lo unused);
-// FP8: the e4m3 hi and lo arrays.  map_vbar: pooled values, 16-bit.  map_q: packed query tiles (DevParams::q_tma).
+// FP8: the e4m3 hi and lo arrays.  map_vbar: pooled values, 16-bit.  map_q: packed query tiles (DevParams::q_box).
 template <bool FP8>
 __global__ void __launch_bounds__(AttnCfg<FP8>::kThreads, AttnCfg<FP8>::kCtasPerSm)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -202,8 +206,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
   constexpr int kSetupThreads = 64;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sQ = smem;                                  // 32 KB (BF16) / 16 KB (raw e4m3)
-  uint8_t* sK = smem + (FP8 ? kRawBytes : kTileBytes); // 32 KB
+  uint8_t* sQ = smem + kQLeadRows * 128;               // 32 KB (BF16) / 16 KB (raw e4m3) and padding
+  uint8_t* sK = smem + AttnCfg<FP8>::kOffK;            // 32 KB
   uint8_t* sV = sK + kTileBytes;                       // 32 KB, 16-bit
   uint8_t* sVraw = sV + kTileBytes;                    // FP8 only: 16 KB raw e4m3 V tile
   (void)sVraw;
@@ -219,7 +223,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
   // A hidden logit thus carries -3.3e9 (raw units), which the exponential turns into an exact zero.
   // Both operands are K-major without swizzle: 8-row x 16-byte core matrices, row r at (r / 8) * 256 + (r % 8) * 16,
   // bytes 16..31 of the row 128 bytes further.
-  uint8_t* sHot = smem + 3 * kTileBytes;
+  uint8_t* sHot = smem + AttnCfg<FP8>::kOffHot;
   uint8_t* sBias = sHot + AttnCfg<FP8>::kBiasBytes;
 
   __shared__ TileInfo info[2];
@@ -385,17 +389,19 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         }
         fence_proxy_async();
       }
-      if (P.q_tma) {
-        // PackGQA (Eq. 13) with a group size that divides 128: the tile is 128 / g tokens x g heads, one TMA box
-        // per 128 bytes of a row (two 64-element halves for BF16, the whole row for e4m3), landing in the swizzled
-        // layout the MMA reads.  Rows past the end of a short last tile get whatever follows; nothing reads them.
+      if (P.q_box) {
+        // one TMA box per 128 bytes of a row (see kQLeadRows), landing in the swizzled layout the MMA reads.  Rows past the
+        // end of a short last tile get whatever follows; nothing reads them.
         if (t64 == 0) {
           const SegInfo& sg = ti.sg;
           const uint64_t pol = l2_policy_evict_first();
-          mbar_arrive_expect_tx(&q_full, FP8 ? kRawBytes : kTileBytes);
-          tma_load_3d_hint(sQ, &map_q, &q_full, 0, sg.h * g, sg.q_tok0 + sg.r0 / g, pol);
+          const int tok0 = sg.r0 / g;
+          uint8_t* dst = sQ - (sg.r0 - tok0 * g) * 128;
+          const uint32_t bytes = (uint32_t)(g * P.q_box_tok) * 128u;
+          mbar_arrive_expect_tx(&q_full, FP8 ? bytes : 2 * bytes);
+          tma_load_3d_hint(dst, &map_q, &q_full, 0, sg.h * g, sg.q_tok0 + tok0, pol);
           if constexpr (!FP8)
-            tma_load_3d_hint(sQ + 16384, &map_q, &q_full, 64, sg.h * g, sg.q_tok0 + sg.r0 / g, pol);
+            tma_load_3d_hint(dst + AttnCfg<FP8>::kQHalf, &map_q, &q_full, 64, sg.h * g, sg.q_tok0 + tok0, pol);
         } else {
           mbar_arrive(&q_full);
         }
@@ -405,7 +411,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         load_q_raw_async(sQ, A.q, ti.sg, P, t64, kSetupThreads);
         cp_async_wait_all();
       }
-      else load_q_tile_async(sQ, A.q, ti.sg, P, t64, kSetupThreads);
+      else load_q_tile_async<AttnCfg<FP8>::kQHalf>(sQ, A.q, ti.sg, P, t64, kSetupThreads);
       fence_proxy_async();
       mbar_arrive(&q_full);
     }
@@ -585,8 +591,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
           } else {
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-              const uint64_t off = (ks >> 2) * 1024 + (ks & 3) * 2;   // descriptor addresses count 16 bytes
-              umma_f16_ss(tmem, q_desc + off, k_desc + off, idesc_qk, ks > 0);
+              // descriptor addresses count 16 bytes
+              umma_f16_ss(tmem, q_desc + ((ks >> 2) * (AttnCfg<FP8>::kQHalf >> 4) + (ks & 3) * 2),
+                          k_desc + ((ks >> 2) * 1024 + (ks & 3) * 2), idesc_qk, ks > 0);
             }
           }
           if (masked) {   // the mask as one more k-step (see sBias)

@@ -545,3 +545,33 @@ def test_launch_counts_are_reported():
     dc.plan.set_split(4)
     dc.sparse()
     assert dc.plan.last_launch_count() == 6           # order (3) + split plan + attention + merge
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("g", [3, 5, 6, 7, 9, 12])
+def test_group_sizes_whose_query_tiles_start_inside_a_box(g, dtype):
+    """Group sizes that do not divide 128: a tile starts r0 % g rows into its TMA box (up to 8 for g = 9), with the box's
+    overhang on padding; g = 12 is the first whose box of two tiles does not fit and takes the element-wise route.  Ragged
+    last tiles, an odd number of tiles (a pair and a single one) and a prefix.  Rows near the start of a sequence put nearly
+    all weight on one value, so the bound follows the values: BF16 rounds every probability and the output by at most 2^-8
+    of itself, together 2^-7 max |v| (fp32 sums and ex2.approx: well below 1e-3)."""
+    spec = inputs.small_spec(seqs=[(700, 0), (1111, 300), (43, 0)], num_q_heads=2 * g, num_kv_heads=2, page_size=16,
+                             dtype=dtype, config_id=130 + g)
+    spec.alpha = 0.25
+    case, dc, wl = make(spec)
+    vmax = max(float(np.abs(wl.kv(b, h)[1]).max()) for b in range(3) for h in range(2))
+    dc.select()
+    dc.status()
+    check_lists(dc, wl)
+    for lists in (dc.lists_host(), None):
+        if lists is not None:
+            dc.sparse()
+        else:
+            dc.dense()
+        dc.status()
+        Oo, Lo = O.scatter_output(wl, O.oracle_attend(wl, lists, None, dense=lists is None), case.total_q)
+        err = np.abs(dc.out.float().cpu().numpy().astype(np.float64) - Oo)[~np.isnan(Oo)]
+        assert err.size and err.max() <= vmax * 2.0 ** -7 + 1e-3, (err.max(), vmax)
+        gl = dc.lse.cpu().numpy().astype(np.float64)
+        ok = ~np.isnan(Lo)
+        assert (np.abs(gl - Lo)[ok] / np.maximum(np.abs(Lo[ok]), 1.0)).max() <= TOL_LSE_REL
