@@ -106,13 +106,13 @@ def _check(code: int, where: str):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()     # ctypes takes a plain integer for a void pointer
 
 
-def _stream(stream) -> C.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
         stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def fp2_status_string(code: int) -> str:

@@ -16,7 +16,7 @@ constexpr int kMaxChunks = kMaxBlocks / 128;
 // padding: at most kQLeadRows rows in front and kQTailRows behind.
 constexpr int kQLeadRows = 8;
 constexpr int kQTailRows = 16;
-constexpr int kCountBuckets = 1024;  // work-order histogram resolution (selected-block count, capped)
+constexpr int kCountBuckets = 128;   // work-order classes per KV head (selected-block count, see order_bucket)
 
 // One (sequence, KV head, tile) segment; built on the host by the planner.
 struct SegInfo {

@@ -238,7 +238,7 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
   pl->ws_k8hi = o; o += pooled8;
   pl->ws_k8lo = o; o += pooled8;
   pl->ws_order = o; o += align_up(4 * (pl->nseg > 0 ? pl->nseg : 1), 1024);
-  pl->ws_hist = o;  o += align_up(4 * ((int64_t)p->num_kv_heads * kCountBuckets + 1), 1024);
+  pl->ws_hist = o;  o += align_up(8 * (int64_t)p->num_kv_heads * kCountBuckets, 1024);
   // KV splitting pays when there are fewer units than a few waves of workers; the unit arrays and the partial
   // results are sized for nseg + 2 workers units, the bound split_plan_kernel keeps
   const int64_t workers = (int64_t)pl->num_sms * AttnCfg<false>::kCtasPerSm;
@@ -310,6 +310,24 @@ extern "C" int32_t fp2_last_launch_count(const fp2_plan* pl) { return pl ? pl->l
 // ------------------------------------------------------------------------------------------------------
 // helpers
 // ------------------------------------------------------------------------------------------------------
+// A kernel launch that may overlap the end of its predecessor on the stream (see pdl_wait: every kernel of this library
+// waits there before it touches global memory).  Select + sparse at 2048 tokens, 4 heads: 48 us with plain launches, two
+// memsets and a scan kernel in the sort, 35 us so.
+template <typename... KArgs, typename... Args>
+static void launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);   // the caller reads cudaGetLastError
+}
+
 // 3-D map over [rows, heads, 128] elements, box = [box_rows, 1, 64 (bf16) | 128 (fp8)], 128-byte swizzle.
 static bool make_map(fp2_plan* pl, CUtensorMap* m, const void* base, int64_t rows, int heads, int box_rows, bool fp8) {
   const int esz = fp8 ? 1 : 2;
@@ -395,40 +413,37 @@ static fp2_status launch_pool(fp2_plan* pl, const void* k, const void* v, const 
   if (row_chunks <= 256 && 256 % row_chunks == 0) {
     const unsigned grid_rows = (unsigned)(pl->nblk_tot * 2);
     if (pl->dev.fp8)
-      pool_rows_kernel<true><<<grid_rows, 256, 0, st>>>((const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off,
+      launch(pool_rows_kernel<true>, grid_rows, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off,
                                                         ks, vs, pl->dev, khi, klo, vb, ws + pl->ws_k8hi,
                                                         ws + pl->ws_k8lo, carry, status);
     else
-      pool_rows_kernel<false><<<grid_rows, 256, 0, st>>>((const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk,
+      launch(pool_rows_kernel<false>, grid_rows, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk,
                                                          pl->d_blk_off, ks, vs, pl->dev, khi, klo, vb, nullptr, nullptr,
                                                          carry, status);
     pl->last_launches += 1;
     return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
   }
   if (pl->dev.fp8)
-    pool_kv_kernel<true><<<grid, 256, 0, st>>>((const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs,
+    launch(pool_kv_kernel<true>, grid, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs,
                                                pl->dev, khi, klo, vb, ws + pl->ws_k8hi, ws + pl->ws_k8lo, carry, status);
   else
-    pool_kv_kernel<false><<<grid, 256, 0, st>>>((const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs,
+    launch(pool_kv_kernel<false>, grid, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs,
                                                 pl->dev, khi, klo, vb, nullptr, nullptr, carry, status);
   pl->last_launches += 1;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }
 
-// counting sort of the segments: KV-head-major, descending block count
-static fp2_status launch_order(fp2_plan* pl, const int32_t* seg_count, uint8_t* ws, cudaStream_t st) {
+// counting sort of the segments: KV-head-major, descending block count.  hist: class counts and cursors (2 nb words).
+static void launch_order(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, int32_t* counter,
+                         cudaStream_t st) {
   const int nseg = (int)pl->nseg;
-  int32_t* hist = reinterpret_cast<int32_t*>(ws + pl->ws_hist);
-  int32_t* order = reinterpret_cast<int32_t*>(ws + pl->ws_order);
   const int nb = pl->prm.num_kv_heads * kCountBuckets;
-  if (cudaMemsetAsync(hist, 0, sizeof(int32_t) * (size_t)(nb + 1), st) != cudaSuccess) return FP2_ERR_CUDA;
-  if (cudaMemsetAsync(ws + pl->ws_counter, 0, 64, st) != cudaSuccess) return FP2_ERR_CUDA;
-  const int blocks = (nseg + 255) / 256;
-  order_hist_kernel<<<blocks, 256, 0, st>>>(pl->d_segs, seg_count, nseg, hist);
-  order_scan_kernel<<<1, 1024, 0, st>>>(hist, nb);
-  order_scatter_kernel<<<blocks, 256, 0, st>>>(pl->d_segs, seg_count, nseg, hist, order);
+  const unsigned blocks = (unsigned)((nseg + 255) / 256);
+  launch(order_clear_kernel, (unsigned)((2 * nb + 255) / 256), 256, 0, st, hist, 2 * nb, counter);
+  launch(order_hist_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, hist);
+  launch(order_scatter_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, nseg / pl->prm.num_kv_heads, hist,
+         hist + nb, order);
   pl->last_launches += 3;
-  return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -461,17 +476,17 @@ extern "C" fp2_status fp2_select_blocks(fp2_plan* pl, const void* q, const void*
   int* status = reinterpret_cast<int*>(ws + pl->ws_status);
   const unsigned grid = (unsigned)(pl->nseg < pl->num_sms ? pl->nseg : pl->num_sms);
   if (pl->dev.fp8)
-    score_select_kernel<true><<<grid, kScoreThreads, kScoreSmemBytes, st>>>(
-        mhi, mlo, mq, (const uint8_t*)q, pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
+    launch(score_select_kernel<true>, grid, kScoreThreads, kScoreSmemBytes, st, mhi, mlo, mq, (const uint8_t*)q,
+           pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
   else if (pl->dev.q_box) {
     // BF16 tiles that come as TMA boxes: pairs of adjacent tiles per pooled-key chunk.  The pair kernel takes the pooled
     // keys in pieces of 64 elements x 128 keys, which is the box of mhi / mlo already.
     const unsigned grid_pairs = (unsigned)(pl->nunits < pl->num_sms ? pl->nunits : pl->num_sms);
-    score_pair_kernel<<<grid_pairs, kPairThreads, kPairSmemBytes, st>>>(mhi, mlo, mq, mq2, pl->d_segs, pl->d_units, pl->nunits,
+    launch(score_pair_kernel, grid_pairs, kPairThreads, kPairSmemBytes, st, mhi, mlo, mq, mq2, pl->d_segs, pl->d_units, pl->nunits,
                                                                         pl->dev, seg_offset, seg_count, blk_idx, status);
   } else
-    score_select_kernel<false><<<grid, kScoreThreads, kScoreSmemBytes, st>>>(
-        mhi, mlo, mq, (const uint8_t*)q, pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
+    launch(score_select_kernel<false>, grid, kScoreThreads, kScoreSmemBytes, st, mhi, mlo, mq, (const uint8_t*)q,
+           pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
   pl->last_launches += 1;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }
@@ -509,11 +524,11 @@ static void launch_attn(fp2_plan* pl, const CUtensorMap& mk, const CUtensorMap& 
   const int64_t workers = (int64_t)pl->num_sms * AttnCfg<false>::kCtasPerSm;
   const unsigned grid = (unsigned)(max_units < workers ? max_units : workers);
   if (pl->dev.fp8)
-    sparse_attn_kernel<true><<<grid, AttnCfg<true>::kThreads, AttnCfg<true>::kSmemBytes, st>>>(mk, mv, mkb, mkb_lo,
+    launch(sparse_attn_kernel<true>, grid, AttnCfg<true>::kThreads, AttnCfg<true>::kSmemBytes, st, mk, mv, mkb, mkb_lo,
                                                                                                  mvb, mq, a, pl->dev);
   else
-    sparse_attn_kernel<false><<<grid, AttnCfg<false>::kThreads, AttnCfg<false>::kSmemBytes, st>>>(
-        mk, mv, mkb, mkb_lo, mvb, mq, a, pl->dev);
+    launch(sparse_attn_kernel<false>, grid, AttnCfg<false>::kThreads, AttnCfg<false>::kSmemBytes, st, mk, mv, mkb, mkb_lo,
+           mvb, mq, a, pl->dev);
 }
 
 static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, const void* v, const int32_t* pt,
@@ -528,7 +543,8 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   pl->last_launches = 0;
   if (pl->nseg == 0) return FP2_OK;
   if (need_pool && (s = launch_pool(pl, k, v, pt, lk, ks, vs, ws, st)) != FP2_OK) return s;
-  if ((s = launch_order(pl, seg_count, ws, st)) != FP2_OK) return s;
+  launch_order(pl, seg_count, reinterpret_cast<int32_t*>(ws + pl->ws_hist), reinterpret_cast<int32_t*>(ws + pl->ws_order),
+               reinterpret_cast<int32_t*>(ws + pl->ws_counter), st);
   const bool fp8 = pl->dev.fp8 != 0;
   const int64_t slots = (int64_t)pl->prm.num_pages * pl->prm.page_size;
   CUtensorMap mk, mv, mkb, mkb_lo, mvb;
@@ -574,7 +590,7 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
     int32_t* n_units = reinterpret_cast<int32_t*>(ws + pl->ws_counter) + 1;
     int32_t* n_split = n_units + 1;
     const int workers = pl->num_sms * AttnCfg<false>::kCtasPerSm;
-    split_plan_kernel<<<1, 1024, 0, st>>>(pl->d_segs, a.order, seg_count, (int)pl->nseg, pl->dev.use_correction,
+    launch(split_plan_kernel, 1, 1024, 0, st, pl->d_segs, a.order, seg_count, (int)pl->nseg, pl->dev.use_correction,
                                           workers, pl->split_target, unit_seg, unit_split, seg_split, split_list, n_units,
                                           n_split);
     pl->last_launches += 1;
@@ -591,8 +607,8 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   pl->last_launches += 1;
   if (split) {
     int32_t* seg_split = reinterpret_cast<int32_t*>(ws + pl->ws_seg_split);
-    split_combine_kernel<<<(unsigned)(pl->num_sms * 8), 128, 0, st>>>(
-        pl->d_segs, seg_split, seg_split + pl->nseg, reinterpret_cast<int32_t*>(ws + pl->ws_counter) + 2, a.part_o,
+    launch(split_combine_kernel, (unsigned)(pl->num_sms * 8), 128, 0, st, pl->d_segs, seg_split, seg_split + pl->nseg,
+           reinterpret_cast<int32_t*>(ws + pl->ws_counter) + 2, a.part_o,
         a.part_ml, fp8 ? vs : nullptr, pl->dev, a.out, lse);
     pl->last_launches += 1;
   }
@@ -625,7 +641,7 @@ constexpr int kStaticMaxSegments = 65536;
 constexpr int kStaticMaxKvHeads = 32;
 constexpr size_t kStaticOffOrder = 1024;
 constexpr size_t kStaticOffHist = kStaticOffOrder + sizeof(int32_t) * kStaticMaxSegments;
-constexpr size_t kStaticBytes = kStaticOffHist + sizeof(int32_t) * ((size_t)kStaticMaxKvHeads * kCountBuckets + 256);
+constexpr size_t kStaticBytes = kStaticOffHist + sizeof(int32_t) * (size_t)kStaticMaxKvHeads * kCountBuckets * 2;
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
 // In host code `g_static_scratch` is only a handle; the device address comes from cudaGetSymbolAddress,
@@ -663,17 +679,10 @@ extern "C" fp2_status fp2_dense_prefill_static(fp2_plan* pl, const void* q, cons
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   pl->last_launches = 0;
   if (pl->nseg == 0) return FP2_OK;
-  const int nseg = (int)pl->nseg;
   int32_t* order = reinterpret_cast<int32_t*>(sw + kStaticOffOrder);
-  int32_t* hist = reinterpret_cast<int32_t*>(sw + kStaticOffHist);
-  const int nb = pl->prm.num_kv_heads * kCountBuckets;
-  // the array keeps the previous call's contents: status, counter and histogram must start at zero
-  if (cudaMemsetAsync(sw, 0, 1024, st) != cudaSuccess) return FP2_ERR_CUDA;
-  if (cudaMemsetAsync(hist, 0, sizeof(int32_t) * (size_t)(nb + 1), st) != cudaSuccess) return FP2_ERR_CUDA;
-  const int blocks = (nseg + 255) / 256;
-  order_hist_kernel<<<blocks, 256, 0, st>>>(pl->d_segs, nullptr, nseg, hist);
-  order_scan_kernel<<<1, 1024, 0, st>>>(hist, nb);
-  order_scatter_kernel<<<blocks, 256, 0, st>>>(pl->d_segs, nullptr, nseg, hist, order);
+  // the array keeps the previous call's contents: the status block must start at zero (the sort clears the rest)
+  if (cudaMemsetAsync(sw, 0, 64, st) != cudaSuccess) return FP2_ERR_CUDA;
+  launch_order(pl, nullptr, reinterpret_cast<int32_t*>(sw + kStaticOffHist), order, reinterpret_cast<int32_t*>(sw + 64), st);
   const int64_t slots = (int64_t)pl->prm.num_pages * pl->prm.page_size;
   CUtensorMap mk, mv;
   const bool fp8 = pl->dev.fp8 != 0;
@@ -781,11 +790,11 @@ extern "C" fp2_status fp2_export_csr(fp2_plan* pl, const int32_t* seg_count, con
   int* status = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(workspace) + pl->ws_status);
   const int nseg = (int)pl->nseg;
   pl->last_launches = 0;
-  csr_count_kernel<<<(nseg + 256) / 256, 256, 0, st>>>(pl->d_segs, seg_count, blk_idx, nseg, tile_tokens, cu, status);
+  launch(csr_count_kernel, (nseg + 256) / 256, 256, 0, st, pl->d_segs, seg_count, blk_idx, nseg, tile_tokens, cu, status);
   pl->last_launches += 1;
   if (nseg > 0) {
-    csr_scan_kernel<<<1, 1024, 0, st>>>(cu, nseg);
-    csr_fill_kernel<<<(unsigned)(((int64_t)nseg * 32 + 255) / 256), 256, 0, st>>>(pl->d_segs, seg_count, blk_idx, nseg,
+    launch(csr_scan_kernel, 1, 1024, 0, st, cu, nseg);
+    launch(csr_fill_kernel, (unsigned)(((int64_t)nseg * 32 + 255) / 256), 256, 0, st, pl->d_segs, seg_count, blk_idx, nseg,
                                                                                  tile_tokens, cu, idx, status);
     pl->last_launches += 2;
   }
@@ -806,8 +815,8 @@ extern "C" fp2_status fp2_page_table_from_token_map(fp2_plan* pl, const int32_t*
   const int64_t n = (int64_t)pl->prm.num_seqs * pl->prm.max_pages_per_seq;
   pl->last_launches = 0;
   if (n == 0) return FP2_OK;
-  page_table_from_token_map_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-      token_to_slot, max_tokens, seqlens_k, pl->prm.num_seqs, pl->prm.page_size, pl->prm.max_pages_per_seq, page_table,
+  launch(page_table_from_token_map_kernel, (unsigned)((n + 255) / 256), 256, 0, st, token_to_slot, max_tokens,
+         seqlens_k, pl->prm.num_seqs, pl->prm.page_size, pl->prm.max_pages_per_seq, page_table,
       status);
   pl->last_launches = 1;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;

@@ -30,9 +30,11 @@ __device__ __forceinline__ int clamped_count(const SegInfo& sg, const int32_t* s
 }
 
 // cu[g + 1] = number of tiles of segment g; cu[0] = 0.  One thread per segment.
-__global__ void csr_count_kernel(const SegInfo* __restrict__ segs, const int32_t* __restrict__ seg_count,
-                                 const int32_t* __restrict__ blk_idx, int nseg, int tile_tokens,
+__global__ void csr_count_kernel(const SegInfo* __restrict__ segs, const int32_t* seg_count,
+                                 const int32_t* blk_idx, int nseg, int tile_tokens,
                                  int32_t* __restrict__ cu, int* __restrict__ status) {
+  pdl_trigger();
+  pdl_wait();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g == 0) cu[0] = 0;
   if (g >= nseg) return;
@@ -54,6 +56,8 @@ constexpr int kScanPerThread = 8;
 __global__ void __launch_bounds__(1024, 1) csr_scan_kernel(int32_t* __restrict__ cu, int n) {
   __shared__ int32_t warp_tot[32];
   __shared__ int32_t s_carry;
+  pdl_trigger();
+  pdl_wait();
   int32_t* v = cu + 1;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   if (t == 0) s_carry = 0;
@@ -96,9 +100,11 @@ __global__ void __launch_bounds__(1024, 1) csr_scan_kernel(int32_t* __restrict__
 }
 
 // one warp per segment: entry k of the list -> its tiles at cu[g] + k tpb
-__global__ void csr_fill_kernel(const SegInfo* __restrict__ segs, const int32_t* __restrict__ seg_count,
-                                const int32_t* __restrict__ blk_idx, int nseg, int tile_tokens,
-                                const int32_t* __restrict__ cu, int32_t* __restrict__ idx, int* __restrict__ status) {
+__global__ void csr_fill_kernel(const SegInfo* __restrict__ segs, const int32_t* seg_count,
+                                const int32_t* blk_idx, int nseg, int tile_tokens,
+                                const int32_t* cu, int32_t* __restrict__ idx, int* __restrict__ status) {
+  pdl_trigger();
+  pdl_wait();
   const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (g >= nseg) return;
   const SegInfo sg = segs[g];
@@ -120,9 +126,11 @@ __global__ void csr_fill_kernel(const SegInfo* __restrict__ segs, const int32_t*
 
 // page_table[b][k] = token_to_slot[b][k p] / p for the pages that hold a token, -1 beyond (Sec. 3.4).  A sampled
 // slot that is not the first of a page is flagged in the status block.
-__global__ void page_table_from_token_map_kernel(const int32_t* __restrict__ token_to_slot, int max_tokens,
-                                                 const int32_t* __restrict__ seqlens_k, int ns, int p, int max_pages,
+__global__ void page_table_from_token_map_kernel(const int32_t* token_to_slot, int max_tokens,
+                                                 const int32_t* seqlens_k, int ns, int p, int max_pages,
                                                  int32_t* __restrict__ page_table, int* __restrict__ status) {
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= ns * max_pages) return;
   const int b = i / max_pages, k = i % max_pages;

@@ -82,7 +82,7 @@ __device__ __forceinline__ void write_pooled(int which, float mean, size_t o, in
 template <bool FP8>
 __global__ void __launch_bounds__(256, 4) pool_kv_kernel(const uint8_t* __restrict__ k_cache,
                                                          const uint8_t* __restrict__ v_cache,
-                                                         const int32_t* __restrict__ page_table,
+                                                         const int32_t* page_table,
                                                          const int32_t* __restrict__ plan_lk,  // [ns], the plan's copy
                                                          const int32_t* __restrict__ blk_off,  // [ns+1]
                                                          const float* __restrict__ k_scale,
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(256, 4) pool_kv_kernel(const uint8_t* __restri
                                                          __nv_bfloat16* __restrict__ vbar,
                                                          uint8_t* __restrict__ kbar8_hi,
                                                          uint8_t* __restrict__ kbar8_lo,
-                                                         const int32_t* __restrict__ carry,
+                                                         const int32_t* carry,
                                                          int* __restrict__ status) {
   constexpr int ROW_BYTES = FP8 ? 128 : 256;
   constexpr int CHUNKS = ROW_BYTES / 16;       // 16-byte chunks per token row
@@ -101,6 +101,8 @@ __global__ void __launch_bounds__(256, 4) pool_kv_kernel(const uint8_t* __restri
   constexpr int PASSES = kBlock / ROWS_PER_PASS;
 
   __shared__ float red[ROWS_PER_PASS][kHeadDim + 4];
+  pdl_trigger();
+  pdl_wait();
 
   const int which = blockIdx.x & 1;            // 0: K, 1: V
   const int bh = blockIdx.x >> 1;
@@ -170,7 +172,7 @@ __global__ void __launch_bounds__(256, 4) pool_kv_kernel(const uint8_t* __restri
 template <bool FP8>
 __global__ void __launch_bounds__(256, 4) pool_rows_kernel(const uint8_t* __restrict__ k_cache,
                                                            const uint8_t* __restrict__ v_cache,
-                                                           const int32_t* __restrict__ page_table,
+                                                           const int32_t* page_table,
                                                            const int32_t* __restrict__ plan_lk,
                                                            const int32_t* __restrict__ blk_off,
                                                            const float* __restrict__ k_scale,
@@ -180,7 +182,7 @@ __global__ void __launch_bounds__(256, 4) pool_rows_kernel(const uint8_t* __rest
                                                            __nv_bfloat16* __restrict__ vbar,
                                                            uint8_t* __restrict__ kbar8_hi,
                                                            uint8_t* __restrict__ kbar8_lo,
-                                                           const int32_t* __restrict__ carry,
+                                                           const int32_t* carry,
                                                            int* __restrict__ status) {
   constexpr int CH = FP8 ? 8 : 16;             // 16-byte chunks per head row
   constexpr int EPC = FP8 ? 16 : 8;            // elements per chunk
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(256, 4) pool_rows_kernel(const uint8_t* __rest
   __shared__ float red[256 * EPC];             // [token group][chunk][element]
   __shared__ int32_t pids[kBlock / 8];         // page ids of the block (page size >= 8)
 
+  pdl_trigger();
   const int which = blockIdx.x & 1;            // 0: K, 1: V
   const int gblk = blockIdx.x >> 1;
   int lo = 0, hi = P.num_seqs;
@@ -195,7 +198,8 @@ __global__ void __launch_bounds__(256, 4) pool_rows_kernel(const uint8_t* __rest
     int mid = (lo + hi) >> 1;
     if (blk_off[mid] <= gblk) lo = mid; else hi = mid;
   }
-  const int b = lo, J = gblk - blk_off[b];
+  const int b = lo, J = gblk - blk_off[b];   // (the plan's table so far: not written by any kernel)
+  pdl_wait();
   if (carry != nullptr && J < carry[3 * b + 2]) return;   // carried over from the previous chunk (pool_carry_kernel)
   const int Lk = plan_lk[b];
   const int ntok = min(kBlock, Lk - J * kBlock);
@@ -257,52 +261,60 @@ __global__ void __launch_bounds__(256, 4) pool_rows_kernel(const uint8_t* __rest
 
 // ----------------------------------------------------------------------------------------
 // Work ordering (Sec. 3.3 "Sparsity-Aware Load Balancing", Eq. 21): segments sorted KV-head-major, then by
-// descending block count (capped), by a counting sort on the device.  Order among equal keys is arbitrary;
-// it only changes which CTA runs a segment, never a result.
+// descending block count, by a counting sort on the device.  Counts below 64 are classes of their own, larger ones fall
+// into eight classes per power of two: heaviest-first needs no finer order, and with 128 classes per head (1024 before)
+// the last kernel finds its own offsets instead of waiting for a kernel that scans the histogram (3 us at 64 segments,
+// 9 us at 44000).  Order inside a class is arbitrary; it only changes which CTA runs a segment,
+// never a result.
 // ----------------------------------------------------------------------------------------
 __device__ __forceinline__ int order_bucket(int h, int count) {
-  int c = count < kCountBuckets - 1 ? count : kCountBuckets - 1;
+  int c = max(count, 0);
+  if (c >= 64) {
+    const int e = 31 - __clz(c);                                    // 6 .. : c in [2^e, 2^(e+1))
+    c = min(64 + (e - 6) * 8 + ((c >> (e - 3)) & 7), kCountBuckets - 1);
+  }
   return h * kCountBuckets + (kCountBuckets - 1 - c);
 }
 
-__global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_t* __restrict__ count, int nseg,
+// Clears histogram and cursors (2 nb words) and the work counter block (16 words).
+__global__ void order_clear_kernel(int32_t* __restrict__ hist, int nb2, int32_t* __restrict__ counter) {
+  pdl_trigger();
+  pdl_wait();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nb2) hist[i] = 0;
+  if (i < 16) counter[i] = 0;
+}
+
+__global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_t* count, int nseg,
                                   int32_t* __restrict__ hist) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_trigger();
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int h = s < nseg ? segs[s].h : 0, J = s < nseg ? segs[s].J_hi : 0;   // the plan's table: not written by any kernel
+  pdl_wait();
   if (s >= nseg) return;
-  int c = count ? count[s] : segs[s].J_hi + 1;
-  atomicAdd(&hist[order_bucket(segs[s].h, c)], 1);
+  atomicAdd(&hist[order_bucket(h, count ? count[s] : J + 1)], 1);
 }
 
-// single CTA of 1024 threads: exclusive scan of nb = Hkv * kCountBuckets counters, in place.
-__global__ void order_scan_kernel(int32_t* __restrict__ hist, int nb) {
-  __shared__ int32_t part[1024];
-  const int per = (nb + 1023) / 1024;
-  const int beg = threadIdx.x * per, end = min(beg + per, nb);
-  int s = 0;
-  for (int i = beg; i < end; ++i) s += hist[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int d = 1; d < 1024; d <<= 1) {
-    int v = threadIdx.x >= d ? part[threadIdx.x - d] : 0;
-    __syncthreads();
-    part[threadIdx.x] += v;
-    __syncthreads();
-  }
-  int run = part[threadIdx.x] - s;
-  for (int i = beg; i < end; ++i) {
-    int v = hist[i];
-    hist[i] = run;
-    run += v;
-  }
-}
-
-__global__ void order_scatter_kernel(const SegInfo* __restrict__ segs, const int32_t* __restrict__ count, int nseg,
-                                     int32_t* __restrict__ cursor, int32_t* __restrict__ order) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
+// Every KV head has the same number of segments, so a segment's place is its head's share, the classes before its own, and
+// a cursor inside the class: each thread adds up the (at most 128) counts in front of it, which the L1 holds.
+__global__ void order_scatter_kernel(const SegInfo* __restrict__ segs, const int32_t* count, int nseg,
+                                     int per_head, const int32_t* hist, int32_t* __restrict__ cursor,
+                                     int32_t* __restrict__ order) {
+  pdl_trigger();
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int h = s < nseg ? segs[s].h : 0, J = s < nseg ? segs[s].J_hi : 0;
+  pdl_wait();
   if (s >= nseg) return;
-  int c = count ? count[s] : segs[s].J_hi + 1;
-  int pos = atomicAdd(&cursor[order_bucket(segs[s].h, c)], 1);
-  order[pos] = s;
+  const int b = order_bucket(h, count ? count[s] : J + 1), before = b - h * kCountBuckets;
+  int pos = h * per_head;
+  const int4* c4 = reinterpret_cast<const int4*>(hist + h * kCountBuckets);
+#pragma unroll 4
+  for (int i = 0; i < before / 4; ++i) {
+    const int4 c = c4[i];
+    pos += c.x + c.y + c.z + c.w;
+  }
+  for (int i = before & ~3; i < before; ++i) pos += hist[h * kCountBuckets + i];
+  order[pos + atomicAdd(&cursor[b], 1)] = s;
 }
 
 // ----------------------------------------------------------------------------------------
@@ -312,12 +324,14 @@ __global__ void order_scatter_kernel(const SegInfo* __restrict__ segs, const int
 // layout to this plan's.  carry[3 b + {0, 1, 2}] = first source row, first destination row, rows to copy of
 // sequence b.  grid (sequences, row groups of 8); a row of one array is Hkv x 128 elements.
 // ----------------------------------------------------------------------------------------
-__global__ void pool_carry_kernel(const int32_t* __restrict__ carry, int row_bytes16, int row_bytes8,
+__global__ void pool_carry_kernel(const int32_t* carry, int row_bytes16, int row_bytes8,
                                   const uint8_t* __restrict__ s_khi, const uint8_t* __restrict__ s_klo,
                                   const uint8_t* __restrict__ s_vbar, const uint8_t* __restrict__ s_k8hi,
                                   const uint8_t* __restrict__ s_k8lo, uint8_t* __restrict__ d_khi,
                                   uint8_t* __restrict__ d_klo, uint8_t* __restrict__ d_vbar,
                                   uint8_t* __restrict__ d_k8hi, uint8_t* __restrict__ d_k8lo) {
+  pdl_trigger();
+  pdl_wait();
   const int b = blockIdx.x;
   const int src0 = carry[3 * b], dst0 = carry[3 * b + 1], n = carry[3 * b + 2];
   for (int j = blockIdx.y * 8; j < n; j += gridDim.y * 8) {

@@ -148,6 +148,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
+  pdl_trigger();
+  pdl_wait();
   // chunks of a unit: those of its last tile (the later tile of a pair has the larger candidate range)
   auto unit_chunks = [](const PairInfo& pi) { return (pi.sg[pi.nt - 1].J_hi + 128) >> 7; };
 

@@ -291,6 +291,8 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
+  pdl_trigger();
+  pdl_wait();
 
   if (warp == 10) {
     // ---------------- set-up (warp 10): segment k of this CTA is number blockIdx.x + k * gridDim.x in heaviest-first order

@@ -279,6 +279,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
+  pdl_trigger();
+  pdl_wait();
   const int g = P.group;
 
   // O += P V (G) has completed.  Safe for a waiter that is at most two iterations behind the issuer.

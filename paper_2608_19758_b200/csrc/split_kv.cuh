@@ -24,12 +24,14 @@ constexpr int kMinPartLen = 12;     // iterations per part below which splitting
 __host__ __device__ inline int32_t pack_split(int u, int U, int slot) { return u | (U << 8) | (slot << 16); }
 
 __global__ void __launch_bounds__(1024, 1)
-split_plan_kernel(const SegInfo* __restrict__ segs, const int32_t* __restrict__ order,
-                  const int32_t* __restrict__ seg_count, int nseg, int use_correction, int workers, int target,
+split_plan_kernel(const SegInfo* __restrict__ segs, const int32_t* order,
+                  const int32_t* seg_count, int nseg, int use_correction, int workers, int target,
                   int32_t* __restrict__ unit_seg, int32_t* __restrict__ unit_split, int32_t* __restrict__ seg_split,
                   int32_t* __restrict__ split_list, int32_t* __restrict__ n_units, int32_t* __restrict__ n_split) {
   __shared__ int32_t part_a[1024], part_b[1024], part_c[1024];
   __shared__ int s_total;
+  pdl_trigger();
+  pdl_wait();
   const int t = threadIdx.x;
   const int per = (nseg + 1023) / 1024;
   const int beg = min(t * per, nseg), end = min(beg + per, nseg);
@@ -95,11 +97,13 @@ split_plan_kernel(const SegInfo* __restrict__ segs, const int32_t* __restrict__ 
 constexpr int kMergeRows = 8;
 
 __global__ void __launch_bounds__(128)
-split_combine_kernel(const SegInfo* __restrict__ segs, const int32_t* __restrict__ seg_split,
-                     const int32_t* __restrict__ split_list, const int32_t* __restrict__ n_split,
-                     const float* __restrict__ part_o, const float2* __restrict__ part_ml,
+split_combine_kernel(const SegInfo* __restrict__ segs, const int32_t* seg_split,
+                     const int32_t* split_list, const int32_t* n_split,
+                     const float* part_o, const float2* part_ml,
                      const float* __restrict__ v_scale, DevParams P, __nv_bfloat16* __restrict__ out,
                      float* __restrict__ lse) {
+  pdl_trigger();
+  pdl_wait();
   constexpr int kGroups = 128 / kMergeRows;
   const int n_items = *n_split * kGroups;
   for (int item = blockIdx.x; item < n_items; item += gridDim.x) {

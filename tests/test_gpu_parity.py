@@ -575,3 +575,29 @@ def test_group_sizes_whose_query_tiles_start_inside_a_box(g, dtype):
         gl = dc.lse.cpu().numpy().astype(np.float64)
         ok = ~np.isnan(Lo)
         assert (np.abs(gl - Lo)[ok] / np.maximum(np.abs(Lo[ok]), 1.0)).max() <= TOL_LSE_REL
+
+
+@pytest.mark.parametrize("n_seg_tokens", [1, 63, 64, 65, 1000])
+def test_work_order_takes_every_segment_once(n_seg_tokens):
+    """The counting sort behind the attention call: caller lists whose lengths sit on the edges of the sort's classes (0,
+    1, 63, 64, 71, 72, 127, 128, 255, 256, 257 blocks), so that a segment dropped or taken twice would leave its rows at the
+    poison value or race on them; compared with the dense result of the same rows where the list is complete."""
+    lk = 257 * 128
+    spec = inputs.small_spec(seqs=[(lk, lk - n_seg_tokens), (300, 0)], num_q_heads=3, num_kv_heads=3, page_size=128,
+                             config_id=150)
+    case, dc, wl = make(spec, use_correction=0)
+    dc.select()
+    dc.status()
+    off = dc.seg_offset.cpu().numpy()
+    edges = [0, 1, 63, 64, 71, 72, 127, 128, 255, 256, 257]
+    cnt = np.zeros(dc.plan.num_segments, dtype=np.int32)
+    idx = dc.blk_idx.cpu().numpy().copy()
+    for s in wl.segs:
+        n = min(edges[s.seg % len(edges)], s.J_hi + 1)
+        cnt[s.seg] = n
+        idx[off[s.seg]:off[s.seg] + n] = np.arange(s.J_hi + 1 - n, s.J_hi + 1)
+    dc.sparse(seg_count=torch.from_numpy(cnt).cuda(), blk_idx=torch.from_numpy(idx).cuda())
+    dc.status()
+    lists = {s.seg: idx[off[s.seg]:off[s.seg] + cnt[s.seg]] for s in wl.segs if cnt[s.seg] > 0}
+    check_attention(dc, wl, lists, list(lists))
+    assert torch.isfinite(dc.out.float()).all()     # rows without a block come out as zeros
