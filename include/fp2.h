@@ -92,7 +92,8 @@ fp2_status fp2_plan_create(const fp2_params* params, const int32_t* h_cu_seqlens
                            fp2_plan** out);
 
 /* Sizes the caller needs: number of segments, capacity of blk_idx in entries (worst case = all candidate
- * pairs), bytes of device workspace (pooled statistics, work order, status block).  Any output may be NULL. */
+ * pairs), bytes of device workspace (pooled statistics, work order, status block; for FP8 plans with enough work also V
+ * as F16, 2 bytes per element of the sequences' values, rewritten by every attention call).  Any output may be NULL. */
 fp2_status fp2_plan_sizes(const fp2_plan* plan, int64_t* num_segments, int64_t* idx_capacity,
                           int64_t* workspace_bytes);
 

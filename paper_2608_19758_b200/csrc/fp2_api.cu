@@ -43,10 +43,12 @@ struct fp2_plan {
   std::vector<int32_t> h_blk_off, h_carry;
   bool carry_valid;
   // workspace layout (byte offsets)
-  int64_t ws_status, ws_counter, ws_khi, ws_klo, ws_vbar, ws_k8hi, ws_k8lo, ws_order, ws_hist, ws_bytes;
+  int64_t ws_status, ws_counter, ws_khi, ws_klo, ws_vbar, ws_k8hi, ws_k8lo, ws_v16, ws_order, ws_hist, ws_bytes;
   // KV splitting (Eq. 18): only plans with few segments carry the buffers
   bool split_capable;
   int32_t split_target;   // < 0 off, 0 automatic, > 0 requested iterations per part
+  int64_t v16_iters;      // FP8: iterations of an attention call from which V as F16 pays (see use_v16)
+  int64_t likely_iters;   // FP8: iterations a sparse call can be expected to have
   int32_t max_iters;      // longest iteration sequence any segment can have (all candidates + all chunks)
   int64_t split_units_cap, ws_unit_seg, ws_unit_split, ws_seg_split, ws_part_ml, ws_part_o;
   EncodeTiledFn encode;
@@ -54,6 +56,14 @@ struct fp2_plan {
   bool attrs_set;
 };
 
+// FP8 attention with V as F16 in the workspace, or widened by the kernel in every iteration?  The copy takes about 6 us and
+// 11 ns per block of a KV head (3 bytes per element at 4.5 TB/s); an iteration without the widening is 450 cycles of an SM
+// shorter (900 of one of its two CTAs), 1.6 ns over 148 SMs.  So it pays from 4000 + 7 blocks x heads iterations.  Measured
+// (whole calls, widened per iteration / copy): 700 tokens, 32 heads on 8 48.3 / 56.4 us, 2000 tokens, 28 on 4 78.8 / 81.1,
+// 8191 tokens 267 / 236, 131072 tokens 8985 / 7990, its last 8192 tokens 777 / 729, 16 sequences of 245000 tokens
+// 3824 / 3579, dense 16384 tokens 1782 / 1486.  A sparse call's lists are not known on the host: 20 blocks per tile (sink,
+// window and diagonal are 7 to 8 of them).
+constexpr int kLikelyListLen = 20;
 static inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 extern "C" const char* fp2_status_string(fp2_status s) {
@@ -136,13 +146,16 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
   }
   blk_off[p->num_seqs] = (int32_t)boff;
   pl->max_iters = 0;
+  pl->likely_iters = 0;
   for (int64_t i = 0; i < pl->nseg; ++i) {
+    pl->likely_iters += std::min(segs[(size_t)i].J_hi + 1, kLikelyListLen);
     segs[(size_t)i].off = off;
     off += segs[(size_t)i].J_hi + 1;
     const int iters = segs[(size_t)i].J_hi + 1 + (segs[(size_t)i].J_lo + 127) / 128;
     pl->max_iters = iters > pl->max_iters ? iters : pl->max_iters;
   }
   pl->idx_capacity = off;
+  pl->v16_iters = 4000 + 7 * nblk_tot * p->num_kv_heads;
   pl->h_blk_off = blk_off;
   pl->carry_valid = false;
   pl->d_carry = nullptr;
@@ -237,6 +250,10 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
   const int64_t pooled8 = p->dtype == FP2_FP8_E4M3 ? align_up(nblk_tot * p->num_kv_heads * kHeadDim, 1024) : 0;
   pl->ws_k8hi = o; o += pooled8;
   pl->ws_k8lo = o; o += pooled8;
+  // and V as F16 (attention kernel, see use_v16)
+  pl->ws_v16 = o;
+  if (p->dtype == FP2_FP8_E4M3 && pl->idx_capacity >= pl->v16_iters)   // (a dense call has that many iterations)
+    o += align_up(nblk_tot * kBlock * p->num_kv_heads * kHeadDim * 2, 1024);
   pl->ws_order = o; o += align_up(4 * (pl->nseg > 0 ? pl->nseg : 1), 1024);
   pl->ws_hist = o;  o += align_up(8 * (int64_t)p->num_kv_heads * kCountBuckets, 1024);
   // KV splitting pays when there are fewer units than a few waves of workers; the unit arrays and the partial
@@ -367,17 +384,21 @@ static fp2_status set_attrs(fp2_plan* pl) {
                            kScoreSmemBytes) != cudaSuccess ||
       cudaFuncSetAttribute(score_select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kScoreSmemBytes) != cudaSuccess ||
-      cudaFuncSetAttribute(sparse_attn_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(sparse_attn_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            AttnCfg<false>::kSmemBytes) != cudaSuccess ||
-      cudaFuncSetAttribute(sparse_attn_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(sparse_attn_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           AttnCfg<true>::kSmemBytes) != cudaSuccess ||
+      cudaFuncSetAttribute(sparse_attn_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            AttnCfg<true>::kSmemBytes) != cudaSuccess)
     return FP2_ERR_CUDA;
   // The attention kernels move registers between warps with setmaxnreg, whose wait is unbounded: launch only
   // if the compiled kernels really own the registers the move assumes.
   cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, sparse_attn_kernel<false>) != cudaSuccess) return FP2_ERR_CUDA;
+  if (cudaFuncGetAttributes(&fa, sparse_attn_kernel<false, false>) != cudaSuccess) return FP2_ERR_CUDA;
   if (fa.numRegs * AttnCfg<false>::kThreads < AttnCfg<false>::kRegsAfterMove) return FP2_ERR_UNSUPPORTED;
-  if (cudaFuncGetAttributes(&fa, sparse_attn_kernel<true>) != cudaSuccess) return FP2_ERR_CUDA;
+  if (cudaFuncGetAttributes(&fa, sparse_attn_kernel<true, false>) != cudaSuccess) return FP2_ERR_CUDA;
+  if (fa.numRegs * AttnCfg<true>::kThreads < AttnCfg<true>::kRegsAfterMove) return FP2_ERR_UNSUPPORTED;
+  if (cudaFuncGetAttributes(&fa, sparse_attn_kernel<true, true>) != cudaSuccess) return FP2_ERR_CUDA;
   if (fa.numRegs * AttnCfg<true>::kThreads < AttnCfg<true>::kRegsAfterMove) return FP2_ERR_UNSUPPORTED;
   pl->attrs_set = true;
   return FP2_OK;
@@ -398,48 +419,35 @@ static fp2_status check_common(fp2_plan* pl, const void* q, const void* k, const
   return set_attrs(pl);
 }
 
-static fp2_status launch_pool(fp2_plan* pl, const void* k, const void* v, const int32_t* pt, const int32_t* lk,
-                              const float* ks, const float* vs, uint8_t* ws, cudaStream_t st,
-                              const int32_t* carry = nullptr) {
+static fp2_status launch_pool(fp2_plan* pl, const void* k, const void* v, const int32_t* pt, const float* ks, const float* vs,
+                              uint8_t* ws, cudaStream_t st, const int32_t* carry = nullptr) {
   if (pl->nblk_tot == 0) return FP2_OK;
-  const unsigned grid = (unsigned)(pl->nblk_tot * pl->prm.num_kv_heads * 2);   // K and V pooled by separate CTAs
   __nv_bfloat16* khi = reinterpret_cast<__nv_bfloat16*>(ws + pl->ws_khi);
   __nv_bfloat16* klo = reinterpret_cast<__nv_bfloat16*>(ws + pl->ws_klo);
   __nv_bfloat16* vb = reinterpret_cast<__nv_bfloat16*>(ws + pl->ws_vbar);
   int* status = reinterpret_cast<int*>(ws + pl->ws_status);
-  (void)lk;   // the lengths the kernel uses are the plan's own copy
-  // whole cache rows per CTA when a row's 16-byte chunks divide 256 (see pool_rows_kernel), else one head per CTA
+  // whole cache rows per CTA when a row's 16-byte chunks divide 256 (see pool_rows_kernel), else one head per CTA;
+  // K and V pooled by separate CTAs.  The lengths the kernels use are the plan's own copy.
   const int row_chunks = pl->prm.num_kv_heads * (pl->dev.fp8 ? 8 : 16);
-  if (row_chunks <= 256 && 256 % row_chunks == 0) {
-    const unsigned grid_rows = (unsigned)(pl->nblk_tot * 2);
-    if (pl->dev.fp8)
-      launch(pool_rows_kernel<true>, grid_rows, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off,
-                                                        ks, vs, pl->dev, khi, klo, vb, ws + pl->ws_k8hi,
-                                                        ws + pl->ws_k8lo, carry, status);
-    else
-      launch(pool_rows_kernel<false>, grid_rows, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk,
-                                                         pl->d_blk_off, ks, vs, pl->dev, khi, klo, vb, nullptr, nullptr,
-                                                         carry, status);
-    pl->last_launches += 1;
-    return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
-  }
-  if (pl->dev.fp8)
-    launch(pool_kv_kernel<true>, grid, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs,
-                                               pl->dev, khi, klo, vb, ws + pl->ws_k8hi, ws + pl->ws_k8lo, carry, status);
-  else
-    launch(pool_kv_kernel<false>, grid, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs,
-                                                pl->dev, khi, klo, vb, nullptr, nullptr, carry, status);
+  const bool rows = row_chunks <= 256 && 256 % row_chunks == 0;
+  const unsigned grid = (unsigned)(pl->nblk_tot * (rows ? 1 : pl->prm.num_kv_heads) * 2);
+  auto kernel = pl->dev.fp8 ? (rows ? pool_rows_kernel<true> : pool_kv_kernel<true>)
+                            : (rows ? pool_rows_kernel<false> : pool_kv_kernel<false>);
+  launch(kernel, grid, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs, pl->dev, khi,
+         klo, vb, ws + pl->ws_k8hi, ws + pl->ws_k8lo, carry, status);
   pl->last_launches += 1;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }
 
-// counting sort of the segments: KV-head-major, descending block count.  hist: class counts and cursors (2 nb words).
-static void launch_order(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, int32_t* counter,
-                         cudaStream_t st) {
+// What an attention call runs before its kernel: the counting sort of the segments (KV-head-major, descending block count;
+// hist: class counts and cursors, 2 nb words), and for FP8 plans with a workspace V as F16 (v16, else NULL).
+static void launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, int32_t* counter,
+                           const void* v, const int32_t* pt, __half* v16, int* status, cudaStream_t st) {
   const int nseg = (int)pl->nseg;
   const int nb = pl->prm.num_kv_heads * kCountBuckets;
-  const unsigned blocks = (unsigned)((nseg + 255) / 256);
-  launch(order_clear_kernel, (unsigned)((2 * nb + 255) / 256), 256, 0, st, hist, 2 * nb, counter);
+  const unsigned blocks = (unsigned)((nseg + 255) / 256), n_clear = (unsigned)((2 * nb + 255) / 256);
+  launch(attn_prepare_kernel, n_clear + (v16 ? (unsigned)(pl->nblk_tot * (kBlock / kWidenTokens)) : 0u), 256, 0, st, hist, 2 * nb, counter, (int)n_clear,
+         (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, pl->dev, v16, status);
   launch(order_hist_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, hist);
   launch(order_scatter_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, nseg / pl->prm.num_kv_heads, hist,
          hist + nb, order);
@@ -463,7 +471,7 @@ extern "C" fp2_status fp2_select_blocks(fp2_plan* pl, const void* q, const void*
   // pooled rows carried over by fp2_pool_carry are used once: by this call
   const int32_t* carry = pl->carry_valid ? pl->d_carry : nullptr;
   pl->carry_valid = false;
-  if ((s = launch_pool(pl, k, v, pt, lk, ks, vs, ws, st, carry)) != FP2_OK) return s;
+  if ((s = launch_pool(pl, k, v, pt, ks, vs, ws, st, carry)) != FP2_OK) return s;
   CUtensorMap mhi, mlo;
   if (!make_map(pl, &mhi, ws + pl->ws_khi, pl->nblk_tot, pl->prm.num_kv_heads, 128, false) ||
       !make_map(pl, &mlo, ws + pl->ws_klo, pl->nblk_tot, pl->prm.num_kv_heads, 128, false))
@@ -503,7 +511,7 @@ extern "C" fp2_status fp2_pool_blocks(fp2_plan* pl, const void* k, const void* v
   if (cudaGetDevice(&dev) != cudaSuccess) return FP2_ERR_CUDA;
   if (dev != pl->device) return FP2_ERR_INVALID_ARG;
   pl->last_launches = 0;
-  return launch_pool(pl, k, v, pt, lk, ks, vs, reinterpret_cast<uint8_t*>(workspace),
+  return launch_pool(pl, k, v, pt, ks, vs, reinterpret_cast<uint8_t*>(workspace),
                      reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -520,15 +528,12 @@ extern "C" void fp2_debug_set_score_prof(long long* p) { cudaMemcpyToSymbol(fp2:
 
 static void launch_attn(fp2_plan* pl, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mkb,
                         const CUtensorMap& mkb_lo, const CUtensorMap& mvb, const CUtensorMap& mq, const AttnArgs& a,
-                        int64_t max_units, cudaStream_t st) {
+                        int64_t max_units, bool widen, cudaStream_t st) {
   const int64_t workers = (int64_t)pl->num_sms * AttnCfg<false>::kCtasPerSm;
   const unsigned grid = (unsigned)(max_units < workers ? max_units : workers);
-  if (pl->dev.fp8)
-    launch(sparse_attn_kernel<true>, grid, AttnCfg<true>::kThreads, AttnCfg<true>::kSmemBytes, st, mk, mv, mkb, mkb_lo,
-                                                                                                 mvb, mq, a, pl->dev);
-  else
-    launch(sparse_attn_kernel<false>, grid, AttnCfg<false>::kThreads, AttnCfg<false>::kSmemBytes, st, mk, mv, mkb, mkb_lo,
-           mvb, mq, a, pl->dev);
+  auto kernel = !pl->dev.fp8 ? sparse_attn_kernel<false, false> : widen ? sparse_attn_kernel<true, true> : sparse_attn_kernel<true, false>;
+  launch(kernel, grid, AttnCfg<false>::kThreads, pl->dev.fp8 ? AttnCfg<true>::kSmemBytes : AttnCfg<false>::kSmemBytes, st, mk,
+         mv, mkb, mkb_lo, mvb, mq, a, pl->dev);
 }
 
 static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, const void* v, const int32_t* pt,
@@ -542,14 +547,18 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   pl->last_launches = 0;
   if (pl->nseg == 0) return FP2_OK;
-  if (need_pool && (s = launch_pool(pl, k, v, pt, lk, ks, vs, ws, st)) != FP2_OK) return s;
-  launch_order(pl, seg_count, reinterpret_cast<int32_t*>(ws + pl->ws_hist), reinterpret_cast<int32_t*>(ws + pl->ws_order),
-               reinterpret_cast<int32_t*>(ws + pl->ws_counter), st);
+  if (need_pool && (s = launch_pool(pl, k, v, pt, ks, vs, ws, st)) != FP2_OK) return s;
+  const bool use_v16 = pl->dev.fp8 && (seg_count ? pl->likely_iters : pl->idx_capacity) >= pl->v16_iters;
+  launch_prepare(pl, seg_count, reinterpret_cast<int32_t*>(ws + pl->ws_hist), reinterpret_cast<int32_t*>(ws + pl->ws_order),
+                 reinterpret_cast<int32_t*>(ws + pl->ws_counter), v, pt,
+                 use_v16 ? reinterpret_cast<__half*>(ws + pl->ws_v16) : nullptr,
+                 reinterpret_cast<int*>(ws + pl->ws_status), st);
   const bool fp8 = pl->dev.fp8 != 0;
   const int64_t slots = (int64_t)pl->prm.num_pages * pl->prm.page_size;
   CUtensorMap mk, mv, mkb, mkb_lo, mvb;
   if (!make_map(pl, &mk, k, slots, pl->prm.num_kv_heads, pl->prm.page_size, fp8) ||
-      !make_map(pl, &mv, v, slots, pl->prm.num_kv_heads, pl->prm.page_size, fp8) ||
+      !(use_v16 ? make_map(pl, &mv, ws + pl->ws_v16, pl->nblk_tot * kBlock, pl->prm.num_kv_heads, kBlock, false)
+                : make_map(pl, &mv, v, slots, pl->prm.num_kv_heads, pl->prm.page_size, fp8)) ||
       !make_map(pl, &mvb, ws + pl->ws_vbar, pl->nblk_tot, pl->prm.num_kv_heads, 128, false))
     return FP2_ERR_CUDA;
   if (fp8) {   // correction chunks: pooled keys as an e4m3 hi + lo pair
@@ -603,7 +612,7 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   }
   CUtensorMap mq = mk;   // unused unless q_box
   if (pl->dev.q_box && !make_q_map(pl, &mq, q, pl->dev.q_box_tok)) return FP2_ERR_CUDA;
-  launch_attn(pl, mk, mv, mkb, mkb_lo, mvb, mq, a, max_units, st);
+  launch_attn(pl, mk, mv, mkb, mkb_lo, mvb, mq, a, max_units, !use_v16, st);
   pl->last_launches += 1;
   if (split) {
     int32_t* seg_split = reinterpret_cast<int32_t*>(ws + pl->ws_seg_split);
@@ -682,7 +691,8 @@ extern "C" fp2_status fp2_dense_prefill_static(fp2_plan* pl, const void* q, cons
   int32_t* order = reinterpret_cast<int32_t*>(sw + kStaticOffOrder);
   // the array keeps the previous call's contents: the status block must start at zero (the sort clears the rest)
   if (cudaMemsetAsync(sw, 0, 64, st) != cudaSuccess) return FP2_ERR_CUDA;
-  launch_order(pl, nullptr, reinterpret_cast<int32_t*>(sw + kStaticOffHist), order, reinterpret_cast<int32_t*>(sw + 64), st);
+  launch_prepare(pl, nullptr, reinterpret_cast<int32_t*>(sw + kStaticOffHist), order, reinterpret_cast<int32_t*>(sw + 64), v,
+                 pt, nullptr, reinterpret_cast<int*>(sw), st);
   const int64_t slots = (int64_t)pl->prm.num_pages * pl->prm.page_size;
   CUtensorMap mk, mv;
   const bool fp8 = pl->dev.fp8 != 0;
@@ -708,7 +718,7 @@ extern "C" fp2_status fp2_dense_prefill_static(fp2_plan* pl, const void* q, cons
 #endif
   CUtensorMap mq = mk;   // unused unless q_box
   if (pl->dev.q_box && !make_q_map(pl, &mq, q, pl->dev.q_box_tok)) return FP2_ERR_CUDA;
-  launch_attn(pl, mk, mv, mk, mk, mv, mq, a, pl->nseg, st);
+  launch_attn(pl, mk, mv, mk, mk, mv, mq, a, pl->nseg, true, st);
   pl->last_launches = 4;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }

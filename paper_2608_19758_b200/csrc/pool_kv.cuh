@@ -276,10 +276,80 @@ __device__ __forceinline__ int order_bucket(int h, int count) {
   return h * kCountBuckets + (kCountBuckets - 1 - c);
 }
 
-// Clears histogram and cursors (2 nb words) and the work counter block (16 words).
-__global__ void order_clear_kernel(int32_t* __restrict__ hist, int nb2, int32_t* __restrict__ counter) {
+// V of FP8 plans as F16 (exact), [nblk_tot * 128, Hkv, 128]: the attention kernel multiplies 16-bit probabilities with it and
+// reads every V tile many times; widened in the kernel, every time, it took the softmax warpgroup ~900 cycles per block.
+// One CTA per 32 tokens of a block, all KV heads (a quarter block: short prompts have few blocks); rows past the end of the
+// sequence are zeros.  Bandwidth-bound: 1 byte read, 2 written per element.  The loads of a batch are unconditional, as in
+// pool_rows_kernel: behind a branch each they went out one at a time (8192 tokens, 4 heads: 27 us, now 8; 245000 tokens, 8 heads: 145 us = 5.2 TB/s).
+constexpr int kWidenTokens = 32;
+__device__ __forceinline__ void widen_v_part(const uint8_t* v_cache, const int32_t* page_table, const int32_t* plan_lk,
+                                             const int32_t* blk_off, const DevParams& P, int part, __half* v16, int* status) {
+  __shared__ int32_t pids[kWidenTokens / 8];   // page ids of the tokens (page size >= 8), -1: nothing to read
+  const int gblk = part / (kBlock / kWidenTokens), tok0 = part % (kBlock / kWidenTokens) * kWidenTokens;
+  int lo = 0, hi = P.num_seqs;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (blk_off[mid] <= gblk) lo = mid; else hi = mid;
+  }
+  const int b = lo, j0 = (gblk - blk_off[b]) * kBlock + tok0;   // first token of the part
+  const int ntok = min(kWidenTokens, plan_lk[b] - j0);
+  const int psz = P.page_size, psz_log2 = 31 - __clz(psz);
+  const int first_page = j0 >> psz_log2;
+  if ((int)threadIdx.x < kWidenTokens / 8) {
+    int pid = -1;
+    const int page = first_page + (int)threadIdx.x;
+    if ((page << psz_log2) < j0 + ntok) {
+      pid = page_table[(size_t)b * P.max_pages_per_seq + page];
+      if (pid < 0 || pid >= P.num_pages) {   // outside the pool: its tokens count as zeros, the call is flagged
+        atomicOr(status + ST_BAD_LIST, 2);
+        pid = -1;
+      }
+    }
+    pids[threadIdx.x] = pid;
+  }
+  __syncthreads();
+  const int C = P.num_kv_heads * 8;            // 16-byte chunks per token row
+  const uint4* src = reinterpret_cast<const uint4*>(v_cache);
+  uint4* dst = reinterpret_cast<uint4*>(v16) + ((size_t)gblk * kBlock + tok0) * C * 2;
+  constexpr int BATCH = 4;
+  const int n = kWidenTokens * C;              // a multiple of 256
+  for (int i0 = threadIdx.x; i0 < n; i0 += BATCH * 256) {
+    uint4 v[BATCH];
+    bool ok[BATCH];
+#pragma unroll
+    for (int u = 0; u < BATCH; ++u) {
+      const int i = min(i0 + u * 256, n - 1), tl = i / C, j = j0 + tl;
+      const int pid = pids[(j >> psz_log2) - first_page];
+      ok[u] = tl < ntok && pid >= 0;
+      const size_t off = ok[u] ? (((size_t)pid << psz_log2) + (j & (psz - 1))) * C + (i - tl * C) : 0;
+      v[u] = __ldg(src + off);
+    }
+#pragma unroll
+    for (int u = 0; u < BATCH; ++u) {
+      const int i = i0 + u * 256;
+      if (i >= n) break;
+      if (!ok[u]) v[u] = make_uint4(0, 0, 0, 0);
+      dst[2 * (size_t)i] = make_uint4(e4m3x2_to_f16x2(v[u].x), e4m3x2_to_f16x2(v[u].x >> 16), e4m3x2_to_f16x2(v[u].y),
+                                      e4m3x2_to_f16x2(v[u].y >> 16));
+      dst[2 * (size_t)i + 1] = make_uint4(e4m3x2_to_f16x2(v[u].z), e4m3x2_to_f16x2(v[u].z >> 16), e4m3x2_to_f16x2(v[u].w),
+                                          e4m3x2_to_f16x2(v[u].w >> 16));
+    }
+  }
+}
+
+// First kernel of an attention call.  The first n_clear CTAs (256 threads) clear histogram and cursors (nb2 words) and the
+// work counter block (16 words); the others, of FP8 plans, widen 32 tokens of V each.
+__global__ void __launch_bounds__(256) attn_prepare_kernel(int32_t* __restrict__ hist, int nb2, int32_t* __restrict__ counter,
+                                                           int n_clear, const uint8_t* v_cache, const int32_t* page_table,
+                                                           const int32_t* __restrict__ plan_lk,
+                                                           const int32_t* __restrict__ blk_off, DevParams P, __half* v16,
+                                                           int* status) {
   pdl_trigger();
   pdl_wait();
+  if ((int)blockIdx.x >= n_clear) {
+    widen_v_part(v_cache, page_table, plan_lk, blk_off, P, (int)blockIdx.x - n_clear, v16, status);
+    return;
+  }
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nb2) hist[i] = 0;
   if (i < 16) counter[i] = 0;

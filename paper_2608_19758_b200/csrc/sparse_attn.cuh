@@ -31,12 +31,15 @@
 // FP8 inputs (Eq. 15; template parameter FP8): S = Q K^T runs as a kind::f8f6f4 MMA straight on the raw e4m3
 // tiles (Q and K both K-major, 128-byte rows, as cp.async / TMA write them), at twice the BF16 rate.  The
 // probabilities stay 16-bit -- a single e4m3 probability tile costs ~0.06 max-abs output error by itself -- so
-// O += P V is a kind::f16 MMA on F16 operands: P packed as F16, V widened (exactly) from its raw e4m3 tile into
-// the F16 V stage by the softmax warpgroup itself at the top of the iteration.  The per-head scales never touch
-// the operands: q_scale * k_scale multiplies the logits of a row, v_scale multiplies the output.  Correction
-// chunks: the pooled keys come as an e4m3 hi + lo pair in raw units (two accumulating MMA groups, ~8 mantissa
-// bits together), the pooled values as F16.  Tile memory: Q 16 KB, K 32 KB (one raw tile, or hi | lo of a
-// chunk), raw V 16 KB, F16 V 32 KB.
+// O += P V is a kind::f16 MMA on F16 operands: P packed as F16, V an F16 copy made for the call in the workspace
+// (attn_prepare_kernel; one contiguous tile per block; map_v is its map).  Short calls and callers without a workspace
+// (template parameter WIDEN) have no such copy: there the softmax warpgroup widens (exactly) the raw e4m3 tile into the F16
+// V stage at the top of the iteration.
+// The per-head scales never touch the operands: q_scale * k_scale multiplies the logits of a row, v_scale multiplies the
+// output.  Correction chunks: the pooled keys come as an e4m3 hi + lo pair in raw units (two accumulating MMA groups, ~8
+// mantissa bits together), the pooled values as F16.  Tile memory: Q 16 KB, K 32 KB (one raw tile, or hi | lo of a
+// chunk), F16 V 32 KB (raw V 16 KB).
+// 16384 tokens dense, 28 heads on 4 KV heads: 1782 us widening per iteration, 1486 us with the copy (its 11 us included).
 #pragma once
 #include <cuda_bf16.h>
 #include "common.cuh"
@@ -197,7 +200,7 @@ __device__ __forceinline__ float row_exp(const uint32_t (&x)[128], uint32_t p_ad
 
 // map_kbar / map_kbar_lo: pooled keys of the correction chunks -- BF16: one BF16 array (map_kbar_lo unused);
 // FP8: the e4m3 hi and lo arrays.  map_vbar: pooled values, 16-bit.  map_q: packed query tiles (DevParams::q_box).
-template <bool FP8>
+template <bool FP8, bool WIDEN>
 __global__ void __launch_bounds__(AttnCfg<FP8>::kThreads, AttnCfg<FP8>::kCtasPerSm)
 sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_kbar, const __grid_constant__ CUtensorMap map_kbar_lo,
@@ -209,7 +212,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
   uint8_t* sQ = smem + kQLeadRows * 128;               // 32 KB (BF16) / 16 KB (raw e4m3) and padding
   uint8_t* sK = smem + AttnCfg<FP8>::kOffK;            // 32 KB
   uint8_t* sV = sK + kTileBytes;                       // 32 KB, 16-bit
-  uint8_t* sVraw = sV + kTileBytes;                    // FP8 only: 16 KB raw e4m3 V tile
+  uint8_t* sVraw = sV + kTileBytes;                    // WIDEN only: 16 KB raw e4m3 V tile
   (void)sVraw;
   // Masks enter the logits through the tensor core: one more k-step S += hot . bias^T (kind::f8f6f4, e5m2 x e5m2,
   // K = 32), which costs 64 cycles of the tensor pipe instead of a TMEM round trip of the softmax warpgroup.
@@ -237,7 +240,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
   __shared__ uint64_t pv_done[2];  // [G & 1], phase (G >> 1) & 1: O += P V (G) has completed -- the V stage is free,
                                    // O holds iteration G.  Two barriers so that a waiter may be two iterations
                                    // behind the issuer without mistaking one phase for another.
-  __shared__ uint64_t vraw_full, vraw_empty;   // FP8: the raw V tile has landed / has been widened
+  __shared__ uint64_t vraw_full, vraw_empty;   // WIDEN: the raw V tile has landed / has been widened
   __shared__ uint64_t p_ready[kPParts];   // slice q (128 / kPParts probabilities of every row) of P (G) is in TMEM
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
@@ -492,17 +495,27 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         if (i < T) {
           const int nvalid = __popc(__ballot_sync(0xffffffffu, pid >= 0));
           if constexpr (FP8) {
-            // raw e4m3 tiles, 128 bytes per token row: K straight into the K stage (the MMA reads it as it
-            // lands), V into the raw slot for the widening warp
+            // raw e4m3 K tile, 128 bytes per token row, straight into the K stage (the MMA reads it as it lands)
             const uint32_t bytes = (uint32_t)nvalid * psz * 128u;
             if (lane == 0) mbar_arrive_expect_tx(&k_full, bytes);
             __syncwarp();
             if (pid >= 0) tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
-            if (rc >= 1) mbar_wait(&vraw_empty, (rc - 1) & 1, ctx, 306);
-            if (lane == 0) mbar_arrive_expect_tx(&vraw_full, bytes);
-            __syncwarp();
-            if (pid >= 0) tma_load_3d_hint(sVraw + lane * psz * 128, &map_v, &vraw_full, 0, sg.h, pid * psz, keep);
-            ++rc;
+            if constexpr (WIDEN) {
+              if (rc >= 1) mbar_wait(&vraw_empty, (rc - 1) & 1, ctx, 306);
+              if (lane == 0) mbar_arrive_expect_tx(&vraw_full, bytes);
+              __syncwarp();
+              if (pid >= 0) tma_load_3d_hint(sVraw + lane * psz * 128, &map_v, &vraw_full, 0, sg.h, pid * psz, keep);
+              ++rc;
+            } else {   // the block's F16 copy is one tile
+              if (G >= 1) wait_pv(G - 1, 304);  // V stage free
+              if (lane == 0) {
+                const int row0 = (sg.blk_off + J_cur) * kBlock;
+                mbar_arrive_expect_tx(&v_full, kTileBytes);
+                tma_load_3d_hint(sV, &map_v, &v_full, 0, sg.h, row0, keep);
+                tma_load_3d_hint(sV + 16384, &map_v, &v_full, 64, sg.h, row0, keep);
+              }
+              __syncwarp();
+            }
           } else {
             const uint32_t bytes = (uint32_t)nvalid * psz * 256u;
             if (lane == 0) mbar_arrive_expect_tx(&k_full, bytes);
@@ -693,7 +706,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             need_mask = true;
           }
         }
-        if constexpr (FP8) {
+        if constexpr (WIDEN) {
           // Exact iteration: widen this iteration's raw e4m3 V tile (exactly) into the F16 V stage before looking
           // at the logits.  128 threads take ~900 cycles (the copy is bound by shared-memory bandwidth next to the
           // other CTA's MMAs); one or two dedicated warps were slower than the time they have, between

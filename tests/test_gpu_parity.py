@@ -601,3 +601,29 @@ def test_work_order_takes_every_segment_once(n_seg_tokens):
     lists = {s.seg: idx[off[s.seg]:off[s.seg] + cnt[s.seg]] for s in wl.segs if cnt[s.seg] > 0}
     check_attention(dc, wl, lists, list(lists))
     assert torch.isfinite(dc.out.float()).all()     # rows without a block come out as zeros
+
+
+@pytest.mark.parametrize("p,hkv,seqs", [
+    (8, 2, [(3000, 0), (130, 2)]),           # ragged last pages, two sequences
+    (128, 2, [(3200, 100)]),                 # whole blocks
+    (32, 3, [(1, 0), (2900, 0), (257, 256)]),  # a head count that no power of two divides, a one-token sequence
+])
+def test_fp8_values_widened_once_per_call(p, hkv, seqs):
+    """FP8 calls with enough iterations (4000 + 7 per block and KV head) read V as an F16 copy in the workspace; shorter ones
+    widen every tile in the kernel.  Both routes against the oracle, sparse and dense, at ragged lengths and the smallest
+    and largest page; and a page id outside the pool is still flagged on the copying route."""
+    spec = inputs.small_spec(seqs=seqs, num_q_heads=8 * hkv, num_kv_heads=hkv, page_size=p, dtype="fp8",
+                             config_id=160 + p)
+    spec.alpha = 0.05
+    case, dc, wl = full_pipeline(spec)
+    assert dc.plan.idx_capacity >= 4000 + 7 * hkv * sum(-(-lk // 128) for lk, _ in seqs)
+    small = inputs.small_spec(seqs=[(400, 0)], num_q_heads=8 * hkv, num_kv_heads=hkv, page_size=p, dtype="fp8", config_id=170)
+    small.alpha = 0.05
+    _, dcs, _ = full_pipeline(small)
+    assert dcs.plan.idx_capacity < 4000
+    good = dc.page_table.clone()
+    dc.page_table[len(seqs) - 1, 0] = dc.prm["num_pages"] + 3
+    dc.dense()
+    code, words = dc.status(raise_on_error=False)
+    assert code == 1 and words[2] & 2
+    dc.page_table.copy_(good)
