@@ -603,6 +603,32 @@ def test_work_order_takes_every_segment_once(n_seg_tokens):
     assert torch.isfinite(dc.out.float()).all()     # rows without a block come out as zeros
 
 
+@pytest.mark.parametrize("hkv", [1, 3])
+def test_work_order_with_a_few_long_segments(hkv):
+    """More segments than workers times eight, so that only some count as long and go first: lists of 0 to 2 blocks (the limit
+    lies between 1 and 2), every 13th with 3, every 101st complete.  A segment dropped by either part of the order would
+    leave its rows at the poison value."""
+    spec = inputs.small_spec(seqs=[(3300 if hkv == 3 else 9900, 0)], num_q_heads=32 * hkv, num_kv_heads=hkv, page_size=128,
+                             config_id=152 + hkv)
+    case, dc, wl = make(spec, use_correction=0)
+    dc.select()
+    dc.status()
+    off = dc.seg_offset.cpu().numpy()
+    cnt = np.zeros(dc.plan.num_segments, dtype=np.int32)
+    idx = dc.blk_idx.cpu().numpy().copy()
+    for s in wl.segs:
+        n = s.J_hi + 1 if s.seg % 101 == 0 else min(3 if s.seg % 13 == 0 else s.seg % 3, s.J_hi + 1)
+        cnt[s.seg] = n
+        idx[off[s.seg]:off[s.seg] + n] = np.arange(s.J_hi + 1 - n, s.J_hi + 1)
+    workers = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert 1.0 < cnt.sum() / (8 * workers) < 2.0
+    dc.sparse(seg_count=torch.from_numpy(cnt).cuda(), blk_idx=torch.from_numpy(idx).cuda())
+    dc.status()
+    some = [s.seg for s in wl.segs if cnt[s.seg] > 0 and (s.seg % 101 == 0 or s.seg % 97 == 0)]
+    check_attention(dc, wl, {s: idx[off[s]:off[s] + cnt[s]] for s in some}, some)
+    assert torch.isfinite(dc.out.float()).all()
+
+
 @pytest.mark.parametrize("p,hkv,seqs", [
     (8, 2, [(3000, 0), (130, 2)]),           # ragged last pages, two sequences
     (128, 2, [(3200, 100)]),                 # whole blocks
