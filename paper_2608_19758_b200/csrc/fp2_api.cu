@@ -162,8 +162,15 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
 
   // Scorer work units (score_pair_kernel): adjacent tiles (t-1, t) of one (sequence, KV head) share their candidate
   // blocks, so they are scored together when the later one has at most kPairMaxCand candidates; heaviest first
-  // (descending segment index, like the single-tile scorer's order).
+  // (descending segment index, like the single-tile scorer's order).  Where every tile has an SM to itself a pair would only
+  // lengthen the chain of its CTA: 768 tokens FP8, 48 tiles, select + sparse
+  // 38.0 us in pairs, 35.6 one by one.
   std::vector<int2> units;
+  int cur_dev = -1, sms = 0;
+  if (cudaGetDevice(&cur_dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cur_dev) != cudaSuccess)
+    (void)cudaGetLastError();
+  const bool pair = pl->nseg > sms;
   {
     int64_t tile_off2 = 0;
     std::vector<int64_t> toff((size_t)p->num_seqs), ntiles((size_t)p->num_seqs);
@@ -177,7 +184,7 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
       for (int h = p->num_kv_heads - 1; h >= 0; --h) {
         const int64_t base = p->num_kv_heads * toff[(size_t)b] + (int64_t)h * ntiles[(size_t)b];
         for (int64_t t = ntiles[(size_t)b] - 1; t >= 0;) {
-          if (t >= 1 && segs[(size_t)(base + t)].J_hi + 1 <= kPairMaxCand) {
+          if (pair && t >= 1 && segs[(size_t)(base + t)].J_hi + 1 <= kPairMaxCand) {
             units.push_back(make_int2((int)(base + t - 1), (int)(base + t)));
             t -= 2;
           } else {
@@ -378,7 +385,9 @@ static bool make_q_map(fp2_plan* pl, CUtensorMap* m, const void* q, int box_toke
 
 static fp2_status set_attrs(fp2_plan* pl) {
   if (pl->attrs_set) return FP2_OK;
-  if (cudaFuncSetAttribute(score_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) !=
+  if (cudaFuncSetAttribute(score_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) !=
+          cudaSuccess ||
+      cudaFuncSetAttribute(score_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) !=
           cudaSuccess ||
       cudaFuncSetAttribute(score_select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kScoreSmemBytes) != cudaSuccess ||
@@ -478,23 +487,20 @@ extern "C" fp2_status fp2_select_blocks(fp2_plan* pl, const void* q, const void*
     return FP2_ERR_CUDA;
   CUtensorMap mq = mhi;   // unused unless the scorer takes its query tiles by TMA
   CUtensorMap mq2 = mhi;
-  if (pl->dev.fp8 ? (pl->dev.q_raw_tma && !make_q_map(pl, &mq, q, pl->dev.q_box_tok))
-                  : (pl->dev.q_box && (!make_q_map(pl, &mq, q, pl->dev.q_box_tok) || !make_q_map(pl, &mq2, q, pl->dev.q_box2_tok))))
+  if (((pl->dev.q_box || pl->dev.q_raw_tma) && !make_q_map(pl, &mq, q, pl->dev.q_box_tok)) ||
+      (pl->dev.q_box && !make_q_map(pl, &mq2, q, pl->dev.q_box2_tok)))
     return FP2_ERR_CUDA;
   int* status = reinterpret_cast<int*>(ws + pl->ws_status);
-  const unsigned grid = (unsigned)(pl->nseg < pl->num_sms ? pl->nseg : pl->num_sms);
-  if (pl->dev.fp8)
-    launch(score_select_kernel<true>, grid, kScoreThreads, kScoreSmemBytes, st, mhi, mlo, mq, (const uint8_t*)q,
-           pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
-  else if (pl->dev.q_box) {
-    // BF16 tiles that come as TMA boxes: pairs of adjacent tiles per pooled-key chunk.  The pair kernel takes the pooled
-    // keys in pieces of 64 elements x 128 keys, which is the box of mhi / mlo already.
-    const unsigned grid_pairs = (unsigned)(pl->nunits < pl->num_sms ? pl->nunits : pl->num_sms);
-    launch(score_pair_kernel, grid_pairs, kPairThreads, kPairSmemBytes, st, mhi, mlo, mq, mq2, pl->d_segs, pl->d_units, pl->nunits,
-                                                                        pl->dev, seg_offset, seg_count, blk_idx, status);
-  } else
-    launch(score_select_kernel<false>, grid, kScoreThreads, kScoreSmemBytes, st, mhi, mlo, mq, (const uint8_t*)q,
-           pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
+  if (pl->dev.q_box) {
+    // pairs of adjacent tiles per pooled-key chunk, in pieces of 64 elements x 128 keys (the box of mhi / mlo)
+    launch(pl->dev.fp8 ? score_pair_kernel<true> : score_pair_kernel<false>,
+           (unsigned)(pl->nunits < pl->num_sms ? pl->nunits : pl->num_sms), kPairThreads, kPairSmemBytes, st, mhi, mlo, mq, mq2,
+           pl->d_segs, pl->d_units, pl->nunits, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
+  } else {
+    launch(pl->dev.fp8 ? score_select_kernel<true> : score_select_kernel<false>,
+           (unsigned)(pl->nseg < pl->num_sms ? pl->nseg : pl->num_sms), kScoreThreads, kScoreSmemBytes, st, mhi, mlo, mq,
+           (const uint8_t*)q, pl->d_segs, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
+  }
   pl->last_launches += 1;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }

@@ -67,9 +67,9 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 // Waits until the phase with the given parity has completed.  Bounded: on expiry the status
-// block records the site and the CTA-wide abort flag makes all later waits fall through.
-__device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtx& ctx, int where) {
-  if (mbar_try_wait(bar, parity)) return;
+// block records the site and the CTA-wide abort flag makes all later waits fall through.  False: the phase has not completed.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtx& ctx, int where) {
+  if (mbar_try_wait(bar, parity)) return true;
   long long t0 = clock64();
   int spins = 0;
   while (!mbar_try_wait(bar, parity)) {
@@ -77,15 +77,16 @@ __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, const 
       if (*ctx.abort) {
         // words 3..7: the wait each role (2xx .. 6xx) of an aborted CTA was found in (last writer wins)
         if (where >= 200 && where < 700) ctx.status[3 + (where / 100 - 2)] = where;
-        return;
+        return false;
       }
       if (clock64() - t0 > ctx.budget) {
         *ctx.abort = 1;
         if (atomicCAS(ctx.status + ST_TIMEOUT, 0, 1) == 0) ctx.status[ST_WHERE] = where;
-        return;
+        return false;
       }
     }
   }
+  return true;
 }
 // After an abort: waits (bounded by `cycles`, whatever the abort flag says) until the barrier's phase has completed.
 // Used on the way out of a kernel to let work in flight finish before its resources are released.
@@ -263,6 +264,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
+}
+// tcgen05.wait::ld that the loaded registers depend on: with other work between load and wait nothing else keeps the
+// compiler from using them too early.
+__device__ __forceinline__ void tmem_wait_ld32(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),
+                 "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
+                 "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])::"memory");
 }
 // registers -> TMEM: 32 lanes x 8 consecutive 32-bit columns.
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {

@@ -1,5 +1,5 @@
-// Fused block scoring and selection (Eq. 19, Eq. 20; Algorithm 1 lines 3-5) for BF16 plans whose packed query tiles
-// come as TMA boxes (DevParams::q_box): score_select_kernel with TWO adjacent query tiles of a KV head per unit.
+// Fused block scoring and selection (Eq. 19, Eq. 20; Algorithm 1 lines 3-5) for plans whose packed query tiles come
+// as TMA boxes (DevParams::q_box): score_select_kernel with TWO adjacent query tiles of a KV head per unit.
 //
 // At long sequences score_select_kernel is bound by the traffic of the pooled keys from L2 into shared memory: every
 // chunk of 128 pooled keys (hi + lo: 64 KB) is fetched once per query tile, 35 bytes per cycle and SM at 131072
@@ -10,15 +10,27 @@
 //
 // Units (built by the planner, heaviest first): a pair of tiles (t-1, t) of one (sequence, KV head) when the later
 // tile has at most 1024 candidate blocks, else a single tile.  CTA b takes units b, b + grid, b + 2 grid, ...
-// Everything else is as in score_select_kernel: the contraction runs transposed, kbar enters as a BF16 (hi, lo) pair
-// accumulated into one fp32 accumulator, two consumer warpgroups alternate over the chunks (two TMEM accumulators
-// of 256 columns) and each takes, per pooled key, maximum and exponential sum over the rows of the first tile and
-// then of the second, log2 energies go to shared memory, and a selection warp applies threshold and forced sets and
-// writes the ordered lists of unit u beside the scoring of unit u+1.
+// As in score_select_kernel the contraction runs transposed and kbar enters as a 16-bit (hi, lo) pair accumulated into one fp32
+// accumulator; per pooled key a consumer thread takes maximum and exponential sum over a tile's rows, log2 energies go to
+// shared memory, and a selection warp applies threshold and forced sets and writes the ordered lists of unit u beside the
+// scoring of unit u+1.
 //
-// Roles: warps 0-3 / 4-7 consumer warpgroups; warp 8 TMA producer of kbar pieces (16 KB: 128 keys x 64 elements, four
-// per chunk: hi | lo x the two halves of d); warp 9 UMMA issuer and TMEM owner; warp 10 unit set-up and query tiles by
-// TMA (two units in flight); warp 11 selection.
+// What bounds it: per chunk of a pair the tensor pipe needs 2048 cycles and the exponentials 2048 of the MUFU pipe; measured
+// about 2700 at the clocks that the power limit leaves at 131072 tokens (without the exponentials 7 % less, without the MMAs
+// the same).  The items (chunk, tile) are dealt to THREE consumer warpgroups, so that one loads or waits while the others
+// exponentiate, and an item goes through in batches (see score_cols), which is what lets three of them fit into the registers.
+// Index stage, two warpgroups with a tile each and 128 columns in one piece / so: 131072 tokens 1099 / 1065 us, 65536 tokens
+// 376 / 365, 32768 tokens 150 / 141, 16 sequences of 245000 tokens 681 / 650, 24 short ones 48.5 / 45.3.  FP8 plans took one
+// tile per chunk in score_select_kernel before: 131072 tokens, 28 heads on 4, 1216 / 1012, 16 sequences 874 / 720, 8191 tokens
+// 53.3 / 48.6.
+//
+// FP8: the raw e4m3 box lands in the second half of a query buffer, where its 128-byte rows are as many as the F16 rows of a
+// half, and the set-up warp widens it in place: elements 0..63 of a row go to the first half, 64..127 over the raw row.  Every
+// row has a multiplier of its own (q_scale), kept per unit in sC.
+//
+// Roles: warps 0-11 consumers; warp 12 TMA producer of kbar pieces (16 KB: 128 keys x 64 elements, four per chunk: hi | lo x
+// the two halves of d); warp 13 UMMA issuer and TMEM owner; warp 14 unit set-up and query tiles by TMA (two units in flight);
+// warp 15 selection.
 // Shared memory: 2 x 64 KB query pairs (and 5 KB of padding each) + 4 x 16 KB pieces + 16 KB energies.  TMEM: 2 x 256
 // columns.
 //
@@ -30,7 +42,9 @@
 
 namespace fp2 {
 
-constexpr int kPairThreads = 384;
+constexpr int kPairGroups = 3;           // consumer warpgroups
+constexpr int kPairConsumers = kPairGroups * 128;
+constexpr int kPairThreads = kPairConsumers + 128;
 constexpr int kPairInfoSlots = 4;        // unit descriptors in flight
 constexpr int kPairQBufs = 2;            // 64 KB query-pair buffers
 constexpr int kPairPieces = 4;           // ring of 16 KB kbar pieces
@@ -48,54 +62,112 @@ struct PairInfo {
 };
 
 // One pooled key (= this thread's TMEM lane) against the 128 query rows of one tile (= 128 TMEM columns at
-// lane_addr): m = max_j x_j, sum = sum_j 2^(x_j - m), x_j = s_j * cs.  PARTIAL: only the first nrows columns are real
-// query rows.  With `release` the accumulator is handed back as soon as it is in registers.
-template <bool PARTIAL>
-__device__ __forceinline__ void score_cols(uint32_t lane_addr, float cs, int nrows, uint64_t* release, float& m_out,
-                                           float& sum_out) {
-  uint32_t xv[128];
+// lane_addr): returns log2 sum_j 2^x_j, x_j = s_j * cs (FP8: s_j * sC[j]).  PARTIAL: only the first nrows columns are real
+// query rows.  The columns go through in batches of W.  The reference of the exponentials is the maximum of the first 16
+// columns instead of all 128 (no need to hold 128 logits, an eighth of the maxima): the sum is then at least 1, so nothing
+// that matters underflows, and a batch after which it comes near the top of fp32 is done again with its own maximum.  The
+// accumulator is handed back once the last batch is in registers.
+template <bool FP8, bool PARTIAL>
+__device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const float* sC, int nrows, uint64_t* release) {
+  constexpr int W = FP8 ? 32 : 64;   // the multipliers take registers too: FP8 with 64 spills (131072 tokens 1010 -> 1590 us)
+  constexpr int kFirst = 16;
+  float m = -INFINITY, total = 0.f;
+  uint64_t s4[4] = {0ull, 0ull, 0ull, 0ull};   // sums of 2^(x_j - m), four independent (lo, hi) accumulators
 #pragma unroll
-  for (int k = 0; k < 4; ++k) tmem_ld32(lane_addr + k * 32, reinterpret_cast<uint32_t(&)[32]>(xv[k * 32]));
-  tmem_wait_ld();
-  if (release != nullptr) {
-    tc_fence_before();
-    mbar_arrive(release);
-  }
-  float x[128];
+  for (int j0 = 0; j0 < kTileRows; j0 += W) {
+    uint32_t xv[W];
 #pragma unroll
-  for (int j = 0; j < 128; ++j) {
-    x[j] = __uint_as_float(xv[j]);
-    if constexpr (PARTIAL) x[j] = (j < nrows) ? x[j] : -INFINITY;
-  }
-  float m8[8];
+    for (int k = 0; k < W; k += 32) tmem_ld32(lane_addr + j0 + k, reinterpret_cast<uint32_t(&)[32]>(xv[k]));
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const float* v = &x[c * 16];
-    m8[c] = max3(max3(max3(v[0], v[1], v[2]), max3(v[3], v[4], v[5]), max3(v[6], v[7], v[8])),
-                 max3(v[9], v[10], v[11]), max3(max3(v[12], v[13], v[14]), v[15], v[15]));
-  }
-  // the multiplier is positive: the maximum is taken over the raw logits and the scaling rides in the fused
-  // multiply-add that subtracts it
-  float m = fmaxf(max3(m8[0], m8[1], m8[2]), max3(max3(m8[3], m8[4], m8[5]), m8[6], m8[7])) * cs;
-  const uint64_t nm2 = f2_pack(-m, -m), mul2 = f2_pack(cs, cs);
-  uint64_t s4[4] = {0ull, 0ull, 0ull, 0ull};
+    for (int k = 0; k < W; k += 32) tmem_wait_ld32(reinterpret_cast<uint32_t(&)[32]>(xv[k]));
+    if (j0 + W == kTileRows) {
+      tc_fence_before();
+      mbar_arrive(release);
+    }
+    auto mult2 = [&](int j) { return FP8 ? *reinterpret_cast<const uint64_t*>(sC + j0 + j) : f2_pack(cs, cs); };
+    auto batch_max = [&](int n) {   // of the first n scaled logits
+      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-  for (int j = 0; j < 128; j += 2) {
-    float d0, d1;
-    f2_unpack(f2_fma(f2_pack(x[j], x[j + 1]), mul2, nm2), d0, d1);
-    s4[(j >> 1) & 3] = f2_add(s4[(j >> 1) & 3], f2_pack(ex2(d0), ex2(d1)));
+      for (int j = 0; j < n; j += 2) {
+        float a, c;
+        if constexpr (FP8) {
+          f2_unpack(f2_mul(f2_pack(__uint_as_float(xv[j]), __uint_as_float(xv[j + 1])), mult2(j)), a, c);
+        } else {   // the multiplier is positive: it commutes with the maximum
+          a = __uint_as_float(xv[j]);
+          c = __uint_as_float(xv[j + 1]);
+        }
+        if constexpr (PARTIAL) {
+          a = j0 + j < nrows ? a : -INFINITY;
+          c = j0 + j + 1 < nrows ? c : -INFINITY;
+        }
+        mx[(j >> 1) & 3] = max3(mx[(j >> 1) & 3], a, c);
+      }
+      const float r = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]);
+      return FP8 ? r : r * cs;
+    };
+    auto add_batch = [&]() {
+      const uint64_t nm2 = f2_pack(-m, -m);
+#pragma unroll
+      for (int j = 0; j < W; j += 2) {
+        float d0, d1;
+        f2_unpack(f2_fma(f2_pack(__uint_as_float(xv[j]), __uint_as_float(xv[j + 1])), mult2(j), nm2), d0, d1);
+        if constexpr (PARTIAL) {
+          d0 = j0 + j < nrows ? d0 : -INFINITY;
+          d1 = j0 + j + 1 < nrows ? d1 : -INFINITY;
+        }
+        s4[(j >> 1) & 3] = f2_add(s4[(j >> 1) & 3], f2_pack(ex2(d0), ex2(d1)));
+      }
+      float t0, t1;
+      f2_unpack(f2_add(f2_add(s4[0], s4[1]), f2_add(s4[2], s4[3])), t0, t1);
+      return t0 + t1;
+    };
+    if (j0 == 0) m = batch_max(kFirst);
+    float sum = add_batch();
+    if (__any_sync(0xffffffffu, sum > 1e36f)) {   // (as one warp: the TMEM accesses are warp-wide)
+      const float m_new = fmaxf(m, batch_max(W));
+      s4[0] = f2_pack(total * ex2(m - m_new), 0.f);   // (total = 0 in the first batch, m is finite)
+      s4[1] = s4[2] = s4[3] = 0ull;
+      m = m_new;
+      sum = add_batch();
+    }
+    total = sum;
   }
-  float t0, t1;
-  f2_unpack(f2_add(f2_add(s4[0], s4[1]), f2_add(s4[2], s4[3])), t0, t1);
-  m_out = m;
-  sum_out = t0 + t1;
+  return m + log2f(total);
 }
 
+// Raw e4m3 rows in the second half of a query buffer -> F16 rows in both halves, in place; one warp, `rows` a multiple of 32.
+// Eight lanes take a row; the rows of a batch are in registers before the first of them is overwritten.
+__device__ __forceinline__ void widen_pair_in_place(uint8_t* half0, uint8_t* half1, int rows, int lane) {
+  for (int i0 = lane; i0 < rows * 8; i0 += 256) {
+    uint4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * 32;
+      v[u] = *reinterpret_cast<const uint4*>(half1 + sw128_offset(i >> 3, i & 7));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * 32, row = i >> 3, c = i & 7;
+      uint8_t* half = c < 4 ? half0 : half1;
+      *reinterpret_cast<uint4*>(half + sw128_offset(row, (c & 3) * 2)) =
+          make_uint4(e4m3x2_to_f16x2(v[u].x), e4m3x2_to_f16x2(v[u].x >> 16), e4m3x2_to_f16x2(v[u].y),
+                     e4m3x2_to_f16x2(v[u].y >> 16));
+      *reinterpret_cast<uint4*>(half + sw128_offset(row, (c & 3) * 2 + 1)) =
+          make_uint4(e4m3x2_to_f16x2(v[u].z), e4m3x2_to_f16x2(v[u].z >> 16), e4m3x2_to_f16x2(v[u].w),
+                     e4m3x2_to_f16x2(v[u].w >> 16));
+    }
+    __syncwarp();
+  }
+}
+
+template <bool FP8>
 __global__ void __launch_bounds__(kPairThreads, 1)
 score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_constant__ CUtensorMap map_klo,
                   const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_q2,
-                  const SegInfo* __restrict__ segs, const int2* __restrict__ units, int nunits, DevParams P, int64_t* __restrict__ seg_offset,
-                  int32_t* __restrict__ seg_count, int32_t* __restrict__ blk_idx, int* __restrict__ status) {
+                  const SegInfo* __restrict__ segs, const int2* __restrict__ units, int nunits, const float* q_scale,
+                  DevParams P, int64_t* __restrict__ seg_offset, int32_t* __restrict__ seg_count,
+                  int32_t* __restrict__ blk_idx, int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // query pair buffer: [half of d][tile][128 rows x 128 bytes] -- the two tiles of a half are 256 consecutive packed rows,
@@ -106,13 +178,16 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
                                                                                 // second tile of a pair 1024 further
 
   __shared__ PairInfo info[kPairInfoSlots];
+  __shared__ __align__(8) float sC[FP8 ? kPairInfoSlots : 1][FP8 ? 2 * kTileRows : 2];   // per-row multipliers of the unit; rewritten
+                                                                            // once the consumers have released the descriptor
   __shared__ uint64_t info_full[kPairInfoSlots], info_empty[kPairInfoSlots], q_full[kPairQBufs], q_empty[kPairQBufs];
+  __shared__ uint64_t raw_full[kPairQBufs];
   __shared__ uint64_t full[kPairPieces], empty[kPairPieces], acc_full[2], acc_empty[2];
   __shared__ uint64_t e_full[2], sel_done[2];   // [unit & 1] energies of the unit are complete / its lists are written
   __shared__ uint64_t drain_bar;
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
-  __shared__ float red[2][2][8];                // [unit & 1][tile][consumer warp] maxima of the log2 energies
+  __shared__ float red[2][2][4 * kPairGroups];                // [unit & 1][tile][consumer warp] maxima of the log2 energies
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   WaitCtx ctx{status, &abort_flag};
@@ -121,17 +196,18 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     abort_flag = 0;
     for (int i = 0; i < kPairInfoSlots; ++i) {
       mbar_init(&info_full[i], 1);
-      mbar_init(&info_empty[i], 2 + 256 + 1);   // producer, issuer, consumers, selection warp
+      mbar_init(&info_empty[i], 2 + kPairConsumers + 1);   // producer, issuer, consumers, selection warp
     }
     for (int i = 0; i < kPairQBufs; ++i) {
       mbar_init(&q_full[i], 1);
       mbar_init(&q_empty[i], 1);
+      mbar_init(&raw_full[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&e_full[i], 256);
+      mbar_init(&e_full[i], kPairConsumers);
       mbar_init(&sel_done[i], 1);
       mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_empty[i], 256);
+      mbar_init(&acc_empty[i], kPairConsumers);
     }
     for (int i = 0; i < kPairPieces; ++i) {
       mbar_init(&full[i], 1);
@@ -140,7 +216,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     mbar_init(&drain_bar, 1);
     fence_barrier_init();
   }
-  if (warp == 9) {
+  if (warp == 4 * kPairGroups + 1) {
     tmem_alloc(&tmem_base_s, 512);
     tmem_relinquish();
   }
@@ -153,10 +229,10 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
   // chunks of a unit: those of its last tile (the later tile of a pair has the larger candidate range)
   auto unit_chunks = [](const PairInfo& pi) { return (pi.sg[pi.nt - 1].J_hi + 128) >> 7; };
 
-  if (warp == 10) {
+  if (warp == 4 * kPairGroups + 2) {
     // ---------------- set-up: unit k of this CTA is number blockIdx.x + k * gridDim.x of the planner's table
     // (heaviest first; a static round-robin, no atomic on the critical path).  Query tiles by TMA, one box per 64-element
-    // half (see kQLeadRows); rows of a short last tile get whatever follows and are not used.
+    // half (FP8: one, see kQLeadRows); rows of a short last tile get whatever follows and are not used.
     const uint64_t pol = l2_policy_evict_first();
     for (int k = 0;; ++k) {
       const int slot = k % kPairInfoSlots, qb = k % kPairQBufs;
@@ -179,20 +255,33 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       __syncwarp();
       if (!valid) break;
       if (k >= kPairQBufs) mbar_wait(&q_empty[qb], ((k / kPairQBufs) - 1) & 1, ctx, 112);
-      if (lane == 0) {
-        const PairInfo& pi = info[slot];
-        const SegInfo& sg = pi.sg[0];
-        const int tok0 = sg.r0 / P.group, lead = sg.r0 - tok0 * P.group;
-        uint8_t* dst = sQ + qb * kPairQBytes - lead * 128;
-        const CUtensorMap* mp = pi.nt > 1 ? &map_q2 : &map_q;
-        const uint32_t rows = (uint32_t)(P.group * (pi.nt > 1 ? P.q_box2_tok : P.q_box_tok));
+      const PairInfo& pi = info[slot];
+      const SegInfo& sg = pi.sg[0];
+      const int tok0 = sg.r0 / P.group, lead = sg.r0 - tok0 * P.group, nt = pi.nt;
+      uint8_t* buf = sQ + qb * kPairQBytes;
+      const CUtensorMap* mp = nt > 1 ? &map_q2 : &map_q;
+      const uint32_t rows = (uint32_t)(P.group * (nt > 1 ? P.q_box2_tok : P.q_box_tok));
+      if constexpr (FP8) {
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&raw_full[qb], rows * 128u);
+          tma_load_3d_hint(buf + kPairQHalf - lead * 128, mp, &raw_full[qb], 0, sg.h * P.group, sg.q_tok0 + tok0, pol);
+        }
+        for (int j = lane; j < nt * kTileRows; j += 32)   // (adjacent tiles: row j of the pair is packed row r0 + j)
+          sC[slot][j] = P.scale_log2 * q_scale[sg.h * P.group + (sg.r0 + j) % P.group];
+        __syncwarp();
+        mbar_wait(&raw_full[qb], (k / kPairQBufs) & 1, ctx, 114);
+        widen_pair_in_place(buf, buf + kPairQHalf, nt * kTileRows, lane);
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&q_full[qb]);
+      } else if (lane == 0) {
         mbar_arrive_expect_tx(&q_full[qb], rows * 256u);
-        tma_load_3d_hint(dst, mp, &q_full[qb], 0, sg.h * P.group, sg.q_tok0 + tok0, pol);
-        tma_load_3d_hint(dst + kPairQHalf, mp, &q_full[qb], 64, sg.h * P.group, sg.q_tok0 + tok0, pol);
+        tma_load_3d_hint(buf - lead * 128, mp, &q_full[qb], 0, sg.h * P.group, sg.q_tok0 + tok0, pol);
+        tma_load_3d_hint(buf + kPairQHalf - lead * 128, mp, &q_full[qb], 64, sg.h * P.group, sg.q_tok0 + tok0, pol);
       }
       __syncwarp();
     }
-  } else if (warp == 11) {
+  } else if (warp == 4 * kPairGroups + 3) {
     // ---------------- selection: threshold, forced blocks, ordered compaction of the tiles of unit `it` ----------------
     for (int it = 0;; ++it) {
       const int slot = it % kPairInfoSlots, eb = it & 1;
@@ -206,7 +295,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
         const float* e = sE + (ncand > kMaxBlocks / 2 ? 0 : eb * (kMaxBlocks / 2) + tt * kPairMaxCand);
         float maxE = red[eb][tt][0];
 #pragma unroll
-        for (int i = 1; i < 8; ++i) maxE = fmaxf(maxE, red[eb][tt][i]);
+        for (int i = 1; i < 4 * kPairGroups; ++i) maxE = fmaxf(maxE, red[eb][tt][i]);
         // J selected  <=>  E_J >= alpha max E  <=>  e_J >= log2(alpha) + max e   (alpha <= 0 selects everything)
         const float thr = P.alpha > 0.f ? maxE + log2f(P.alpha) : -INFINITY;
         const int win_lo = sg.J_lo - P.window_blocks;
@@ -231,37 +320,41 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
         mbar_arrive(&info_empty[slot]);
       }
     }
-  } else if (warp == 8) {
+  } else if (warp == 4 * kPairGroups) {
     // ---------------- producer: kbar pieces of every 128-block chunk (hi then lo, each in its two halves of d) ----------------
     if (lane == 0) {
       tma_prefetch_desc(&map_khi);
       tma_prefetch_desc(&map_klo);
       const uint64_t keep = l2_policy_evict_last();
       uint32_t pc = 0;
-      for (int it = 0;; ++it) {
-        const int slot = it % kPairInfoSlots;
-        mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 121);
-        const PairInfo& pi = info[slot];
-        if (!pi.valid) break;
-        const int h = pi.sg[0].h, blk_off = pi.sg[0].blk_off;
-        const int nchunks = unit_chunks(pi);
-        for (int c = 0; c < nchunks; ++c) {
-#pragma unroll
-          for (int p = 0; p < 4; ++p, ++pc) {
-            const int s = pc % kPairPieces;
-            if (pc >= kPairPieces) mbar_wait(&empty[s], ((pc / kPairPieces) - 1) & 1, ctx, 122);
-            mbar_arrive_expect_tx(&full[s], kPairPieceBytes);
-            tma_load_3d_hint(sStage + s * kPairPieceBytes, p < 2 ? &map_khi : &map_klo, &full[s], (p & 1) * 64, h,
-                             blk_off + c * 128, keep);
+      auto produce = [&]() {
+        for (int it = 0;; ++it) {
+          const int slot = it % kPairInfoSlots;
+          mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 121);
+          const PairInfo& pi = info[slot];
+          if (!pi.valid) break;
+          const int h = pi.sg[0].h, blk_off = pi.sg[0].blk_off;
+          const int nchunks = unit_chunks(pi);
+          for (int c = 0; c < nchunks; ++c) {
+  #pragma unroll
+            for (int p = 0; p < 4; ++p, ++pc) {
+              const int s = pc % kPairPieces;
+              if (pc >= kPairPieces && !mbar_wait(&empty[s], ((pc / kPairPieces) - 1) & 1, ctx, 122)) return;   // nothing more after an abort
+              mbar_arrive_expect_tx(&full[s], kPairPieceBytes);
+              tma_load_3d_hint(sStage + s * kPairPieceBytes, p < 2 ? &map_khi : &map_klo, &full[s], (p & 1) * 64, h,
+                               blk_off + c * 128, keep);
+            }
           }
+          mbar_arrive(&info_empty[slot]);
         }
-        mbar_arrive(&info_empty[slot]);
-      }
+      };
+      produce();
     }
-  } else if (warp == 9) {
+  } else if (warp == 4 * kPairGroups + 1) {
     // ---------------- UMMA issuer: acc[chunk & 1] = kbar_hi Q^T + kbar_lo Q^T over the unit's one or two tiles ----------------
     // the whole warp walks the loop, one elected lane issues (see the attention kernel's issuer)
     const bool leader = elect_one();
+    constexpr int kFmt = FP8 ? 0 : 1;             // F16 / BF16 operands
     uint32_t pc = 0, ac0 = 0, ac1 = 0, gc0 = 0;   // gc0: chunks of all earlier units
     for (int it = 0;; ++it) {
       const int slot = it % kPairInfoSlots, qb = it % kPairQBufs;
@@ -269,7 +362,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       const PairInfo& pi = info[slot];
       if (!pi.valid) break;
       const int nchunks = unit_chunks(pi);
-      const uint32_t idesc = make_idesc(128, 128 * pi.nt, 1, 1, 0, 0);
+      const uint32_t idesc = make_idesc(128, 128 * pi.nt, kFmt, kFmt, 0, 0);
       mbar_wait(&q_full[qb], (it / kPairQBufs) & 1, ctx, 132);
       const uint64_t q_desc = make_smem_desc_sw128(smem_u32(sQ + qb * kPairQBytes), 16, 1024);
       for (int c = 0; c < nchunks; ++c) {
@@ -280,10 +373,10 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
 #pragma unroll
         for (int p = 0; p < 4; ++p, ++pc) {
           const int s = pc % kPairPieces;
-          mbar_wait(&full[s], (pc / kPairPieces) & 1, ctx, 134);
+          const bool ready = mbar_wait(&full[s], (pc / kPairPieces) & 1, ctx, 134);
           tc_fence_after();
           const uint64_t a_desc = make_smem_desc_sw128(smem_u32(sStage + s * kPairPieceBytes), 16, 1024);
-          if (leader) {
+          if (leader && ready) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
               umma_f16_ss(tmem + a * 256, a_desc + ks * 2, q_desc + ((p & 1) * (kPairQHalf >> 4) + ks * 2), idesc, (p | ks) != 0);
@@ -305,8 +398,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     const int key = (warp & 3) * 32 + lane;  // TMEM lane = pooled key within the chunk
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float cs = P.scale_log2;
-    uint32_t uc0 = 0, uc1 = 0;   // uses of the two accumulators
     uint32_t gc0 = 0;  // chunks of all earlier units
+    int turn = 0;      // warpgroup whose turn the next item (chunk, tile) is
     bool prev_big = false;
     for (int it = 0;; ++it) {
       const int slot = it % kPairInfoSlots;
@@ -319,7 +412,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       const int nrows0 = pi.sg[0].nrows, nrows1 = nt > 1 ? pi.sg[1].nrows : 0;
       // per candidate: log2 of its energy, e_J = m_J + log2(S_J)  (Eq. 1-2 / Eq. 20 in the log domain: the common
       // factor 2^-M of Eq. 20 cancels in the comparison with alpha * max)
-      float lmax0 = -INFINITY;
+      float lmax0 = -INFINITY, lmax1 = -INFINITY;
       const int eb = it & 1;
       const bool big = ncand0 > kMaxBlocks / 2;    // a single tile that takes the whole energy buffer
       float* e0 = sE + (big ? 0 : eb * (kMaxBlocks / 2));
@@ -329,47 +422,42 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       if (it >= 2) mbar_wait(&sel_done[eb], ((it >> 1) - 1) & 1, ctx, 143);
       if (it >= 1 && (big || prev_big)) mbar_wait(&sel_done[eb ^ 1], ((it - 1) >> 1) & 1, ctx, 144);
       prev_big = big;
-      // Accumulators alternate by a chunk count that runs across units.  In a pair, warpgroup w takes tile w of
-      // every chunk, and both hand the accumulator back as soon as their columns are in registers, so the MMAs of
-      // the chunk after next start at once.  In a single-tile unit the warpgroups alternate over the chunks (the
-      // one whose turn it is not only passes the accumulator on).
+      // Accumulators alternate by a chunk count that runs across units, items by a turn that does.  Every warpgroup waits for
+      // every chunk and hands its accumulator back, also where it has no item of the chunk: a warpgroup that were passed by
+      // two chunks of one accumulator could not tell the barrier's phases apart.
       for (int c = 0; c < nchunks; ++c) {
-        const int a = (int)((gc0 + (uint32_t)c) & 1u);
-        uint32_t& ua = a ? uc1 : uc0;
-        mbar_wait(&acc_full[a], ua & 1, ctx, 142);
-        ++ua;
+        const uint32_t n = gc0 + (uint32_t)c;
+        const int a = (int)(n & 1u);
+        mbar_wait(&acc_full[a], (n >> 1) & 1, ctx, 142);
+        int tt = wg - turn;                        // this warpgroup's tile of the chunk, if below nt
+        if (tt < 0) tt += kPairGroups;
+        turn = turn + nt >= kPairGroups ? turn + nt - kPairGroups : turn + nt;
+        if (tt >= nt) {
+          mbar_arrive(&acc_empty[a]);
+          continue;
+        }
         tc_fence_after();
         const int J = c * 128 + key;
-        float m, sum;
-        if (nt > 1) {
-          const uint32_t lane_addr = lane_base + a * 256 + wg * 128;
-          const int nrows = wg ? nrows1 : nrows0;
-          if (nrows == kTileRows) score_cols<false>(lane_addr, cs, kTileRows, &acc_empty[a], m, sum);
-          else score_cols<true>(lane_addr, cs, nrows, &acc_empty[a], m, sum);
-          if (J < (wg ? ncand1 : ncand0)) {
-            const float e = m + log2f(sum);
-            (wg ? e1 : e0)[J] = e;
-            lmax0 = fmaxf(lmax0, e);
-          }
-        } else if (a == wg) {
-          if (nrows0 == kTileRows) score_cols<false>(lane_base + a * 256, cs, kTileRows, &acc_empty[a], m, sum);
-          else score_cols<true>(lane_base + a * 256, cs, nrows0, &acc_empty[a], m, sum);
-          if (J < ncand0) {
-            const float e = m + log2f(sum);
-            e0[J] = e;
-            lmax0 = fmaxf(lmax0, e);
-          }
-        } else {
-          mbar_arrive(&acc_empty[a]);
+        const int nrows = tt ? nrows1 : nrows0;
+        const uint32_t lane_addr = lane_base + a * 256 + tt * 128;
+        const float* mult = &sC[FP8 ? slot : 0][FP8 ? tt * kTileRows : 0];
+        const float e = nrows == kTileRows ? score_cols<FP8, false>(lane_addr, cs, mult, kTileRows, &acc_empty[a])
+                                           : score_cols<FP8, true>(lane_addr, cs, mult, nrows, &acc_empty[a]);
+        if (J < (tt ? ncand1 : ncand0)) {
+          (tt ? e1 : e0)[J] = e;
+          if (tt) lmax1 = fmaxf(lmax1, e);
+          else lmax0 = fmaxf(lmax0, e);
         }
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) lmax0 = fmaxf(lmax0, __shfl_xor_sync(0xffffffffu, lmax0, o));
-      // hand the unit to the selection warp and go on: in a pair the warps of warpgroup w hold maxima of tile w
+      for (int o = 16; o > 0; o >>= 1) {
+        lmax0 = fmaxf(lmax0, __shfl_xor_sync(0xffffffffu, lmax0, o));
+        lmax1 = fmaxf(lmax1, __shfl_xor_sync(0xffffffffu, lmax1, o));
+      }
+      // hand the unit to the selection warp and go on
       if (lane == 0) {
-        const int tt = nt > 1 ? wg : 0;
-        red[eb][tt][warp] = lmax0;
-        red[eb][tt ^ 1][warp] = -INFINITY;
+        red[eb][0][warp] = lmax0;
+        red[eb][1][warp] = lmax1;
       }
       __syncwarp();
       mbar_arrive(&e_full[eb]);
@@ -378,7 +466,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     }
   }
   if (abort_flag) {   // MMAs and bulk copies may still be in flight: let them finish before tensor memory goes
-    if (warp == 9 && elect_one()) {
+    if (warp == 4 * kPairGroups + 1 && elect_one()) {
       umma_commit(&drain_bar);
       mbar_wait_drain(&drain_bar, 0, 200000000ll);
     }
@@ -386,7 +474,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 9) tmem_dealloc(tmem, 512);
+  if (warp == 4 * kPairGroups + 1) tmem_dealloc(tmem, 512);
 }
 
 }  // namespace fp2

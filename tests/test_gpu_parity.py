@@ -377,6 +377,21 @@ def test_scorer_units_pairs_and_singles_of_every_size():
     check_attention(dc, wl, lists, dtype=spec.dtype)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+def test_scorer_pairs_beside_single_tiles_with_more_tiles_than_sms(dtype):
+    """Tiles are only paired where there are more of them than SMs: the three kinds of unit again with four times the tiles,
+    in both data types, odd tile counts and ragged last tiles among them; lists, twice."""
+    spec = inputs.small_spec(seqs=[(900, 0), (140000 + 1100, 140000), (1300, 300), (266240 + 700, 266240), (385, 0)],
+                             num_q_heads=8, num_kv_heads=2, page_size=64, dtype=dtype, config_id=63)
+    spec.alpha = 0.05
+    case, dc, wl = make(spec)
+    assert dc.plan.num_segments > torch.cuda.get_device_properties(0).multi_processor_count
+    for _ in range(2):
+        dc.select()
+        dc.status()
+        check_lists(dc, wl)
+
+
 @pytest.mark.parametrize("alpha", [0.0, 2.0, 1.0])
 def test_alpha_extremes(alpha):
     spec = inputs.small_spec(seqs=[(2000, 0)], num_q_heads=4, num_kv_heads=1, page_size=64, config_id=81, sink=False)
@@ -601,6 +616,28 @@ def test_work_order_takes_every_segment_once(n_seg_tokens):
     lists = {s.seg: idx[off[s.seg]:off[s.seg] + cnt[s.seg]] for s in wl.segs if cnt[s.seg] > 0}
     check_attention(dc, wl, lists, list(lists))
     assert torch.isfinite(dc.out.float()).all()     # rows without a block come out as zeros
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("first_loud", [16, 20, 32])
+def test_scores_far_above_those_of_the_first_rows(first_loud, dtype):
+    """The scorer's exponentials refer to the first 16 rows of a tile; logits more than 2^119 above them must send a batch
+    through again.  One KV head, 32 query heads (a tile is 4 tokens), the queries of the heads from first_loud on 64 times as
+    large (logits in the hundreds): the first batch, a later batch, and with 32 the next token's rows stay quiet throughout.
+    Lists only: probabilities that sharp say nothing more about the attention kernel."""
+    spec = inputs.small_spec(seqs=[(5000, 1000), (901, 0)], num_q_heads=32, num_kv_heads=1, page_size=32, dtype=dtype,
+                             config_id=160 + first_loud)
+    spec.alpha = 0.2
+
+    def louder(case):
+        if dtype == "fp8":
+            case.q_scale[first_loud:] *= 64
+        else:
+            case.q[:, first_loud:] *= 64
+    case, dc, wl = make(spec, edit_case=louder)
+    dc.select()
+    dc.status()
+    check_lists(dc, wl)
 
 
 @pytest.mark.parametrize("hkv", [1, 3])
