@@ -196,7 +196,10 @@ fp2_status fp2_pool_carry_count(const fp2_plan* dst, const fp2_plan* src, const 
  *   is what the workspace is sized for).
  * Larger plans are never split and ignore the setting; so do calls in which no segment could yield two parts.
  * On B200 the split did not pay in any case measured (the attention kernel already keeps two independent CTAs per
- * SM, and the two extra launches cost ~10 us), hence the default.  Host-side, takes effect at the next stage call. */
+ * SM, and the two extra launches cost ~10 us), hence the default.  Host-side, takes effect at the next stage call.
+ * With the default, calls of plans with few segments (under 16 per worker CTA) and long sequences (candidate ranges of 512
+ * blocks and more) still cut segments that are longer than the mean load per worker, and merge their parts in one more
+ * kernel: such a segment would be all that the call waits for at its end. */
 fp2_status fp2_plan_set_split(fp2_plan* plan, int32_t target);
 
 /* Index export (Algorithm 1 line 5; Sec. 3.3 "Index-Driven Sparse Traversal", Eq. 17).  Turns the padded lists

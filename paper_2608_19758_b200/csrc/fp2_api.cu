@@ -50,6 +50,8 @@ struct fp2_plan {
   int64_t v16_iters;      // FP8: iterations of an attention call from which V as F16 pays (see use_v16)
   int64_t likely_iters;   // FP8: iterations a sparse call can be expected to have
   int32_t max_iters;      // longest iteration sequence any segment can have (all candidates + all chunks)
+  int32_t cut_slots;      // partial-result slots of attention calls that cut their longest segments (see order_scatter_kernel), 0: no cutting
+  int64_t ws_cut_split;   // [nseg + cut_slots]: part of every unit of such a call, then [nseg] and [cut_slots / 2] for the merge
   int64_t split_units_cap, ws_unit_seg, ws_unit_split, ws_seg_split, ws_part_ml, ws_part_o;
   EncodeTiledFn encode;
   int32_t last_launches;
@@ -64,6 +66,8 @@ struct fp2_plan {
 // 3824 / 3579, dense 16384 tokens 1782 / 1486.  A sparse call's lists are not known on the host: 20 blocks per tile (sink,
 // window and diagonal are 7 to 8 of them).
 constexpr int kLikelyListLen = 20;
+constexpr int kCutSlots = 256;       // 16.7 MB of partial results
+constexpr int kCutMinCand = 512;     // longest candidate range (60160 tokens, 4 heads, nothing to cut: the launch costs 2 of 101 us)
 static inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 extern "C" const char* fp2_status_string(fp2_status s) {
@@ -261,19 +265,25 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
   pl->ws_v16 = o;
   if (p->dtype == FP2_FP8_E4M3 && pl->idx_capacity >= pl->v16_iters)   // (a dense call has that many iterations)
     o += align_up(nblk_tot * kBlock * p->num_kv_heads * kHeadDim * 2, 1024);
-  pl->ws_order = o; o += align_up(4 * (pl->nseg > 0 ? pl->nseg : 1), 1024);
+  // Attention calls cut their longest segments where one can outlast a worker's share: not with 16 segments per worker and
+  // more (the longest is seldom half a share then), and not where no list can be long (a launch more and two loads per unit
+  // would be all that comes of it).
+  const int64_t workers = (int64_t)pl->num_sms * AttnCfg<false>::kCtasPerSm;
+  pl->cut_slots = pl->nseg > 0 && pl->nseg < 16 * workers && pl->max_iters >= kCutMinCand ? kCutSlots : 0;
+  pl->ws_order = o; o += align_up(4 * (pl->nseg > 0 ? pl->nseg + pl->cut_slots : 1), 1024);
+  pl->ws_cut_split = o; o += align_up(pl->cut_slots ? 4 * (2 * pl->nseg + 2 * pl->cut_slots) : 0, 1024);
   pl->ws_hist = o;  o += align_up(8 * (int64_t)p->num_kv_heads * kCountBuckets, 1024);
   // KV splitting pays when there are fewer units than a few waves of workers; the unit arrays and the partial
   // results are sized for nseg + 2 workers units, the bound split_plan_kernel keeps
-  const int64_t workers = (int64_t)pl->num_sms * AttnCfg<false>::kCtasPerSm;
   pl->split_target = -1;   // off unless asked for: see fp2_plan_set_split
   pl->split_capable = pl->num_sms > 0 && pl->nseg > 0 && pl->nseg < 4 * workers && pl->nseg + 2 * workers < 65536;
   pl->split_units_cap = pl->split_capable ? pl->nseg + 2 * workers : 0;
   pl->ws_unit_seg = o;   o += align_up(4 * pl->split_units_cap, 1024);
   pl->ws_unit_split = o; o += align_up(4 * pl->split_units_cap, 1024);
   pl->ws_seg_split = o;  o += align_up(pl->split_capable ? 8 * pl->nseg : 0, 1024);   // per-segment word + list of split segments
-  pl->ws_part_ml = o;    o += align_up(pl->split_units_cap * 128 * 8, 1024);
-  pl->ws_part_o = o;     o += pl->split_units_cap * 128 * 128 * 4;
+  const int64_t part_slots = std::max<int64_t>(pl->split_units_cap, pl->cut_slots);
+  pl->ws_part_ml = o;    o += align_up(part_slots * 128 * 8, 1024);
+  pl->ws_part_o = o;     o += part_slots * 128 * 128 * 4;
   pl->ws_bytes = o;
 
   DevParams& d = pl->dev;
@@ -450,16 +460,18 @@ static fp2_status launch_pool(fp2_plan* pl, const void* k, const void* v, const 
 
 // What an attention call runs before its kernel: the counting sort of the segments (KV-head-major, descending block count;
 // hist: class counts and cursors, 2 nb words), and for FP8 plans with a workspace V as F16 (v16, else NULL).
-static void launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, int32_t* counter,
-                           const void* v, const int32_t* pt, __half* v16, int* status, cudaStream_t st) {
+// cut: see order_scatter_kernel.
+static void launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, const CutLists& cut,
+                           int32_t* counter, const void* v, const int32_t* pt, __half* v16, int* status, cudaStream_t st) {
   const int nseg = (int)pl->nseg;
   const int nb = pl->prm.num_kv_heads * kCountBuckets;
   const unsigned blocks = (unsigned)((nseg + 255) / 256), n_clear = (unsigned)((2 * nb + 255) / 256);
   launch(attn_prepare_kernel, n_clear + (v16 ? (unsigned)(pl->nblk_tot * (kBlock / kWidenTokens)) : 0u), 256, 0, st, hist, 2 * nb, counter, (int)n_clear,
          (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, pl->dev, v16, status);
   launch(order_hist_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, hist);
-  launch(order_scatter_kernel, blocks, 256, sizeof(int32_t) * pl->prm.num_kv_heads, st, pl->d_segs, seg_count, nseg,
-         nseg / pl->prm.num_kv_heads, pl->prm.num_kv_heads, pl->num_sms * AttnCfg<false>::kCtasPerSm, hist, hist + nb, order);
+  launch(cut.unit_split ? order_scatter_kernel<true> : order_scatter_kernel<false>, blocks, 256, sizeof(int32_t) * pl->prm.num_kv_heads, st, pl->d_segs, seg_count, nseg,
+         nseg / pl->prm.num_kv_heads, pl->prm.num_kv_heads, pl->num_sms * AttnCfg<false>::kCtasPerSm, hist, hist + nb, order,
+         cut);
   pl->last_launches += 3;
 }
 
@@ -555,8 +567,18 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   if (pl->nseg == 0) return FP2_OK;
   if (need_pool && (s = launch_pool(pl, k, v, pt, ks, vs, ws, st)) != FP2_OK) return s;
   const bool use_v16 = pl->dev.fp8 && (seg_count ? pl->likely_iters : pl->idx_capacity) >= pl->v16_iters;
+  CutLists cut = {};
+  int32_t* const counter = reinterpret_cast<int32_t*>(ws + pl->ws_counter);
+  if (pl->cut_slots > 0 && pl->split_target < 0) {
+    cut.unit_split = reinterpret_cast<int32_t*>(ws + pl->ws_cut_split);
+    cut.seg_split = cut.unit_split + pl->nseg + pl->cut_slots;
+    cut.split_list = cut.seg_split + pl->nseg;
+    cut.n_units = counter + 1;
+    cut.n_split = counter + 2;
+    cut.max_slots = pl->cut_slots;
+  }
   launch_prepare(pl, seg_count, reinterpret_cast<int32_t*>(ws + pl->ws_hist), reinterpret_cast<int32_t*>(ws + pl->ws_order),
-                 reinterpret_cast<int32_t*>(ws + pl->ws_counter), v, pt,
+                 cut, counter, v, pt,
                  use_v16 ? reinterpret_cast<__half*>(ws + pl->ws_v16) : nullptr,
                  reinterpret_cast<int*>(ws + pl->ws_status), st);
   const bool fp8 = pl->dev.fp8 != 0;
@@ -587,7 +609,10 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   a.lse = lse;
   a.work_counter = reinterpret_cast<int*>(ws + pl->ws_counter);
   a.status = reinterpret_cast<int*>(ws + pl->ws_status);
-  a.unit_split = nullptr; a.n_units = nullptr; a.part_o = nullptr; a.part_ml = nullptr;
+  a.unit_split = cut.unit_split;
+  a.n_units = cut.n_units;
+  a.part_o = reinterpret_cast<float*>(ws + pl->ws_part_o);
+  a.part_ml = reinterpret_cast<float2*>(ws + pl->ws_part_ml);
 #ifdef FP2_PROFILE
   a.prof = g_prof_ptr;
 #endif
@@ -595,14 +620,14 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   // longest candidate range (plus its correction chunks) is below one and a half such parts
   const int min_len = pl->split_target > 0 ? pl->split_target : kMinPartLen;
   const bool split = pl->split_capable && pl->split_target >= 0 && 2 * pl->max_iters >= 3 * min_len;
-  int64_t max_units = pl->nseg;
+  int64_t max_units = pl->nseg + cut.max_slots;
   if (split) {
     // device-side scheduler prep (Eq. 18): units = parts of segments, in the work order
     int32_t* unit_seg = reinterpret_cast<int32_t*>(ws + pl->ws_unit_seg);
     int32_t* unit_split = reinterpret_cast<int32_t*>(ws + pl->ws_unit_split);
     int32_t* seg_split = reinterpret_cast<int32_t*>(ws + pl->ws_seg_split);
     int32_t* split_list = seg_split + pl->nseg;
-    int32_t* n_units = reinterpret_cast<int32_t*>(ws + pl->ws_counter) + 1;
+    int32_t* n_units = counter + 1;
     int32_t* n_split = n_units + 1;
     const int workers = pl->num_sms * AttnCfg<false>::kCtasPerSm;
     launch(split_plan_kernel, 1, 1024, 0, st, pl->d_segs, a.order, seg_count, (int)pl->nseg, pl->dev.use_correction,
@@ -612,19 +637,17 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
     a.order = unit_seg;
     a.unit_split = unit_split;
     a.n_units = n_units;
-    a.part_o = reinterpret_cast<float*>(ws + pl->ws_part_o);
-    a.part_ml = reinterpret_cast<float2*>(ws + pl->ws_part_ml);
     max_units = pl->split_units_cap;
   }
   CUtensorMap mq = mk;   // unused unless q_box
   if (pl->dev.q_box && !make_q_map(pl, &mq, q, pl->dev.q_box_tok)) return FP2_ERR_CUDA;
   launch_attn(pl, mk, mv, mkb, mkb_lo, mvb, mq, a, max_units, !use_v16, st);
   pl->last_launches += 1;
-  if (split) {
-    int32_t* seg_split = reinterpret_cast<int32_t*>(ws + pl->ws_seg_split);
-    launch(split_combine_kernel, (unsigned)(pl->num_sms * 8), 128, 0, st, pl->d_segs, seg_split, seg_split + pl->nseg,
-           reinterpret_cast<int32_t*>(ws + pl->ws_counter) + 2, a.part_o,
-        a.part_ml, fp8 ? vs : nullptr, pl->dev, a.out, lse);
+  if (split || cut.unit_split != nullptr) {
+    int32_t* seg_split = split ? reinterpret_cast<int32_t*>(ws + pl->ws_seg_split) : cut.seg_split;
+    launch(split_combine_kernel, (unsigned)(pl->num_sms * 8), 128, 0, st, pl->d_segs, seg_split,
+           split ? seg_split + pl->nseg : cut.split_list, counter + 2, a.part_o, a.part_ml, fp8 ? vs : nullptr, pl->dev, a.out,
+           lse);
     pl->last_launches += 1;
   }
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
@@ -697,8 +720,8 @@ extern "C" fp2_status fp2_dense_prefill_static(fp2_plan* pl, const void* q, cons
   int32_t* order = reinterpret_cast<int32_t*>(sw + kStaticOffOrder);
   // the array keeps the previous call's contents: the status block must start at zero (the sort clears the rest)
   if (cudaMemsetAsync(sw, 0, 64, st) != cudaSuccess) return FP2_ERR_CUDA;
-  launch_prepare(pl, nullptr, reinterpret_cast<int32_t*>(sw + kStaticOffHist), order, reinterpret_cast<int32_t*>(sw + 64), v,
-                 pt, nullptr, reinterpret_cast<int*>(sw), st);
+  launch_prepare(pl, nullptr, reinterpret_cast<int32_t*>(sw + kStaticOffHist), order, CutLists{},
+                 reinterpret_cast<int32_t*>(sw + 64), v, pt, nullptr, reinterpret_cast<int*>(sw), st);
   const int64_t slots = (int64_t)pl->prm.num_pages * pl->prm.page_size;
   CUtensorMap mk, mv;
   const bool fp8 = pl->dev.fp8 != 0;

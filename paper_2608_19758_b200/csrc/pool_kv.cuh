@@ -17,6 +17,7 @@
 #include <cuda_fp8.h>
 #include "common.cuh"
 #include "ptx.cuh"
+#include "split_kv.cuh"   // pack_split
 
 namespace fp2 {
 
@@ -380,14 +381,55 @@ __device__ __forceinline__ int class_min_count(int c) {   // smallest block coun
   const int v = kCountBuckets - 1 - c;
   return v < 64 ? v : (8 + (v & 7)) << ((v - 64) / 8 + 3);
 }
+// Cutting (Eq. 18).  A segment longer than a worker's share outlasts the rest even when it starts first (the last 8192 of
+// 131072 tokens: one list of 408 blocks against a share of 349).  Calls that can have such segments (template parameter CUT, see
+// fp2_plan_create) ask for units instead of segments: if the longest class exceeds kCutFrom shares, segments longer than half a
+// share become parts of about that length, longest classes first while their partial results fit into max_slots, and the
+// merge kernel of the split path puts them together.  That call 1279 -> 1056 us; where the longest list is three quarters of a
+// share cutting gained nothing (107371-token chunk 978 / 989).
+// unit_split[w]: see pack_split; *n_units: units; seg_split, split_list, *n_split: what the merge kernel reads.
+struct ClassScan {   // exclusive prefix over the classes, four per lane of a warp
+  int before[4], total;
+  __device__ __forceinline__ ClassScan(const int (&c)[4], int lane) {
+    const int mine = c[0] + c[1] + c[2] + c[3];
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    int run = incl - mine;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      before[i] = run;
+      run += c[i];
+    }
+    total = __shfl_sync(0xffffffffu, incl, 31);
+  }
+};
+constexpr float kCutFrom = 1.0f;
+constexpr int kCutMin = 64;           // blocks of a segment below which cutting costs more (Q tile, partial result, merge) than it gives
+constexpr int kMaxCuts = 8;           // parts of a segment
+struct CutLists {
+  int32_t* unit_split;
+  int32_t* seg_split;
+  int32_t* split_list;
+  int32_t* n_units;
+  int32_t* n_split;
+  int32_t max_slots;
+};
+template <bool CUT>
 __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __restrict__ segs, const int32_t* count, int nseg,
                                                             int per_head, int num_heads, int workers, const int32_t* hist,
-                                                            int32_t* __restrict__ cursor, int32_t* __restrict__ order) {
+                                                            int32_t* __restrict__ cursor, int32_t* __restrict__ order,
+                                                            CutLists cut) {
   static_assert(kCountBuckets == 128, "thread t adds up class t mod 128; a lane of the scan takes four classes");
   extern __shared__ int32_t head_long[];       // [num_heads] long segments per head
   __shared__ int32_t col[2][kCountBuckets];    // segments per class over all heads (two halves of the heads)
-  __shared__ int32_t before[kCountBuckets];    // long segments of the classes in front of this one
-  __shared__ int s_first_short, s_num_long;    // first class that is not long; number of long segments
+  __shared__ int32_t before[kCountBuckets];    // units of the long segments of the classes in front of this one
+  __shared__ int32_t parts[kCountBuckets];      // parts per segment of the class
+  __shared__ int32_t slots_before[kCountBuckets], cuts_before[kCountBuckets];   // partial-result slots, cut segments likewise
+  __shared__ int s_first_short, s_num_long;    // first class that is not long; units of the long segments
   pdl_trigger();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int s = blockIdx.x * blockDim.x + t;
@@ -398,42 +440,67 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
   for (int i = t >> 7; i < num_heads; i += 2) sum += hist[i * kCountBuckets + (t & 127)];
   col[t >> 7][t & 127] = sum;
   __syncthreads();
-  if (warp == 0) {   // scan over the classes, four per lane
-    int c[4], mine = 0;
+  if (warp == 0) {   // scans over the classes, four per lane
+    int c[4], u[4], x[4];
     float blocks = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       c[i] = col[0][lane * 4 + i] + col[1][lane * 4 + i];
       blocks += (float)c[i] * (float)class_min_count(lane * 4 + i);
-      mine += c[i];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) blocks += __shfl_xor_sync(0xffffffffu, blocks, o);
-    int incl = mine;
+    const float share = blocks / (float)workers;
+    int longest = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    int run = incl - mine, n_long = 0, long_classes = 0;
-    const float limit = blocks / ((float)workers * kLongShare);
+    for (int i = 0; i < 4; ++i) longest = max(longest, c[i] > 0 ? class_min_count(lane * 4 + i) : 0);
+    longest = CUT ? __reduce_max_sync(0xffffffffu, longest) : 0;
+    const bool cutting = CUT && longest >= kCutMin && (float)longest > kCutFrom * share;
+    int n_long = 0, n_cut = 0, long_classes = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      before[lane * 4 + i] = run;
-      run += c[i];
-      if ((float)class_min_count(lane * 4 + i) > limit) {   // (holds for the first classes: they count down)
+      const float len = (float)class_min_count(lane * 4 + i);
+      const bool is_long = len * kLongShare > share;   // (holds for the first classes: they count down)
+      if (is_long) {
         ++long_classes;
         n_long += c[i];
+      } else {
+        c[i] = 0;
       }
+      u[i] = is_long && cutting && len >= (float)kCutMin ? min(kMaxCuts, max(1, (int)ceilf(len / (0.5f * share)))) : 1;
+      x[i] = u[i] > 1 ? c[i] * u[i] : 0;
+    }
+    if (cutting) {
+      const ClassScan slots(x, lane), segs_before(c, lane);   // (classes that are cut come before those that are not)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (slots.before[i] + x[i] > cut.max_slots) u[i] = 1;   // (a prefix: from the first class that does not fit, none is cut)
+        n_cut += u[i] > 1 ? c[i] : 0;
+        slots_before[lane * 4 + i] = slots.before[i];
+        cuts_before[lane * 4 + i] = segs_before.before[i];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = c[i] * u[i];
+    const ClassScan units(x, lane);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      before[lane * 4 + i] = units.before[i];
+      if constexpr (CUT) parts[lane * 4 + i] = u[i];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       n_long += __shfl_xor_sync(0xffffffffu, n_long, o);
+      n_cut += __shfl_xor_sync(0xffffffffu, n_cut, o);
       long_classes += __shfl_xor_sync(0xffffffffu, long_classes, o);
     }
     if (lane == 0) {
-      s_num_long = n_long;
+      s_num_long = units.total;
       s_first_short = long_classes;
+      if (CUT && blockIdx.x == 0) {
+        *cut.n_units = units.total + nseg - n_long;
+        *cut.n_split = n_cut;
+      }
     }
   }
   __syncthreads();
@@ -450,7 +517,16 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
   if (s >= nseg) return;
   const int b = order_bucket(h, n), cls = b - h * kCountBuckets;
   if (cls < first_short) {
-    order[before[cls] + atomicAdd(&cursor[cls], 1)] = s;   // (the cursors of head 0's long classes serve all heads)
+    const int k = atomicAdd(&cursor[cls], 1), U = CUT ? parts[cls] : 1;   // (the cursors of head 0's long classes serve all heads)
+    const int slot = U > 1 ? slots_before[cls] + k * U : 0;
+    for (int u = 0; u < U; ++u) {
+      order[before[cls] + k * U + u] = s;
+      if constexpr (CUT) cut.unit_split[before[cls] + k * U + u] = pack_split(u, U, slot);
+    }
+    if (U > 1) {
+      cut.seg_split[s] = pack_split(0, U, slot);
+      cut.split_list[cuts_before[cls] + k] = s;
+    }
     return;
   }
   int pos = s_num_long + h * per_head;
@@ -458,7 +534,9 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
   const int32_t* row = hist + h * kCountBuckets;
 #pragma unroll 4
   for (int i = first_short; i < cls; ++i) pos += row[i];
-  order[pos + atomicAdd(&cursor[b], 1)] = s;
+  pos += atomicAdd(&cursor[b], 1);
+  order[pos] = s;
+  if constexpr (CUT) cut.unit_split[pos] = pack_split(0, 1, 0);
 }
 
 // ----------------------------------------------------------------------------------------

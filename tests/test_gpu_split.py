@@ -76,3 +76,36 @@ def test_large_plans_are_not_split():
     dc.plan.set_split(1)
     dc.select(); dc.sparse(); dc.status()
     assert dc.plan.last_launch_count() == 4
+
+
+@pytest.mark.parametrize("dtype,g,hkv,seqs", [
+    ("bf16", 4, 1, [(66000, 65700), (9000, 8000), (129, 0)]),    # ragged last tiles
+    ("bf16", 7, 1, [(70000, 69300)]),
+    ("fp8", 4, 2, [(66000, 65500), (5000, 4000)]),
+])
+def test_longest_segments_are_cut_without_being_asked(dtype, g, hkv, seqs):
+    """Caller lists: every 9th segment complete (500 blocks and more, above a worker's share), the others the diagonal band.
+    The attention call cuts the long ones into parts and merges them (one launch more).  The second run equals the first bit
+    for bit; dense, where all segments of the long sequence are that long, and more of them than partial results fit."""
+    spec = inputs.small_spec(seqs=seqs, num_q_heads=g * hkv, num_kv_heads=hkv, page_size=64, dtype=dtype, config_id=180 + g)
+    case, dc, wl = make(spec)
+    dc.select(); dc.status()
+    off = dc.seg_offset.cpu().numpy()
+    cnt = np.zeros(dc.plan.num_segments, dtype=np.int32)
+    idx = dc.blk_idx.cpu().numpy().copy()
+    for s in wl.segs:
+        first = 0 if s.seg % 9 == 0 else s.J_lo
+        cnt[s.seg] = s.J_hi + 1 - first
+        idx[off[s.seg]:off[s.seg] + cnt[s.seg]] = np.arange(first, s.J_hi + 1)
+    workers = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert cnt.max() >= 500 and cnt.max() > cnt.sum() / workers
+    lists = {s.seg: idx[off[s.seg]:off[s.seg] + cnt[s.seg]] for s in wl.segs}
+    c, i = torch.from_numpy(cnt).cuda(), torch.from_numpy(idx).cuda()
+    dc.sparse(seg_count=c, blk_idx=i); dc.status()
+    assert dc.plan.last_launch_count() == 5
+    check_attention(dc, wl, lists, dtype=dtype)
+    o, l = dc.out.clone(), dc.lse.clone()
+    dc.sparse(seg_count=c, blk_idx=i); dc.status()
+    assert torch.equal(o, dc.out) and torch.equal(l, dc.lse)
+    dc.dense(); dc.status()
+    check_attention(dc, wl, None, dense=True, dtype=dtype)
