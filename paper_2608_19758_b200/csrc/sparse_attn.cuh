@@ -460,7 +460,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       const int32_t* list = A.blk_idx + sg.off;
       const int32_t* pt = A.page_table + (size_t)sg.b * P.max_pages_per_seq;
       // page id of this lane's page of exact iteration i (-1: past the end of the sequence, or not an exact
-      // iteration).  Fetched one iteration ahead: list entry -> page-table entry are two dependent global loads.
+      // iteration).  Fetched one iteration ahead, behind the K tile's copies: list entry -> page-table entry are two dependent
+      // global loads, and the first K tile of a unit should not wait for the second's.
       int J_fetched = 0;   // block id of the iteration fetch_pid was last asked for (warp-uniform)
       auto fetch_pid = [&](int i) -> int {
         if (i >= T) return -1;
@@ -499,7 +500,6 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       for (int i = ti.it_begin; i < ti.it_end; ++i, ++G) {
         const int pid = pid_next;
         const int J_cur = J_fetched;
-        pid_next = fetch_pid(i + 1);
         if (G >= 1) mbar_wait(&s_done, (G - 1) & 1, ctx, 302);   // K stage free
         if (i < ti.ndiag && P.diag_mma) {
           // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c
@@ -517,6 +517,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             if (lane == 0) mbar_arrive_expect_tx(&k_full, bytes);
             __syncwarp();
             if (pid >= 0) tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
+            pid_next = fetch_pid(i + 1);
             if constexpr (WIDEN) {
               if (rc >= 1) mbar_wait(&vraw_empty, (rc - 1) & 1, ctx, 306);
               if (lane == 0) mbar_arrive_expect_tx(&vraw_full, bytes);
@@ -541,6 +542,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
               tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
               tma_load_3d_hint(sK + 16384 + lane * psz * 128, &map_k, &k_full, 64, sg.h, pid * psz, keep);
             }
+            pid_next = fetch_pid(i + 1);
             if (G >= 1) wait_pv(G - 1, 303);  // V stage free
             if (lane == 0) mbar_arrive_expect_tx(&v_full, bytes);
             __syncwarp();
