@@ -829,10 +829,11 @@ extern "C" fp2_status fp2_export_csr(fp2_plan* pl, const int32_t* seg_count, con
   int* status = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(workspace) + pl->ws_status);
   const int nseg = (int)pl->nseg;
   pl->last_launches = 0;
-  launch(csr_count_kernel, (nseg + 256) / 256, 256, 0, st, pl->d_segs, seg_count, blk_idx, nseg, tile_tokens, cu, status);
+  launch(csr_count_kernel, (unsigned)std::max(1, (nseg + kCsrGroup - 1) / kCsrGroup), kCsrGroup, 0, st, pl->d_segs, seg_count,
+         blk_idx, nseg, tile_tokens, cu, status);
   pl->last_launches += 1;
   if (nseg > 0) {
-    launch(csr_scan_kernel, 1, 1024, 0, st, cu, nseg);
+    launch(csr_offset_kernel, 1, 1024, 0, st, cu, nseg);
     launch(csr_fill_kernel, (unsigned)(((int64_t)nseg * 32 + 255) / 256), 256, 0, st, pl->d_segs, seg_count, blk_idx, nseg,
                                                                                  tile_tokens, cu, idx, status);
     pl->last_launches += 2;

@@ -45,6 +45,17 @@ def test_export_matches_oracle(tile, seqs, g, hkv, p):
     assert n > 0
 
 
+@pytest.mark.parametrize("tokens,hkv", [(255, 1), (256, 1), (257, 1), (171, 3), (2049, 1)])
+def test_export_at_the_edges_of_the_offset_groups(tokens, hkv):
+    """A tile per token (128 query heads per KV head): 255, 256, 257, 513 and 2049 segments around the groups of 256 whose
+    counts are scanned by one CTA each."""
+    spec = inputs.small_spec(seqs=[(tokens, 0)], num_q_heads=128 * hkv, num_kv_heads=hkv, page_size=16, config_id=67)
+    case, dc, wl = make(spec)
+    assert dc.plan.num_segments == tokens * hkv
+    dc.select(); dc.status()
+    check_export(dc, wl, 64)
+
+
 def test_export_of_dense_lists_config2():
     """All candidates listed at 32K: 2 tiles per block, 2 x 1 052 672 entries."""
     spec = inputs.config_spec(2)
