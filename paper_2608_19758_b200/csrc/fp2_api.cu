@@ -468,9 +468,10 @@ static void launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist
   const unsigned blocks = (unsigned)((nseg + 255) / 256), n_clear = (unsigned)((2 * nb + 255) / 256);
   launch(attn_prepare_kernel, n_clear + (v16 ? (unsigned)(pl->nblk_tot * (kBlock / kWidenTokens)) : 0u), 256, 0, st, hist, 2 * nb, counter, (int)n_clear,
          (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, pl->dev, v16, status);
-  launch(order_hist_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, hist);
+  const int workers = pl->num_sms * AttnCfg<false>::kCtasPerSm;
+  launch(order_hist_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, cut.unit_split ? 0 : workers, hist);
   launch(cut.unit_split ? order_scatter_kernel<true> : order_scatter_kernel<false>, blocks, 256, sizeof(int32_t) * pl->prm.num_kv_heads, st, pl->d_segs, seg_count, nseg,
-         nseg / pl->prm.num_kv_heads, pl->prm.num_kv_heads, pl->num_sms * AttnCfg<false>::kCtasPerSm, hist, hist + nb, order,
+         nseg / pl->prm.num_kv_heads, pl->prm.num_kv_heads, workers, hist, hist + nb, order,
          cut);
   pl->last_launches += 3;
 }

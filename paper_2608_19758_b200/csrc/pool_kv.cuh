@@ -356,13 +356,15 @@ __global__ void __launch_bounds__(256) attn_prepare_kernel(int32_t* __restrict__
   if (i < 16) counter[i] = 0;
 }
 
-__global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_t* count, int nseg,
+// Where every segment has a worker of its own (nseg <= workers) all of them start at once: there is nothing to sort, the order
+// is the segments' own.  Select + sparse, 768 tokens FP8 35.1 -> 32.9 us, 2370 tokens 38.6 -> 36.9; dense, 839 tokens 21.5 -> 21.0.
+__global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_t* count, int nseg, int workers,
                                   int32_t* __restrict__ hist) {
   pdl_trigger();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   const int h = s < nseg ? segs[s].h : 0, J = s < nseg ? segs[s].J_hi : 0;   // the plan's table: not written by any kernel
   pdl_wait();
-  if (s >= nseg) return;
+  if (s >= nseg || nseg <= workers) return;
   atomicAdd(&hist[order_bucket(h, count ? count[s] : J + 1)], 1);
 }
 
@@ -435,6 +437,10 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
   const int s = blockIdx.x * blockDim.x + t;
   const int h = s < nseg ? segs[s].h : 0, J = s < nseg ? segs[s].J_hi : 0;
   pdl_wait();
+  if (!CUT && nseg <= workers) {
+    if (s < nseg) order[s] = s;
+    return;
+  }
   const int n = s >= nseg ? 0 : count ? count[s] : J + 1;
   int sum = 0;
   for (int i = t >> 7; i < num_heads; i += 2) sum += hist[i * kCountBuckets + (t & 127)];
