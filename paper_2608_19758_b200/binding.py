@@ -109,10 +109,16 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()     # ctypes takes a plain integer for a void pointer
 
 
+# The current stream's handle without a Stream object around it (4.3 us per stage call, of 11 to 15 us on the host).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def fp2_status_string(code: int) -> str:
