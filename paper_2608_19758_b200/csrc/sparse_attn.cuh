@@ -100,7 +100,24 @@ struct AttnArgs {
 #define PF_END(k)
 #endif
 
-constexpr int kPParts = 4;   // P is handed to the issuer in this many column slices (4 or 8)
+// P is handed to the issuer in column slices.  Each hand-over stalls the warp for its TMEM stores, and what follows the last one
+// (the slice's MMAs, then S = Q K^T) is what the warp waits for; so: a short first slice to get O += P V going, a long middle
+// one, a short last one.  In k-steps (of eight), us at the power limit: 32768 tokens dense BF16 4 x 2 8290, 4 + 4 7920, 2 + 5 + 1
+// 7600, 2 + 4 + 2 7360; 131072 tokens 8930 / 8620 / 8530 / 8330; dense 16384 tokens FP8 1492 / 1488 / 1411 / 1484, 16 sequences
+// FP8 3376 / 3270 / 3295 / 3321.  16 columns a store, except FP8, whose middle slice ends inside 16 (8 there: 1411, 16: 1465).
+constexpr int kPParts = 3;
+template <bool FP8>
+struct PSlices {
+  static constexpr int kStore = FP8 ? 8 : 16;   // packed registers (= P columns) per TMEM store
+  // k-steps (16 probabilities of a row, 8 columns) that are there once slice h is
+  __host__ __device__ static constexpr int end(int h) { return h == 0 ? 2 : h == 1 ? (FP8 ? 7 : 6) : 8; }
+  // slice that is complete after this many k-steps, -1: none
+  __host__ __device__ static constexpr int complete(int steps) {
+    for (int h = 0; h < kPParts; ++h)
+      if (end(h) == steps) return h;
+    return -1;
+  }
+};
 
 template <bool FP8>
 struct AttnCfg {
@@ -165,16 +182,17 @@ __device__ __forceinline__ float row_load_max(uint32_t s_addr, uint32_t (&x)[128
 }
 
 // p = 2^(x * cs + neg_m) for the 128 logits in registers, written as BF16 (F16) pairs to the 64 columns at p_addr.
-// Scaling and row sum use packed fp32x2 instructions.  After the first 64 probabilities the thread arrives on
-// half_ready.  Returns the row sum.
+// Scaling and row sum use packed fp32x2 instructions.  The thread arrives on part_ready as the slices (but the last) are
+// complete.  Returns the row sum.
 template <bool F16>
 __device__ __forceinline__ float row_exp(const uint32_t (&x)[128], uint32_t p_addr, float cs, float neg_m,
                                          uint64_t* part_ready) {
   const uint64_t cs2 = f2_pack(cs, cs), nm2 = f2_pack(neg_m, neg_m);
   uint64_t sum2[4] = {0ull, 0ull, 0ull, 0ull};   // four independent (lo, hi) accumulators, +0.0f bit patterns
+  using Slices = PSlices<F16>;
+  constexpr int W = Slices::kStore;
 #pragma unroll
-  for (int k = 0; k < kPParts; ++k) {
-    constexpr int W = 64 / kPParts;   // packed registers (= P columns) per part
+  for (int k = 0; k < 64 / W; ++k) {
     uint32_t pk[W];
 #pragma unroll
     for (int j = 0; j < W; ++j) {
@@ -187,10 +205,11 @@ __device__ __forceinline__ float row_exp(const uint32_t (&x)[128], uint32_t p_ad
       pk[j] = F16 ? pack_f16x2(p0, p1) : pack_bf16x2(p0, p1);
     }
     tmem_st_cols(p_addr + k * W, pk);
-    if (k + 1 < kPParts) {   // a part of P: O += P V may run its next k-steps
+    const int slice = Slices::complete((k + 1) * W / 8);
+    if (slice >= 0 && slice + 1 < kPParts) {   // O += P V may run the slice's k-steps
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(&part_ready[k]);
+      mbar_arrive(&part_ready[slice]);
     }
   }
   float a0, a1;
@@ -241,7 +260,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
                                    // O holds iteration G.  Two barriers so that a waiter may be two iterations
                                    // behind the issuer without mistaking one phase for another.
   __shared__ uint64_t vraw_full, vraw_empty;   // WIDEN: the raw V tile has landed / has been widened
-  __shared__ uint64_t p_ready[kPParts];   // slice q (128 / kPParts probabilities of every row) of P (G) is in TMEM
+  __shared__ uint64_t p_ready[kPParts];   // slice q (see PSlices) of P (G) is in TMEM
   __shared__ uint32_t tmem_base_s;
   __shared__ int abort_flag;
   __shared__ int ndiag_s, unit_s;
@@ -653,7 +672,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
           tc_fence_after();
           if (leader) {
 #pragma unroll
-            for (int ks = (8 / kPParts) * h; ks < (8 / kPParts) * (h + 1); ++ks)
+            for (int ks = h ? PSlices<FP8>::end(h - 1) : 0; ks < PSlices<FP8>::end(h); ++ks)
               umma_f16_ts(tmem + 128, tmem + ks * 8, v_desc + ks * 128, idesc_pv, (i > i0) || ks > 0);
           }
         }
@@ -677,7 +696,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         tc_fence_after();
         if (leader) {
 #pragma unroll
-          for (int ks = 8 - 8 / kPParts; ks < 8; ++ks)
+          for (int ks = PSlices<FP8>::end(kPParts - 2); ks < 8; ++ks)
             umma_f16_ts(tmem + 128, tmem + ks * 8, v_desc + ks * 128, idesc_pv, 1u);
           umma_commit(&pv_done[G & 1]);
           if (qk_issued) issue_qk(masked, chunk, last);
