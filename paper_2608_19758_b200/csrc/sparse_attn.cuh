@@ -23,7 +23,7 @@
 // Everything is single-buffered: S = Q K^T of iteration i+1 is issued behind O += P V of iteration i (which
 // reads P out of the S columns), the K tile of i+1 is requested when S = Q K^T (i) has completed and the V tile
 // when O += P V (i) has.  The other CTA of the SM fills the bubbles this leaves.  P is handed to the issuer in
-// kPParts column slices, so O += P V runs its first k-steps under the remaining exponentials.
+// kPParts column slices (see PSlices), so O += P V runs its first k-steps under the remaining exponentials.
 //
 // Roles: warps 0..3 softmax + epilogue; warp 4 TMA producer (Eq. 22); warp 5 UMMA issuer (and TMEM owner);
 // warps 6, 7 unit set-up (fetch the next unit, validate its list, build the correction masks, stage Q).
@@ -320,8 +320,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     // A chain of dependent global loads (work counter -> order -> segment and count -> list -> page table), which at the start
     // of a call nothing hides: both warps load what they need themselves instead of passing it on, the page-table entries of
     // the list go to the L1 for the producer, the first unit is the CTA's own number, and its query tile is requested as soon
-    // as the segment is known.  2048 tokens: logits of the first block after 8000 cycles of the kernel (9100 before); see the issuer for
-    // whole calls.
+    // as the segment is known.  2048 tokens: logits of the first block after 8000 cycles of the kernel (9100 before), whole call
+    // 38.6 -> 37.4 us; 16 sequences of 245000 tokens 3561 -> 3513, 60160 tokens with 4 heads 100.8 -> 96.1.
     setmaxnreg_dec<AttnCfg<FP8>::kRegsService>();
     const int t64 = tid - 32 * 6;
     const bool corr = P.use_correction != 0;
@@ -644,9 +644,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     // Look-ahead.  A shared-memory wait that follows a commit in this warp is held until the commit has been taken: from the last
     // slice of O += P V to S = Q K^T (G+1) it took some 500 cycles although K (G+1) had long landed.  So what S = Q K^T (G+1)
     // needs is looked at BEFORE the last slice of P (G) is waited for, across a unit boundary too, and where it is there its
-    // MMAs follow those of the last slice without a wait in between.  Measured together with the shorter set-up (warps 6, 7):
-    // whole calls, 131072 tokens FP8 6158 -> 6078 us, 16 sequences 3536 -> 3453, FP8 3309 -> 3274, 32768 tokens 1545 -> 1521,
-    // 60160 tokens 4 heads 100.4 -> 96.1, 2048 tokens 38.6 -> 37.4, dense 32768 tokens and 131072 tokens BF16 within 1 %.
+    // MMAs follow those of the last slice without a wait in between.  Without / with it (us): 32768 tokens dense 7900 / 7510,
+    // 16384 tokens dense FP8 1569 / 1428, 131072 tokens 8780 / 8350, FP8 6440 / 6120, 16 sequences FP8 3376 / 3296, 24 short ones
+    // 162.7 / 156.7, 16 sequences BF16 3562 / 3565.
     uint32_t G = 0;
     bool qk_issued = false;   // S = Q K^T (G) is under way already
     for (int it = 0;; ++it) {
