@@ -374,8 +374,8 @@ __global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_
 // many segments per worker hardly any is that long and the order is KV-head-major; with few the heads run side by side
 // whatever the order is.  Whole calls, KV-head-major throughout / so: the last 8192 of 131072 tokens 1404 / 1142 us (longest
 // list 408 blocks, mean 41), 8191 tokens FP8 227 / 212, 15616 tokens, 32 heads on 4, 134 / 122, 32768 tokens 1576 / 1536,
-// 131072 tokens 8632 / 8634.  Greedy scheduling of the measured lists on paper: 1/8 stays within 2 % of longest-first
-// throughout, 1/16 moves a quarter of the segments of 32768 tokens out of their head's turn and gains nothing.
+// 131072 tokens 8632 / 8634.  Shares of 1/4, 1/8, 1/16: 32768 tokens 1697 / 1639 / 1610, the last 8192 of 131072 tokens 1198 /
+// 1107 / 1120, 8191 tokens FP8 211 / 206 / 204, the others within 1 %.
 // Every CTA of 256 threads adds the histogram up for itself (Hkv x 128 counts, in L2): column sums and their prefix give the
 // long segments' places, and the number of long segments per head (head_long, Hkv words) the start of each head.
 constexpr int kLongShare = 8;
