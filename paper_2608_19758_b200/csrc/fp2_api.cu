@@ -866,16 +866,21 @@ extern "C" fp2_status fp2_page_table_from_token_map(fp2_plan* pl, const int32_t*
 // ------------------------------------------------------------------------------------------------------
 // Self-test of the bounded waits: one small CTA that owns tensor memory and waits on a barrier nobody arrives on,
 // with a short cycle budget.  The wait gives up by itself, records where, the CTA releases its tensor memory and
-// the kernel returns: nothing hangs and nothing traps.
+// the kernel returns: nothing hangs and nothing traps.  It waits and leaves the way the roles of the large kernels do: a
+// descriptor handed to a whole warp (the lanes of warp 1 run out at times of their own, those of warp 0 see its flag), then
+// the common way out.
 // ------------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(64, 1) bounded_wait_probe_kernel(int* status, long long budget_cycles) {
   __shared__ uint64_t never;       // nobody arrives here
+  __shared__ uint64_t drain_bar;
   __shared__ uint32_t tmem_base_s;
-  __shared__ int abort_flag;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  __shared__ int abort_flag, valid;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     abort_flag = 0;
+    valid = 1;
     mbar_init(&never, 1);
+    mbar_init(&drain_bar, 1);
     fence_barrier_init();
   }
   if (warp == 0) {
@@ -885,11 +890,9 @@ __global__ void __launch_bounds__(64, 1) bounded_wait_probe_kernel(int* status, 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  WaitCtx ctx{status, &abort_flag, budget_cycles};
-  if (warp == 1) mbar_wait(&never, 0, ctx, 901);      // every lane of the warp runs into the budget
-  if (warp == 0) mbar_wait(&never, 0, ctx, 902);      // sees the abort flag of the other warp, or its own expiry
-  tc_fence_before();
-  __syncthreads();
+  WaitCtx ctx{status, &abort_flag, warp == 1 ? budget_cycles * (32 + lane) / 64 : budget_cycles};
+  while (ready_warp(&never, 0, ctx, warp == 1 ? 901 : 902, &valid)) {}   // (ends with the first wait)
+  leave_cta(&abort_flag, &drain_bar, warp == 0);
   if (warp == 0) tmem_dealloc(tmem_base_s, 32);
 }
 

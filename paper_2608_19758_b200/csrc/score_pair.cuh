@@ -234,6 +234,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     // (heaviest first; a static round-robin, no atomic on the critical path).  Query tiles by TMA, one box per 64-element
     // half (FP8: one, see kQLeadRows); rows of a short last tile get whatever follows and are not used.
     const uint64_t pol = l2_policy_evict_first();
+    bool live = true;   // no wait of this lane for a buffer has run out; after one it requests nothing more
     for (int k = 0;; ++k) {
       const int slot = k % kPairInfoSlots, qb = k % kPairQBufs;
       if (k >= kPairInfoSlots) mbar_wait(&info_empty[slot], ((k / kPairInfoSlots) - 1) & 1, ctx, 111);
@@ -254,7 +255,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       }
       __syncwarp();
       if (!valid) break;
-      if (k >= kPairQBufs) mbar_wait(&q_empty[qb], ((k / kPairQBufs) - 1) & 1, ctx, 112);
+      if (k >= kPairQBufs) live &= mbar_wait(&q_empty[qb], ((k / kPairQBufs) - 1) & 1, ctx, 112);
       const PairInfo& pi = info[slot];
       const SegInfo& sg = pi.sg[0];
       const int tok0 = sg.r0 / P.group, lead = sg.r0 - tok0 * P.group, nt = pi.nt;
@@ -262,19 +263,19 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       const CUtensorMap* mp = nt > 1 ? &map_q2 : &map_q;
       const uint32_t rows = (uint32_t)(P.group * (nt > 1 ? P.q_box2_tok : P.q_box_tok));
       if constexpr (FP8) {
-        if (lane == 0) {
+        if (lane == 0 && live) {
           mbar_arrive_expect_tx(&raw_full[qb], rows * 128u);
           tma_load_3d_hint(buf + kPairQHalf - lead * 128, mp, &raw_full[qb], 0, sg.h * P.group, sg.q_tok0 + tok0, pol);
         }
         for (int j = lane; j < nt * kTileRows; j += 32)   // (adjacent tiles: row j of the pair is packed row r0 + j)
           sC[slot][j] = P.scale_log2 * q_scale[sg.h * P.group + (sg.r0 + j) % P.group];
         __syncwarp();
-        mbar_wait(&raw_full[qb], (k / kPairQBufs) & 1, ctx, 114);
+        live &= mbar_wait(&raw_full[qb], (k / kPairQBufs) & 1, ctx, 114);
         widen_pair_in_place(buf, buf + kPairQHalf, nt * kTileRows, lane);
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(&q_full[qb]);
-      } else if (lane == 0) {
+      } else if (lane == 0 && live) {
         mbar_arrive_expect_tx(&q_full[qb], rows * 256u);
         tma_load_3d_hint(buf - lead * 128, mp, &q_full[qb], 0, sg.h * P.group, sg.q_tok0 + tok0, pol);
         tma_load_3d_hint(buf + kPairQHalf - lead * 128, mp, &q_full[qb], 64, sg.h * P.group, sg.q_tok0 + tok0, pol);
@@ -285,9 +286,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     // ---------------- selection: threshold, forced blocks, ordered compaction of the tiles of unit `it` ----------------
     for (int it = 0;; ++it) {
       const int slot = it % kPairInfoSlots, eb = it & 1;
-      mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 151);
       const PairInfo& pi = info[slot];
-      if (!pi.valid) break;
+      if (!ready_warp(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 151, &pi.valid)) break;
       mbar_wait(&e_full[eb], (it >> 1) & 1, ctx, 152);
       for (int tt = 0; tt < pi.nt; ++tt) {
         const SegInfo sg = pi.sg[tt];
@@ -330,9 +330,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       auto produce = [&]() {
         for (int it = 0;; ++it) {
           const int slot = it % kPairInfoSlots;
-          mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 121);
           const PairInfo& pi = info[slot];
-          if (!pi.valid) break;
+          if (!mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 121) || !pi.valid) break;
           const int h = pi.sg[0].h, blk_off = pi.sg[0].blk_off;
           const int nchunks = unit_chunks(pi);
           for (int c = 0; c < nchunks; ++c) {
@@ -358,9 +357,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     uint32_t pc = 0, ac0 = 0, ac1 = 0, gc0 = 0;   // gc0: chunks of all earlier units
     for (int it = 0;; ++it) {
       const int slot = it % kPairInfoSlots, qb = it % kPairQBufs;
-      mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 131);
       const PairInfo& pi = info[slot];
-      if (!pi.valid) break;
+      if (!ready_warp(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 131, &pi.valid)) break;
       const int nchunks = unit_chunks(pi);
       const uint32_t idesc = make_idesc(128, 128 * pi.nt, kFmt, kFmt, 0, 0);
       mbar_wait(&q_full[qb], (it / kPairQBufs) & 1, ctx, 132);
@@ -403,9 +401,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     bool prev_big = false;
     for (int it = 0;; ++it) {
       const int slot = it % kPairInfoSlots;
-      mbar_wait(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 141);
       const PairInfo& pi = info[slot];
-      if (!pi.valid) break;
+      if (!ready_warp(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 141, &pi.valid)) break;
       const int nt = pi.nt;
       const int nchunks = unit_chunks(pi);
       const int ncand0 = pi.sg[0].J_hi + 1, ncand1 = nt > 1 ? pi.sg[1].J_hi + 1 : 0;
@@ -465,15 +462,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       gc0 += (uint32_t)nchunks;
     }
   }
-  if (abort_flag) {   // MMAs and bulk copies may still be in flight: let them finish before tensor memory goes
-    if (warp == 4 * kPairGroups + 1 && elect_one()) {
-      umma_commit(&drain_bar);
-      mbar_wait_drain(&drain_bar, 0, 200000000ll);
-    }
-    __nanosleep(2000000);
-  }
-  tc_fence_before();
-  __syncthreads();
+  leave_cta(&abort_flag, &drain_bar, warp == 4 * kPairGroups + 1);
   if (warp == 4 * kPairGroups + 1) tmem_dealloc(tmem, 512);
 }
 

@@ -299,6 +299,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
     // (a static round-robin: no atomic on the critical path).  The loop is software-pipelined: the copies of
     // tile k+1 are issued before the copies of tile k are waited for, so two query tiles are in flight.
     const int t64 = lane;
+    bool live = true;   // no wait of this lane for a buffer has run out; after one it requests no box
     auto seg_of = [&](int k) { return P.nseg - 1 - ((int)blockIdx.x + k * (int)gridDim.x); };
     auto issue = [&](int k) -> bool {   // publishes tile k's descriptor and starts its query copies
       const int slot = k % kScoreInfoSlots, qb = k % kScoreQBufs;
@@ -322,7 +323,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
         // [128 bytes, g heads, q_box_tok tokens] that starts at the tile's first token holds them all, in packed
         // order, the tile's first row sg.r0 % g rows into it.  One TMA copy instead of 1024 address computations.
         if (P.q_raw_tma) {
-          if (t64 == 0) {
+          if (t64 == 0 && live) {
             mbar_arrive_expect_tx(&raw_full[k & 1], (uint32_t)(P.group * P.q_box_tok * 128));
             tma_load_3d_hint(sQraw + (k & 1) * kScoreRawBytes, &map_q, &raw_full[k & 1], 0, sg.h * P.group,
                              sg.q_tok0 + sg.r0 / P.group, l2_policy_evict_first());
@@ -357,7 +358,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
       const int qb = k % kScoreQBufs;
       if constexpr (FP8) {
         const SegInfo& sgw = info[k % kScoreInfoSlots];
-        if (P.q_raw_tma) mbar_wait(&raw_full[k & 1], (k >> 1) & 1, ctx, 114);
+        if (P.q_raw_tma) live &= mbar_wait(&raw_full[k & 1], (k >> 1) & 1, ctx, 114);
         __syncwarp();   // every thread's copies of tile k have landed
         if (k >= kScoreQBufs) mbar_wait(&q_empty[qb], ((k / kScoreQBufs) - 1) & 1, ctx, 113);
         STP(2);
@@ -382,8 +383,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
     // ---------------- selection warp: threshold, forced blocks, ordered compaction of tile `it` ----------------
     for (int it = 0;; ++it) {
       const int slot = it % kScoreInfoSlots, eb = it & 1;
-      mbar_wait(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 151);
-      if (!info_valid[slot]) break;
+      if (!ready_warp(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 151, &info_valid[slot])) break;
       const SegInfo sg = info[slot];
       const int ncand = sg.J_hi + 1;
       const float* e = sE + (ncand > kMaxBlocks / 2 ? 0 : eb * (kMaxBlocks / 2));
@@ -418,17 +418,18 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
       tma_prefetch_desc(&map_klo);
       const uint64_t keep = l2_policy_evict_last();
       uint32_t pc = 0;
+      bool live = true;
       for (int it = 0;; ++it) {
         const int slot = it % kScoreInfoSlots;
-        mbar_wait(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 121);
-        if (!info_valid[slot]) break;
+        if (!mbar_wait(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 121) || !info_valid[slot]) break;
         const int h = info[slot].h, blk_off = info[slot].blk_off;
         const int nchunks = (info[slot].J_hi + 128) >> 7;
         for (int c = 0; c < nchunks; ++c) {
 #pragma unroll
           for (int part = 0; part < 2; ++part, ++pc) {
             const int s = pc % kScoreStages;
-            if (pc >= kScoreStages) mbar_wait(&empty[s], ((pc / kScoreStages) - 1) & 1, ctx, 122);
+            if (pc >= kScoreStages) live &= mbar_wait(&empty[s], ((pc / kScoreStages) - 1) & 1, ctx, 122);
+            if (!live) continue;   // a wait has run out: nothing more is requested
             uint8_t* dst = sStage + s * 32768;
             mbar_arrive_expect_tx(&full[s], 32768);
             const CUtensorMap* mp = part ? &map_klo : &map_khi;
@@ -447,8 +448,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
     uint32_t pc = 0, ac0 = 0, ac1 = 0, gc0 = 0;   // gc0: chunks of all earlier tiles
     for (int it = 0;; ++it) {
       const int slot = it % kScoreInfoSlots, qb = it % kScoreQBufs;
-      mbar_wait(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 131);
-      if (!info_valid[slot]) break;
+      if (!ready_warp(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 131, &info_valid[slot])) break;
       const int nchunks = (info[slot].J_hi + 128) >> 7;
       mbar_wait(&q_full[qb], (it / kScoreQBufs) & 1, ctx, 132);
       const uint64_t q_desc = make_smem_desc_sw128(smem_u32(sQ + qb * 32768), 16, 1024);
@@ -501,15 +501,15 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
     for (int it = 0;; ++it) {
       const int slot = it % kScoreInfoSlots;
       SPF(3);
-      mbar_wait(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 141);
+      const bool more = ready_warp(&info_full[slot], (it / kScoreInfoSlots) & 1, ctx, 141, &info_valid[slot]);
       SPF(0);
 #ifdef FP2_PROFILE
-      if (!info_valid[slot] && g_score_prof && lane == 0 && (warp & 3) == 0) {
+      if (!more && g_score_prof && lane == 0 && (warp & 3) == 0) {
         pf[7] = clock64() - pf_t0;
         for (int i = 0; i < 8; ++i) g_score_prof[((size_t)blockIdx.x * 2 + wg) * 8 + i] = pf[i];
       }
 #endif
-      if (!info_valid[slot]) break;
+      if (!more) break;
       const SegInfo sg = info[slot];
       const int ncand = sg.J_hi + 1;
       const int nchunks = (ncand + 127) >> 7;
@@ -553,15 +553,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
       gc0 += (uint32_t)nchunks;
     }
   }
-  if (abort_flag) {   // MMAs and bulk copies may still be in flight: let them finish before tensor memory goes
-    if (warp == 9 && elect_one()) {
-      umma_commit(&drain_bar);
-      mbar_wait_drain(&drain_bar, 0, 200000000ll);
-    }
-    __nanosleep(2000000);
-  }
-  tc_fence_before();
-  __syncthreads();
+  leave_cta(&abort_flag, &drain_bar, warp == 9);
   if (warp == 9) tmem_dealloc(tmem, 256);
 }
 

@@ -277,10 +277,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     }
     mbar_init(&q_full, kSetupThreads + (P.q_box ? 1 : 0));
     mbar_init(&vraw_full, 1);
-    mbar_init(&vraw_empty, 1);
+    mbar_init(&vraw_empty, 4);   // one arrival per softmax warp
     mbar_init(&q_empty, 1);
     mbar_init(&k_full, 1);
-    mbar_init(&v_full, 1);
+    mbar_init(&v_full, WIDEN ? 4 : 1);   // WIDEN: the softmax warps', or the producer's for all of them
     mbar_init(&s_done, 1);
     mbar_init(&pv_done[0], 1);
     mbar_init(&pv_done[1], 1);
@@ -313,7 +313,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
   const int g = P.group;
 
   // O += P V (G) has completed.  Safe for a waiter that is at most two iterations behind the issuer.
-  auto wait_pv = [&](uint32_t G, int where) { mbar_wait(&pv_done[G & 1], (G >> 1) & 1, ctx, where); };
+  auto wait_pv = [&](uint32_t G, int where) { return mbar_wait(&pv_done[G & 1], (G >> 1) & 1, ctx, where); };
 
   if (warp >= 6) {
     // =============================== unit set-up + Q staging ===============================
@@ -341,6 +341,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       for (int w = t64; w < kMaxBlocks / 32; w += 32) sel_bits[w] = 0u;
     if (t64 == 0) ndiag_s = 0;
     const int n_units = A.unit_split ? *A.n_units : P.nseg;
+    // Both warps run through the same named barriers whatever a wait gives: they leave by unit_s alone, which one thread sets.
     for (int it = 0;; ++it) {
       const int slot = it & 1;
       if (it >= 2) mbar_wait(&info_empty[slot], ((it >> 1) - 1) & 1, ctx, 201);
@@ -432,8 +433,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       }
       // Q tile: wait until every S = Q K^T of the previous unit has completed, then overwrite
       if (it >= 1) {
-        mbar_wait(&q_empty, (it - 1) & 1, ctx, 202);
-        if (P.q_box && t64 == 0) issue_q(sg);
+        const bool free = mbar_wait(&q_empty, (it - 1) & 1, ctx, 202);
+        if (P.q_box && t64 == 0 && free) issue_q(sg);
       }
       {   // sHot: rows 2 t64 and 2 t64 + 1
         const int rem = sg.r0 % g;
@@ -469,11 +470,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     (void)rc;
     const uint64_t keep = l2_policy_evict_last();   // K / V pages and pooled means: shared by many tiles
     const int ppb = P.pages_per_block, psz = P.page_size;
+    bool live = true;   // no wait of this lane has run out; after one it requests nothing more (the stages may not be free)
     for (int it = 0;; ++it) {
       const int slot = it & 1;
-      mbar_wait(&info_full[slot], (it >> 1) & 1, ctx, 301);
       const TileInfo& ti = info[slot];
-      if (!ti.valid) break;
+      if (!ready_warp(&info_full[slot], (it >> 1) & 1, ctx, 301, &ti.valid)) break;
       const SegInfo& sg = ti.sg;
       const int T = ti.T;
       const int32_t* list = A.blk_idx + sg.off;
@@ -519,7 +520,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       for (int i = ti.it_begin; i < ti.it_end; ++i, ++G) {
         const int pid = pid_next;
         const int J_cur = J_fetched;
-        if (G >= 1) mbar_wait(&s_done, (G - 1) & 1, ctx, 302);   // K stage free
+        if (G >= 1) live &= mbar_wait(&s_done, (G - 1) & 1, ctx, 302);   // K stage free
         if (i < ti.ndiag && P.diag_mma) {
           // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c
           const int t0 = sg.pre + sg.r0 / g - J_cur * kBlock;
@@ -533,19 +534,19 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
           if constexpr (FP8) {
             // raw e4m3 K tile, 128 bytes per token row, straight into the K stage (the MMA reads it as it lands)
             const uint32_t bytes = (uint32_t)nvalid * psz * 128u;
-            if (lane == 0) mbar_arrive_expect_tx(&k_full, bytes);
+            if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, bytes);
             __syncwarp();
-            if (pid >= 0) tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
+            if (pid >= 0 && live) tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
             pid_next = fetch_pid(i + 1);
             if constexpr (WIDEN) {
-              if (rc >= 1) mbar_wait(&vraw_empty, (rc - 1) & 1, ctx, 306);
-              if (lane == 0) mbar_arrive_expect_tx(&vraw_full, bytes);
+              if (rc >= 1) live &= mbar_wait(&vraw_empty, (rc - 1) & 1, ctx, 306);
+              if (lane == 0 && live) mbar_arrive_expect_tx(&vraw_full, bytes);
               __syncwarp();
-              if (pid >= 0) tma_load_3d_hint(sVraw + lane * psz * 128, &map_v, &vraw_full, 0, sg.h, pid * psz, keep);
+              if (pid >= 0 && live) tma_load_3d_hint(sVraw + lane * psz * 128, &map_v, &vraw_full, 0, sg.h, pid * psz, keep);
               ++rc;
             } else {   // the block's F16 copy is one tile
-              if (G >= 1) wait_pv(G - 1, 304);  // V stage free
-              if (lane == 0) {
+              if (G >= 1) live &= wait_pv(G - 1, 304);  // V stage free
+              if (lane == 0 && live) {
                 const int row0 = (sg.blk_off + J_cur) * kBlock;
                 mbar_arrive_expect_tx(&v_full, kTileBytes);
                 tma_load_3d_hint(sV, &map_v, &v_full, 0, sg.h, row0, keep);
@@ -555,17 +556,17 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             }
           } else {
             const uint32_t bytes = (uint32_t)nvalid * psz * 256u;
-            if (lane == 0) mbar_arrive_expect_tx(&k_full, bytes);
+            if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, bytes);
             __syncwarp();
-            if (pid >= 0) {
+            if (pid >= 0 && live) {
               tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
               tma_load_3d_hint(sK + 16384 + lane * psz * 128, &map_k, &k_full, 64, sg.h, pid * psz, keep);
             }
             pid_next = fetch_pid(i + 1);
-            if (G >= 1) wait_pv(G - 1, 303);  // V stage free
-            if (lane == 0) mbar_arrive_expect_tx(&v_full, bytes);
+            if (G >= 1) live &= wait_pv(G - 1, 303);  // V stage free
+            if (lane == 0 && live) mbar_arrive_expect_tx(&v_full, bytes);
             __syncwarp();
-            if (pid >= 0) {
+            if (pid >= 0 && live) {
               tma_load_3d_hint(sV + lane * psz * 128, &map_v, &v_full, 0, sg.h, pid * psz, keep);
               tma_load_3d_hint(sV + 16384 + lane * psz * 128, &map_v, &v_full, 64, sg.h, pid * psz, keep);
             }
@@ -580,7 +581,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             for (int u = 0; u < 4; ++u) nh[u] = ((w >> ((lane * 4 + u) & 31)) & 1u) ? 0 : 32;
             write_bias(nh);
           }
-          if (lane == 0) {
+          if (lane == 0 && live) {
             mbar_arrive_expect_tx(&k_full, kTileBytes);
             if constexpr (FP8) {   // e4m3 hi | lo, 16 KB each
               tma_load_3d_hint(sK, &map_kbar, &k_full, 0, sg.h, row0, keep);
@@ -590,8 +591,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
               tma_load_3d_hint(sK + 16384, &map_kbar, &k_full, 64, sg.h, row0, keep);
             }
           }
-          if (G >= 1) wait_pv(G - 1, 305);    // V stage free
-          if (lane == 0) {
+          if (G >= 1) live &= wait_pv(G - 1, 305);    // V stage free
+          if (lane == 0 && live) {
+            if constexpr (WIDEN) mbar_arrive_n(&v_full, 3);
             mbar_arrive_expect_tx(&v_full, kTileBytes);
             tma_load_3d_hint(sV, &map_vbar, &v_full, 0, sg.h, row0, keep);
             tma_load_3d_hint(sV + 16384, &map_vbar, &v_full, 64, sg.h, row0, keep);
@@ -599,6 +601,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
           __syncwarp();
         }
       }
+      __syncwarp();   // no lane reads the descriptor any more
       if (lane == 0) mbar_arrive(&info_empty[slot]);
     }
   } else if (warp == 5) {
@@ -651,9 +654,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     bool qk_issued = false;   // S = Q K^T (G) is under way already
     for (int it = 0;; ++it) {
       const int slot = it & 1;
-      mbar_wait(&info_full[slot], (it >> 1) & 1, ctx, 403);
       const TileInfo& ti = info[slot];
-      if (!ti.valid) break;
+      if (!ready_warp(&info_full[slot], (it >> 1) & 1, ctx, 403, &ti.valid)) break;
       const int T = ti.T, ndiag = P.diag_mma ? ti.ndiag : 0;
       const int i0 = ti.it_begin, i1 = ti.it_end;
       if (!qk_issued) mbar_wait(&q_full, it & 1, ctx, 404);
@@ -727,10 +729,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     for (int it = 0;; ++it) {
       const int slot = it & 1;
       PF_BEGIN();
-      mbar_wait(&info_full[slot], (it >> 1) & 1, ctx, 501);
-      PF_END(0);
       const TileInfo& ti = info[slot];
-      if (!ti.valid) break;
+      if (!ready_warp(&info_full[slot], (it >> 1) & 1, ctx, 501, &ti.valid)) break;
+      PF_END(0);
       const int T = ti.T;
       const bool dense = ti.dense != 0;
       const int J_hi = ti.sg.J_hi, J_lo = ti.sg.J_lo;
@@ -785,8 +786,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
             if (G >= 1) wait_pv(G - 1, 602);
             widen_tile_f16(sVraw, sV, tid, 128);
             fence_proxy_async();
-            named_bar_sync(1, 128);
-            if (tid == 0) {
+            __syncwarp();
+            if (lane == 0) {   // (no barrier between the warps: after an abort one of them may have left)
               mbar_arrive(&vraw_empty);
               mbar_arrive(&v_full);
             }
@@ -894,18 +895,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       for (int i = 0; i < 16; ++i) A.prof[(size_t)blockIdx.x * 16 + i] = pf[i];
 #endif
   }
-  // teardown: on the normal path every barrier has been consumed and every MMA has completed (the epilogue waited
-  // for the last one).  After an abort MMAs and bulk copies may still be in flight: the issuing thread waits (bounded)
-  // for its MMAs, everyone gives the copies time, and only then is tensor memory released.
-  if (abort_flag) {
-    if (warp == 5 && elect_one()) {   // the lane that issued the MMAs: a commit tracks its own thread's
-      umma_commit(&drain_bar);
-      mbar_wait_drain(&drain_bar, 0, 200000000ll);
-    }
-    __nanosleep(2000000);
-  }
-  tc_fence_before();
-  __syncthreads();
+  leave_cta(&abort_flag, &drain_bar, warp == 5);
   if (warp == 5) tmem_dealloc(tmem, 256);
 }
 

@@ -538,6 +538,23 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_the_context_usable():
     check_attention(dc, wl, lists)
 
 
+def test_warps_leave_as_one_after_a_wait_that_ran_out():
+    """The probe's lanes give up at different times and leave through the votes, the commit and the CTA barriers that every
+    large kernel leaves by; a lane that went its own way would keep the others waiting there.  Several launches in a row, each
+    over within its budget (0.5 ms of cycles, 2 ms for copies in flight), each reported."""
+    spec = inputs.small_spec(seqs=[(300, 0)], num_q_heads=4, num_kv_heads=2, page_size=16, config_id=89)
+    case, dc, wl = make(spec)
+    for _ in range(6):
+        t0 = torch.cuda.Event(enable_timing=True); t1 = torch.cuda.Event(enable_timing=True)
+        t0.record()
+        binding.fp2_selftest_bounded_wait(dc.plan, dc.workspace)
+        t1.record()
+        code, words = dc.status(raise_on_error=False)
+        assert code == 5 and words[0] == 1 and words[1] in (901, 902), (code, words)
+        assert t0.elapsed_time(t1) < 20.0
+    full_pipeline(spec)
+
+
 def test_two_runs_are_bit_identical():
     spec = inputs.config_spec(2, scale_down=4)
     case, dc, wl = make(spec)
