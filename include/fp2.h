@@ -23,6 +23,8 @@
  *       q_scale [num_q_heads], k_scale / v_scale [num_kv_heads]  fp32 de-quantisation scales, FP8 only
  *                     (NULL for BF16); per-tensor scaling (Eq. 15) is the case of equal entries
  *       lse           fp32 [num_q_heads, total_q], natural log of the softmax denominator (may be NULL)
+ *     Alignment: q, k_cache and v_cache 16 bytes, out 32 bytes (rows are stored in pieces of that size), workspace 1024;
+ *     anything less is refused with FP2_ERR_INVALID_ARG.
  *     Query i of sequence b sits at absolute position (seqlens_k[b] - Lq_b) + i: the causal mask is aligned
  *     to the end of the KV sequence, so cached prefixes (chunked prefill) are visible to every new token.
  *   - Segments.  With g = num_q_heads / num_kv_heads, packed row r of a KV head's query matrix is position

@@ -425,6 +425,9 @@ static fp2_status set_attrs(fp2_plan* pl) {
 
 static bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
+// The attention kernel stores rows of `out` in pieces of 32 bytes (st_global_v8), which fault on anything less aligned.
+static bool out_ok(const fp2_plan* pl, const void* out) { return out && aligned(out, pl && pl->nseg > 0 ? 32 : 16); }
+
 static fp2_status check_common(fp2_plan* pl, const void* q, const void* k, const void* v, const int32_t* pt,
                                const int32_t* cu, const int32_t* lk, const float* qs, const float* ks,
                                const float* vs, const void* ws) {
@@ -559,9 +562,9 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
                                 const int32_t* cu, const int32_t* lk, const int32_t* seg_count,
                                 const int32_t* blk_idx, const float* qs, const float* ks, const float* vs, void* out,
                                 float* lse, void* workspace, bool need_pool, fp2_stream stream) {
+  if (!out_ok(pl, out)) return FP2_ERR_INVALID_ARG;
   fp2_status s = check_common(pl, q, k, v, pt, cu, lk, qs, ks, vs, workspace);
   if (s != FP2_OK) return s;
-  if (!out || !aligned(out, 16)) return FP2_ERR_INVALID_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   pl->last_launches = 0;
@@ -703,8 +706,8 @@ extern "C" fp2_status fp2_dense_prefill_static(fp2_plan* pl, const void* q, cons
                                                const int32_t* pt, const int32_t* cu, const int32_t* lk,
                                                const float* qs, const float* ks, const float* vs, void* out,
                                                float* lse, fp2_stream stream) {
-  if (!pl || !q || !k || !v || !pt || !cu || !lk || !out) return FP2_ERR_INVALID_ARG;
-  if (!aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16) || !aligned(out, 16)) return FP2_ERR_INVALID_ARG;
+  if (!pl || !q || !k || !v || !pt || !cu || !lk || !out_ok(pl, out)) return FP2_ERR_INVALID_ARG;
+  if (!aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16)) return FP2_ERR_INVALID_ARG;
   if (pl->device < 0) return FP2_ERR_CUDA;
   if (pl->dev.fp8 && (!qs || !ks || !vs)) return FP2_ERR_INVALID_ARG;
   if (pl->nseg > kStaticMaxSegments || pl->prm.num_kv_heads > kStaticMaxKvHeads) return FP2_ERR_CAPACITY;

@@ -110,6 +110,23 @@ def test_stage_calls_fail_loudly_without_a_device():
     plan.close()
 
 
+@pytest.mark.parametrize("offset,code", [(16, 1), (48, 1), (8, 1), (32, 4), (0, 4)])
+def test_outputs_need_32_byte_alignment(offset, code):
+    """Rows of the output are stored in pieces of 32 bytes: a pointer that is only 16-byte aligned is refused by every attention
+    entry point before anything else is looked at, so it never reaches a kernel.  Others go on to FP2_ERR_CUDA.  (Not with a
+    device: the pointers are made up.)"""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("a device is present")
+    plan = binding.Plan(base_params(), [0, 300], [400])
+    lib = binding.load()
+    p, out = C.c_void_p(1024), C.c_void_p(4096 + offset)
+    assert lib.fp2_dense_prefill(plan.handle, p, p, p, p, p, p, None, None, None, out, None, p, None) == code
+    assert lib.fp2_dense_prefill_static(plan.handle, p, p, p, p, p, p, None, None, None, out, None, None) == code
+    assert lib.fp2_sparse_prefill(plan.handle, p, p, p, p, p, p, p, p, p, None, None, None, out, None, p, 1, None) == code
+    plan.close()
+
+
 def test_pool_carry_count_is_host_only_and_counts_complete_blocks():
     """Blocks carried between chunks = blocks complete in both (floor(min(Lk) / 128)); needs no device."""
     from paper_2608_19758_b200 import binding
