@@ -45,7 +45,7 @@ __device__ __forceinline__ void accum16(const uint4& v, float* acc) {
 
 // One pooled mean -> the operand formats the scorer and the correction chunks read (see the head of the file).
 template <bool FP8>
-__device__ __forceinline__ void write_pooled(int which, float mean, size_t o, int h, const float* __restrict__ k_scale,
+__device__ __forceinline__ void write_pooled(int which, float mean, size_t o, int h, const float* k_scale,
                                              __nv_bfloat16* __restrict__ kbar_hi, __nv_bfloat16* __restrict__ kbar_lo,
                                              __nv_bfloat16* __restrict__ vbar, uint8_t* __restrict__ kbar8_hi,
                                              uint8_t* __restrict__ kbar8_lo) {
@@ -81,13 +81,13 @@ __device__ __forceinline__ void write_pooled(int which, float mean, size_t o, in
 // 128 token rows of 256 B (BF16) / 128 B (FP8).  256 threads, every load of a thread issued before the first
 // use; small enough in registers for four CTAs per SM, which is what hides the page-table -> data dependency.
 template <bool FP8>
-__global__ void __launch_bounds__(256, 4) pool_kv_kernel(const uint8_t* __restrict__ k_cache,
-                                                         const uint8_t* __restrict__ v_cache,
+__global__ void __launch_bounds__(256, 4) pool_kv_kernel(const uint8_t* k_cache,
+                                                         const uint8_t* v_cache,
                                                          const int32_t* page_table,
                                                          const int32_t* __restrict__ plan_lk,  // [ns], the plan's copy
                                                          const int32_t* __restrict__ blk_off,  // [ns+1]
-                                                         const float* __restrict__ k_scale,
-                                                         const float* __restrict__ v_scale, DevParams P,
+                                                         const float* k_scale,
+                                                         const float* v_scale, DevParams P,
                                                          __nv_bfloat16* __restrict__ kbar_hi,
                                                          __nv_bfloat16* __restrict__ kbar_lo,
                                                          __nv_bfloat16* __restrict__ vbar,
@@ -171,13 +171,13 @@ __global__ void __launch_bounds__(256, 4) pool_kv_kernel(const uint8_t* __restri
 // of a token takes a shift and a mask (a division per load made the kernel ALU-bound: 143 -> 110 us at 128K).
 // Measured at 131072 tokens, 8 BF16 heads: 93 us for 537 MB = 5.8 TB/s; a bare streaming read reaches 6.8 TB/s.
 template <bool FP8>
-__global__ void __launch_bounds__(256, 4) pool_rows_kernel(const uint8_t* __restrict__ k_cache,
-                                                           const uint8_t* __restrict__ v_cache,
+__global__ void __launch_bounds__(256, 4) pool_rows_kernel(const uint8_t* k_cache,
+                                                           const uint8_t* v_cache,
                                                            const int32_t* page_table,
                                                            const int32_t* __restrict__ plan_lk,
                                                            const int32_t* __restrict__ blk_off,
-                                                           const float* __restrict__ k_scale,
-                                                           const float* __restrict__ v_scale, DevParams P,
+                                                           const float* k_scale,
+                                                           const float* v_scale, DevParams P,
                                                            __nv_bfloat16* __restrict__ kbar_hi,
                                                            __nv_bfloat16* __restrict__ kbar_lo,
                                                            __nv_bfloat16* __restrict__ vbar,
@@ -553,9 +553,9 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
 // sequence b.  grid (sequences, row groups of 8); a row of one array is Hkv x 128 elements.
 // ----------------------------------------------------------------------------------------
 __global__ void pool_carry_kernel(const int32_t* carry, int row_bytes16, int row_bytes8,
-                                  const uint8_t* __restrict__ s_khi, const uint8_t* __restrict__ s_klo,
-                                  const uint8_t* __restrict__ s_vbar, const uint8_t* __restrict__ s_k8hi,
-                                  const uint8_t* __restrict__ s_k8lo, uint8_t* __restrict__ d_khi,
+                                  const uint8_t* s_khi, const uint8_t* s_klo,
+                                  const uint8_t* s_vbar, const uint8_t* s_k8hi,
+                                  const uint8_t* s_k8lo, uint8_t* __restrict__ d_khi,
                                   uint8_t* __restrict__ d_klo, uint8_t* __restrict__ d_vbar,
                                   uint8_t* __restrict__ d_k8hi, uint8_t* __restrict__ d_k8lo) {
   pdl_trigger();

@@ -116,8 +116,10 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t* bar, uint32_t parity, 
 // Programmatic dependent launch: every kernel of a stage call may be started while its predecessor drains.  It then sets
 // itself up (barriers, tensor memory) and waits here before it touches global memory; the wait ends when the predecessor has
 // completed, so a chain of kernels is ordered as if each had been launched after the other.  pdl_trigger lets the successor
-// start as early as it finds room.  Arrays that an earlier kernel may have written are not declared const __restrict__: such
-// loads count as invariant, and the compiler may move them in front of the wait.
+// start as early as it finds room.  Arrays that an earlier kernel may have written -- of this library or of the caller, whose own
+// kernels may let their dependents start early too -- are not declared const __restrict__: such loads count as invariant, and
+// the compiler may move them in front of the wait.  Only the plan's tables are.  (__ldg counts the same way: it is used on the
+// caches, at addresses that come from page ids loaded behind the wait.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -43,7 +43,7 @@ constexpr int kScoreSmemBytes = 1024 /*align*/ + kScoreQSlots * 32768 + kScoreSt
 // BF16: two 64-column halves of [128 rows x 128 B]; FP8 is widened to BF16 on the way (exact).
 // Rows >= nrows are zero-filled.  Called by `nthr` threads with local index `t`.
 template <bool FP8, int BATCH = 8>
-__device__ __forceinline__ void load_q_tile_bf16(uint8_t* sQ, const uint8_t* __restrict__ q, const SegInfo& sg,
+__device__ __forceinline__ void load_q_tile_bf16(uint8_t* sQ, const uint8_t* q, const SegInfo& sg,
                                                  const DevParams& P, int t, int nthr) {
   const int g = P.group;
   for (int i0 = t; i0 < kTileRows * 16; i0 += nthr * BATCH) {
@@ -120,7 +120,7 @@ __device__ __forceinline__ void widen_tile_f16(const uint8_t* __restrict__ raw, 
 }
 
 // Raw FP8 query tile -> shared memory with cp.async in the layout widen_tile_f16 reads (128-byte rows, swizzled).
-__device__ __forceinline__ void load_q_raw_async(uint8_t* sRaw, const uint8_t* __restrict__ q, const SegInfo& sg,
+__device__ __forceinline__ void load_q_raw_async(uint8_t* sRaw, const uint8_t* q, const SegInfo& sg,
                                                  const DevParams& P, int t, int nthr) {
   const int g = P.group;
   const uint32_t base = smem_u32(sRaw);
@@ -200,7 +200,7 @@ __device__ __forceinline__ void score_chunk(uint32_t lane_addr, float cs, const 
 // per ~12 us).  Same layout and zero fill as load_q_tile_bf16; with `wait` it returns after the copies have landed,
 // otherwise the caller closes a cp.async group and waits for it later.
 template <int HALF = 16384>   // bytes from one 64-element half of the tile to the other
-__device__ __forceinline__ void load_q_tile_async(uint8_t* sQ, const uint8_t* __restrict__ q, const SegInfo& sg,
+__device__ __forceinline__ void load_q_tile_async(uint8_t* sQ, const uint8_t* q, const SegInfo& sg,
                                                   const DevParams& P, int t, int nthr, bool wait = true) {
   const int g = P.group;
   const uint32_t base = smem_u32(sQ);
@@ -224,7 +224,7 @@ __device__ __forceinline__ void load_q_tile_async(uint8_t* sQ, const uint8_t* __
 template <bool FP8>
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_constant__ CUtensorMap map_klo,
-                    const __grid_constant__ CUtensorMap map_q, const uint8_t* __restrict__ q, const SegInfo* __restrict__ segs, const float* __restrict__ q_scale,
+                    const __grid_constant__ CUtensorMap map_q, const uint8_t* q, const SegInfo* __restrict__ segs, const float* q_scale,
                     DevParams P, int64_t* __restrict__ seg_offset, int32_t* __restrict__ seg_count,
                     int32_t* __restrict__ blk_idx, int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];

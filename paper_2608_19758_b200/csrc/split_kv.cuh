@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(128)
 split_combine_kernel(const SegInfo* __restrict__ segs, const int32_t* seg_split,
                      const int32_t* split_list, const int32_t* n_split,
                      const float* part_o, const float2* part_ml,
-                     const float* __restrict__ v_scale, DevParams P, __nv_bfloat16* __restrict__ out,
+                     const float* v_scale, DevParams P, __nv_bfloat16* __restrict__ out,
                      float* __restrict__ lse) {
   pdl_trigger();
   pdl_wait();

@@ -127,6 +127,22 @@ def test_outputs_need_32_byte_alignment(offset, code):
     plan.close()
 
 
+def test_only_the_plans_tables_are_declared_invariant():
+    """Kernels start before their predecessor has ended (programmatic dependent launch).  A pointer to const with __restrict__ says
+    that nobody writes the array, and the compiler may then load from it in front of the wait: true for the plan's tables, not
+    for what a caller's or another kernel may just have written."""
+    tables = {"segs", "units", "plan_lk", "blk_off"}
+    csrc = os.path.join(ROOT, "paper_2608_19758_b200", "csrc")
+    seen = 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for m in re.finditer(r"__global__\s[^{;]*?\(([^{;]*)\)\s*\{", text, flags=re.S):
+            seen += 1
+            for ident in re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", m.group(1)):
+                assert ident in tables, f"{name}: {ident}"
+    assert seen >= 14
+
+
 def test_pool_carry_count_is_host_only_and_counts_complete_blocks():
     """Blocks carried between chunks = blocks complete in both (floor(min(Lk) / 128)); needs no device."""
     from paper_2608_19758_b200 import binding
