@@ -187,21 +187,22 @@ fp2_status fp2_pool_carry(fp2_plan* dst, void* dst_workspace, const fp2_plan* sr
 fp2_status fp2_pool_carry_count(const fp2_plan* dst, const fp2_plan* src, const int32_t* h_src_seq,
                                 int32_t* h_blocks);
 
-/* KV splitting (Eq. 18; Sec. 3.3 "Sparsity-Aware Load Balancing"), off by default.  Plans with few segments
+/* KV splitting (Eq. 18; Sec. 3.3 "Sparsity-Aware Load Balancing") on request, off by default.  Plans with few segments
  * (fewer than four per worker CTA of the attention kernel) can cut the iteration sequence of a heavy segment --
  * its list backwards, then its correction chunks -- into up to 16 contiguous parts of about equal count, run the
  * parts as separate work units and merge their partial results by log-sum-exp weights; fp2_sparse_prefill and
  * fp2_dense_prefill then enqueue two more kernels (the device-side split plan and the merge).  The result is the
  * same up to rounding.
- *   target < 0 (default): never split;  0: automatic, parts of about the mean load per worker and at least 12
+ *   target < 0 (default): no splitting on request;  0: automatic, parts of about the mean load per worker and at least 12
  *   iterations;  > 0: parts of about `target` iterations (never more than nseg + 2 workers parts in all, which
  *   is what the workspace is sized for).
  * Larger plans are never split and ignore the setting; so do calls in which no segment could yield two parts.
  * On B200 the split did not pay in any case measured (the attention kernel already keeps two independent CTAs per
  * SM, and the two extra launches cost ~10 us), hence the default.  Host-side, takes effect at the next stage call.
- * With the default, calls of plans with few segments (under 16 per worker CTA) and long sequences (candidate ranges of 512
- * blocks and more) still cut segments that are longer than the mean load per worker, and merge their parts in one more
- * kernel: such a segment would be all that the call waits for at its end. */
+ * Independently of the setting, calls that are not split on request, of plans with few segments (under 16 per worker CTA) and
+ * long sequences (candidate ranges of 512 blocks and more), cut segments that are longer than the mean load per worker and
+ * merge their parts in one more kernel: such a segment would be all that the call waits for at its end.  Same result up to
+ * rounding, and the same in every run. */
 fp2_status fp2_plan_set_split(fp2_plan* plan, int32_t target);
 
 /* Index export (Algorithm 1 line 5; Sec. 3.3 "Index-Driven Sparse Traversal", Eq. 17).  Turns the padded lists

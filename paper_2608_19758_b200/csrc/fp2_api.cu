@@ -571,9 +571,14 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
   if (pl->nseg == 0) return FP2_OK;
   if (need_pool && (s = launch_pool(pl, k, v, pt, ks, vs, ws, st)) != FP2_OK) return s;
   const bool use_v16 = pl->dev.fp8 && (seg_count ? pl->likely_iters : pl->idx_capacity) >= pl->v16_iters;
+  // Splitting on request (Eq. 18): a part is never shorter than kMinPartLen iterations (or the requested length), so there is
+  // nothing to split when even the longest candidate range (plus its correction chunks) is below one and a half such parts.
+  // Calls that do not split cut their longest segments where the plan allows it, whatever the setting.
+  const int min_len = pl->split_target > 0 ? pl->split_target : kMinPartLen;
+  const bool split = pl->split_capable && pl->split_target >= 0 && 2 * (int64_t)pl->max_iters >= 3 * (int64_t)min_len;
   CutLists cut = {};
   int32_t* const counter = reinterpret_cast<int32_t*>(ws + pl->ws_counter);
-  if (pl->cut_slots > 0 && pl->split_target < 0) {
+  if (pl->cut_slots > 0 && !split) {
     cut.unit_split = reinterpret_cast<int32_t*>(ws + pl->ws_cut_split);
     cut.seg_split = cut.unit_split + pl->nseg + pl->cut_slots;
     cut.split_list = cut.seg_split + pl->nseg;
@@ -620,10 +625,6 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
 #ifdef FP2_PROFILE
   a.prof = g_prof_ptr;
 #endif
-  // a part is never shorter than kMinPartLen iterations (or the requested length): nothing to split when even the
-  // longest candidate range (plus its correction chunks) is below one and a half such parts
-  const int min_len = pl->split_target > 0 ? pl->split_target : kMinPartLen;
-  const bool split = pl->split_capable && pl->split_target >= 0 && 2 * pl->max_iters >= 3 * min_len;
   int64_t max_units = pl->nseg + cut.max_slots;
   if (split) {
     // device-side scheduler prep (Eq. 18): units = parts of segments, in the work order

@@ -70,6 +70,52 @@ def test_split_is_deterministic_and_equals_unsplit_within_rounding():
     assert torch.allclose(la, dc.lse, rtol=1e-5, atol=1e-5)
 
 
+@pytest.mark.parametrize("target", [0, 1, 100000])
+def test_a_split_request_that_does_not_apply_leaves_the_cutting_on(target):
+    """Plans of 4 to 16 segments per worker are never split on request, and a part of 100000 iterations fits nothing; such calls are
+    what they are by default: segments longer than a worker's share are cut, with the same launches and the same bits.  One
+    page for all tokens keeps the cache small."""
+    workers = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    n_seg = 4 * workers + 16 if target < 100000 else 40
+    hq, lk = 64, 520 * 128
+    lq = 2 * n_seg                                       # 64 heads on one: 2 tokens per tile
+    prm = dict(num_seqs=1, total_q=lq, num_q_heads=hq, num_kv_heads=1, head_dim=128, block_size=128, tile_rows=128,
+               page_size=128, num_pages=4, max_pages_per_seq=520, sink_tokens=256, window_tokens=512, use_correction=1,
+               alpha=0.1, softmax_scale=0.0, dtype=0)
+    plan = binding.Plan(prm, [0, lq], [lk])
+    assert plan.num_segments == n_seg
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v = (torch.randn(*s, 128, generator=g, device="cuda").to(torch.bfloat16)
+               for s in ((lq, hq), (4, 128, 1), (4, 128, 1)))
+    pt = (torch.arange(520, device="cuda") % 4).to(torch.int32)[None]
+    cu = torch.tensor([0, lq], dtype=torch.int32, device="cuda")
+    lk_t = torch.tensor([lk], dtype=torch.int32, device="cuda")
+    ws = plan.new_workspace()
+    off, cnt, idx = plan.new_lists()
+    binding.fp2_select_blocks(plan, q, k, v, pt, cu, lk_t, None, None, None, off, cnt, idx, ws)
+    # every 40th list complete: far above a worker's share
+    o, c, i = off.cpu(), cnt.cpu(), idx.cpu()
+    for s in range(n_seg):
+        d = plan.segment(s)
+        first = 0 if s % 40 == 7 else d["J_hi"] - 6
+        c[s] = d["J_hi"] + 1 - first
+        i[int(o[s]):int(o[s]) + int(c[s])] = torch.arange(first, d["J_hi"] + 1, dtype=torch.int32)
+    assert int(c.max()) >= 500 and int(c.max()) > int(c.sum()) / workers
+    cnt, idx = c.cuda(), i.cuda()
+
+    def run():
+        out = torch.full((lq, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+        lse = torch.full((hq, lq), float("nan"), device="cuda")
+        binding.fp2_sparse_prefill(plan, q, k, v, pt, cu, lk_t, off, cnt, idx, None, None, None, out, lse, ws)
+        binding.fp2_read_status(plan, ws)
+        return out, lse, plan.last_launch_count()
+    o0, l0, n0 = run()
+    plan.set_split(target)
+    o1, l1, n1 = run()
+    assert n0 == n1 == 5
+    assert torch.equal(o0, o1) and torch.equal(l0, l1)
+
+
 def test_large_plans_are_not_split():
     spec = inputs.config_spec(2, scale_down=2)           # 16K tokens: 4096 segments, more than 4 per worker
     case, dc, wl = make(spec)
