@@ -463,8 +463,9 @@ static fp2_status launch_pool(fp2_plan* pl, const void* k, const void* v, const 
 
 // What an attention call runs before its kernel: the counting sort of the segments (KV-head-major, descending block count;
 // hist: class counts and cursors, 2 nb words), and for FP8 plans with a workspace V as F16 (v16, else NULL).
-// cut: see order_scatter_kernel.
-static void launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, const CutLists& cut,
+// cut: see order_scatter_kernel.  A launch that fails is reported before the attention kernel is launched on an order that was
+// not written.
+static fp2_status launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, const CutLists& cut,
                            int32_t* counter, const void* v, const int32_t* pt, __half* v16, int* status, cudaStream_t st) {
   const int nseg = (int)pl->nseg;
   const int nb = pl->prm.num_kv_heads * kCountBuckets;
@@ -473,10 +474,12 @@ static void launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist
          (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, pl->dev, v16, status);
   const int workers = pl->num_sms * AttnCfg<false>::kCtasPerSm;
   launch(order_hist_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, cut.unit_split ? 0 : workers, hist);
-  launch(cut.unit_split ? order_scatter_kernel<true> : order_scatter_kernel<false>, blocks, 256, sizeof(int32_t) * pl->prm.num_kv_heads, st, pl->d_segs, seg_count, nseg,
-         nseg / pl->prm.num_kv_heads, pl->prm.num_kv_heads, workers, hist, hist + nb, order,
-         cut);
+  const int heads = pl->prm.num_kv_heads;
+  launch(cut.unit_split ? order_scatter_kernel<true> : order_scatter_kernel<false>, blocks, 256,
+         heads <= kMaxLongHeads ? sizeof(int32_t) * heads : 0, st, pl->d_segs, seg_count, nseg, nseg / heads, heads, workers, hist,
+         hist + nb, order, cut);
   pl->last_launches += 3;
+  return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -586,10 +589,11 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
     cut.n_split = counter + 2;
     cut.max_slots = pl->cut_slots;
   }
-  launch_prepare(pl, seg_count, reinterpret_cast<int32_t*>(ws + pl->ws_hist), reinterpret_cast<int32_t*>(ws + pl->ws_order),
-                 cut, counter, v, pt,
-                 use_v16 ? reinterpret_cast<__half*>(ws + pl->ws_v16) : nullptr,
-                 reinterpret_cast<int*>(ws + pl->ws_status), st);
+  if ((s = launch_prepare(pl, seg_count, reinterpret_cast<int32_t*>(ws + pl->ws_hist),
+                          reinterpret_cast<int32_t*>(ws + pl->ws_order), cut, counter, v, pt,
+                          use_v16 ? reinterpret_cast<__half*>(ws + pl->ws_v16) : nullptr,
+                          reinterpret_cast<int*>(ws + pl->ws_status), st)) != FP2_OK)
+    return s;
   const bool fp8 = pl->dev.fp8 != 0;
   const int64_t slots = (int64_t)pl->prm.num_pages * pl->prm.page_size;
   CUtensorMap mk, mv, mkb, mkb_lo, mvb;
@@ -639,6 +643,7 @@ static fp2_status run_attention(fp2_plan* pl, const void* q, const void* k, cons
                                           workers, pl->split_target, unit_seg, unit_split, seg_split, split_list, n_units,
                                           n_split);
     pl->last_launches += 1;
+    if (cudaGetLastError() != cudaSuccess) return FP2_ERR_CUDA;
     a.order = unit_seg;
     a.unit_split = unit_split;
     a.n_units = n_units;
@@ -725,8 +730,9 @@ extern "C" fp2_status fp2_dense_prefill_static(fp2_plan* pl, const void* q, cons
   int32_t* order = reinterpret_cast<int32_t*>(sw + kStaticOffOrder);
   // the array keeps the previous call's contents: the status block must start at zero (the sort clears the rest)
   if (cudaMemsetAsync(sw, 0, 64, st) != cudaSuccess) return FP2_ERR_CUDA;
-  launch_prepare(pl, nullptr, reinterpret_cast<int32_t*>(sw + kStaticOffHist), order, CutLists{},
-                 reinterpret_cast<int32_t*>(sw + 64), v, pt, nullptr, reinterpret_cast<int*>(sw), st);
+  if ((s = launch_prepare(pl, nullptr, reinterpret_cast<int32_t*>(sw + kStaticOffHist), order, CutLists{},
+                          reinterpret_cast<int32_t*>(sw + 64), v, pt, nullptr, reinterpret_cast<int*>(sw), st)) != FP2_OK)
+    return s;
   const int64_t slots = (int64_t)pl->prm.num_pages * pl->prm.page_size;
   CUtensorMap mk, mv;
   const bool fp8 = pl->dev.fp8 != 0;

@@ -377,8 +377,11 @@ __global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_
 // 131072 tokens 8632 / 8634.  Shares of 1/4, 1/8, 1/16: 32768 tokens 1697 / 1639 / 1610, the last 8192 of 131072 tokens 1198 /
 // 1107 / 1120, 8191 tokens FP8 211 / 206 / 204, the others within 1 %.
 // Every CTA of 256 threads adds the histogram up for itself (Hkv x 128 counts, in L2): column sums and their prefix give the
-// long segments' places, and the number of long segments per head (head_long, Hkv words) the start of each head.
+// long segments' places, and the number of long segments per head (head_long, Hkv words of shared memory) the start of each
+// head.  Above kMaxLongHeads heads (32 KB; the launch's limit with the static arrays is 48) the order is KV-head-major
+// throughout: with 28 segments per worker and more the end of the call is a small part of it.
 constexpr int kLongShare = 8;
+constexpr int kMaxLongHeads = 8192;
 __device__ __forceinline__ int class_min_count(int c) {   // smallest block count of class c (0 .. kCountBuckets - 1)
   const int v = kCountBuckets - 1 - c;
   return v < 64 ? v : (8 + (v & 7)) << ((v - 64) / 8 + 3);
@@ -426,7 +429,7 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
                                                             int32_t* __restrict__ cursor, int32_t* __restrict__ order,
                                                             CutLists cut) {
   static_assert(kCountBuckets == 128, "thread t adds up class t mod 128; a lane of the scan takes four classes");
-  extern __shared__ int32_t head_long[];       // [num_heads] long segments per head
+  extern __shared__ int32_t head_long[];       // [num_heads] long segments per head (up to kMaxLongHeads heads, else unused)
   __shared__ int32_t col[2][kCountBuckets];    // segments per class over all heads (two halves of the heads)
   __shared__ int32_t before[kCountBuckets];    // units of the long segments of the classes in front of this one
   __shared__ int32_t parts[kCountBuckets];      // parts per segment of the class
@@ -466,7 +469,7 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float len = (float)class_min_count(lane * 4 + i);
-      const bool is_long = len * kLongShare > share;   // (holds for the first classes: they count down)
+      const bool is_long = num_heads <= kMaxLongHeads && len * kLongShare > share;   // (holds for the first classes: they count down)
       if (is_long) {
         ++long_classes;
         n_long += c[i];
@@ -511,7 +514,7 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
   }
   __syncthreads();
   const int first_short = s_first_short;
-  for (int i = warp; i < num_heads; i += 8) {
+  for (int i = warp; first_short > 0 && i < num_heads; i += 8) {
     const int4 c = reinterpret_cast<const int4*>(hist + i * kCountBuckets)[lane];
     int x = (lane * 4 < first_short ? c.x : 0) + (lane * 4 + 1 < first_short ? c.y : 0) +
             (lane * 4 + 2 < first_short ? c.z : 0) + (lane * 4 + 3 < first_short ? c.w : 0);
@@ -536,7 +539,7 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const SegInfo* __res
     return;
   }
   int pos = s_num_long + h * per_head;
-  for (int i = 0; i < h; ++i) pos -= head_long[i];
+  for (int i = 0; first_short > 0 && i < h; ++i) pos -= head_long[i];
   const int32_t* row = hist + h * kCountBuckets;
 #pragma unroll 4
   for (int i = first_short; i < cls; ++i) pos += row[i];

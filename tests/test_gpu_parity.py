@@ -683,6 +683,36 @@ def test_work_order_with_a_few_long_segments(hkv):
     assert torch.isfinite(dc.out.float()).all()
 
 
+@pytest.mark.parametrize("hkv", [8192, 8193, 12300])
+def test_work_order_of_very_many_heads(hkv):
+    """The order's per-head counts are in shared memory up to 8192 KV heads; more than about 11700 would not fit.  Beyond, the order
+    is KV-head-major without them.  One query head per KV head, nine tokens in two pages; dense against fp32 attention
+    (tolerance as for the oracle)."""
+    n = 9
+    prm = dict(num_seqs=1, total_q=n, num_q_heads=hkv, num_kv_heads=hkv, head_dim=128, block_size=128, tile_rows=128,
+               page_size=8, num_pages=3, max_pages_per_seq=2, sink_tokens=256, window_tokens=512, use_correction=1,
+               alpha=0.1, softmax_scale=0.0, dtype=0)
+    plan = binding.Plan(prm, [0, n], [n])
+    g = torch.Generator(device="cuda").manual_seed(hkv)
+    q, k, v = (torch.randn(*s, hkv, 128, generator=g, device="cuda").to(torch.bfloat16) for s in ((n,), (3, 8), (3, 8)))
+    pt = torch.tensor([[2, 0]], dtype=torch.int32, device="cuda")
+    cu = torch.tensor([0, n], dtype=torch.int32, device="cuda")
+    lk = torch.tensor([n], dtype=torch.int32, device="cuda")
+    ws = plan.new_workspace()
+    out = torch.full((n, hkv, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((hkv, n), float("nan"), device="cuda")
+    binding.fp2_dense_prefill(plan, q, k, v, pt, cu, lk, None, None, None, out, lse, ws)
+    binding.fp2_read_status(plan, ws)
+    K, V = (torch.cat([x[2], x[0]])[:n].float() for x in (k, v))
+    s = torch.einsum("ihd,jhd->hij", q.float(), K) / 128 ** 0.5
+    s = s.masked_fill(torch.ones(n, n, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    ref = torch.einsum("hij,jhd->ihd", s.softmax(-1), V)
+    vmax = V.abs().max().item()                    # P and the output each round by 2^-9 of a value: 2^-7 vmax holds both
+    assert (out.float() - ref).abs().max().item() <= vmax * 2.0 ** -7 + 1e-3
+    assert (lse - torch.logsumexp(s, -1)).abs().max().item() <= TOL_LSE_REL
+    plan.close()
+
+
 @pytest.mark.parametrize("p,hkv,seqs", [
     (8, 2, [(3000, 0), (130, 2)]),           # ragged last pages, two sequences
     (128, 2, [(3200, 100)]),                 # whole blocks
