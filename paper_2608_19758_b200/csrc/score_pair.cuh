@@ -66,7 +66,9 @@ struct PairInfo {
 // query rows.  The columns go through in batches of W.  The reference of the exponentials is the maximum of the first 16
 // columns instead of all 128 (no need to hold 128 logits, an eighth of the maxima): the sum is then at least 1, so nothing
 // that matters underflows, and a batch after which it comes near the top of fp32 is done again with its own maximum.  The
-// accumulator is handed back once the last batch is in registers.
+// reference is kept finite: where the first 16 logits are all below the range of fp32 (-inf; queries of -3e38 will do) the
+// others count as ever.  A key whose logits are all -inf has no energy: NaN, which no threshold keeps.  The accumulator is
+// handed back once the last batch is in registers.
 template <bool FP8, bool PARTIAL>
 __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const float* sC, int nrows, uint64_t* release) {
   constexpr int W = FP8 ? 32 : 64;   // the multipliers take registers too: FP8 with 64 spills (131072 tokens 1010 -> 1590 us)
@@ -121,7 +123,7 @@ __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const 
       f2_unpack(f2_add(f2_add(s4[0], s4[1]), f2_add(s4[2], s4[3])), t0, t1);
       return t0 + t1;
     };
-    if (j0 == 0) m = batch_max(kFirst);
+    if (j0 == 0) m = fmaxf(batch_max(kFirst), -3.402823466e38f);
     float sum = add_batch();
     if (__any_sync(0xffffffffu, sum > 1e36f)) {   // (as one warp: the TMEM accesses are warp-wide)
       const float m_new = fmaxf(m, batch_max(W));
@@ -132,7 +134,7 @@ __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const 
     }
     total = sum;
   }
-  return m + log2f(total);
+  return total > 0.f ? m + log2f(total) : __int_as_float(0x7fc00000);
 }
 
 // Raw e4m3 rows in the second half of a query buffer -> F16 rows in both halves, in place; one warp, `rows` a multiple of 32.

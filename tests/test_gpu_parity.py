@@ -657,6 +657,37 @@ def test_scores_far_above_those_of_the_first_rows(first_loud, dtype):
     check_lists(dc, wl)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("quiet", [16, 31])
+def test_scores_whose_first_rows_are_below_the_range_of_fp32(quiet, dtype):
+    """The scorer takes its reference from the first 16 rows of a tile.  Where all of their logits overflow to -inf (heads 0 .. 15
+    query one dimension with -3e38, in which every key is positive), they contribute nothing and the other rows' energies
+    decide, as they do in exact arithmetic.  Whole and partial tiles, pairs and a single tile; no block is forced into a list,
+    and the threshold divides the candidates."""
+    spec = inputs.small_spec(seqs=[(5000, 4001), (901, 0)], num_q_heads=32, num_kv_heads=1, page_size=32, dtype=dtype,
+                             config_id=190, locality_a=0.5)
+    spec.alpha = 0.3
+
+    def lowest(case):
+        if dtype == "fp8":
+            case.k_cache[..., 0] = 0x70                 # 128 in raw units
+            case.q[:, :quiet] = 0
+            case.q[:, :quiet, 0] = 0xFE                 # -448
+            case.q_scale[:quiet] = 1e38
+        else:
+            case.k_cache[..., 0] = 16.0
+            case.q[:, :quiet] = 0
+            case.q[:, :quiet, 0] = -3e38
+    case, dc, wl = make(spec, edit_case=lowest, sink_tokens=0, window_tokens=0)
+    qt = O.tile_queries(wl.q_seq(0), wl.p, wl.segs[0])
+    s = qt @ wl.kv(0, 0)[2].T * wl.p.scale * np.log2(np.e)
+    assert s[:quiet].max() < -3.5e38 and np.abs(s[quiet:32]).max() < 1e4
+    dc.select()
+    dc.status()
+    tot, _ = check_lists(dc, wl)
+    assert 0.1 < tot / dc.plan.idx_capacity < 0.9
+
+
 @pytest.mark.parametrize("hkv", [1, 3])
 def test_work_order_with_a_few_long_segments(hkv):
     """More segments than workers times eight, so that only some count as long and go first: lists of 0 to 2 blocks (the limit
