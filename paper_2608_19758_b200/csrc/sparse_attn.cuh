@@ -749,6 +749,7 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       // visible logit of the row, the warp masks in TMEM as well.
       bool weak_bias = false;
       if constexpr (FP8) weak_bias = __any_sync(0xffffffffu, !(cs_all * 3.0e9f > 256.f));
+      const bool row_ok = row < ti.sg.nrows;   // else padding: whatever queries follow, those of other sequences among them
       float m = -INFINITY, l = 0.f;
       // block id of the next exact iteration, fetched one iteration ahead
       const int i0 = ti.it_begin, i1 = ti.it_end;
@@ -807,8 +808,10 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         const float mx = fmaf(row_load_max(s_addr, x), cs_all, shift);  // cs > 0: scaling commutes with the maximum
         const float m_new = fmaxf(m, mx);
         // lazy rescale: only when some row of the warp moved its maximum by more than 2^8.  O is at rest: the
-        // MMAs complete in issue order, so S (G) in TMEM means O += P V (G-1) has been added.
-        if (__any_sync(0xffffffffu, m_new > m + 8.0f)) {
+        // MMAs complete in issue order, so S (G) in TMEM means O += P V (G-1) has been added.  Padding rows have no say (their
+        // probabilities may overflow, which stays in their own rows): when a row is rescaled decides how its probabilities round,
+        // and that must not hang on what the batch holds beside its sequence.
+        if (__any_sync(0xffffffffu, row_ok && m_new > m + 8.0f)) {
           const float f = (m == -INFINITY) ? 0.f : ex2(m - m_new);
           if (i > i0) {
 #pragma unroll 1
@@ -837,7 +840,6 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       const SegInfo& sg = ti.sg;
       const float inv = l > 0.f ? out_scale / l : 0.f;
       const bool have_o = i1 > i0;
-      const bool row_ok = row < sg.nrows;
       const size_t tok = (size_t)sg.q_tok0 + r / g;
       const int head = sg.h * g + r % g;
       __nv_bfloat16* orow = A.out + (tok * P.num_q_heads + head) * kHeadDim;

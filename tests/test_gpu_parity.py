@@ -636,6 +636,37 @@ def test_work_order_takes_every_segment_once(n_seg_tokens):
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("g", [4, 7, 12])
+def test_a_sequence_does_not_depend_on_its_neighbours(g, dtype):
+    """The rows behind the end of a sequence in its last tile hold other sequences' queries.  The same sequences with queries of quite
+    another size behind them give the same bits: lists, outputs and LSE."""
+    spec = inputs.small_spec(seqs=[(701, 100), (333, 0), (915, 700)], num_q_heads=2 * g, num_kv_heads=2, page_size=16,
+                             dtype=dtype, config_id=210 + g)
+    spec.alpha = 0.2
+    res = []
+    for loud in (False, True):
+        def edit(case):
+            if loud:                                   # the second sequence: other queries, a hundred times as large
+                a, b = case.cu_seqlens_q.tolist()[1:3]
+                if dtype == "fp8":
+                    case.q[a:b] = (case.q[a:b].flip(0) & 0x80) | 0x7E
+                else:
+                    case.q[a:b] = case.q[a:b].flip(0) * 100
+        case, dc, wl = make(spec, edit_case=edit)
+        dc.select(); dc.sparse(); dc.status()
+        sp = dc.out.clone(), dc.lse.clone(), dc.lists_host()
+        dc.dense(); dc.status()
+        res.append((case.cu_seqlens_q.tolist(), sp, (dc.out.clone(), dc.lse.clone())))
+    (cu, (o0, l0, i0), (d0, e0)), (_, (o1, l1, i1), (d1, e1)) = res
+    for a, b in ((0, cu[1]), (cu[2], cu[3])):
+        assert torch.equal(o0[a:b], o1[a:b]) and torch.equal(l0[:, a:b], l1[:, a:b])
+        assert torch.equal(d0[a:b], d1[a:b]) and torch.equal(e0[:, a:b], e1[:, a:b])
+    for s in wl.segs:
+        if s.b != 1:
+            assert np.array_equal(i0[s.seg], i1[s.seg])
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
 @pytest.mark.parametrize("first_loud", [16, 20, 32])
 def test_scores_far_above_those_of_the_first_rows(first_loud, dtype):
     """The scorer's exponentials refer to the first 16 rows of a tile; logits more than 2^119 above them must send a batch
