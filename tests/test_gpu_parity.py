@@ -671,8 +671,8 @@ def test_a_sequence_does_not_depend_on_its_neighbours(g, dtype):
 def test_scores_far_above_those_of_the_first_rows(first_loud, dtype):
     """The scorer's exponentials refer to the first 16 rows of a tile; logits more than 2^119 above them must send a batch
     through again.  One KV head, 32 query heads (a tile is 4 tokens), the queries of the heads from first_loud on 64 times as
-    large (logits in the hundreds): the first batch, a later batch, and with 32 the next token's rows stay quiet throughout.
-    Lists only: probabilities that sharp say nothing more about the attention kernel."""
+    large (logits in the hundreds), so that the first batch holds the loudest rows already (with 32 no head is: the plain
+    case).  Lists only: probabilities that sharp say nothing more about the attention kernel."""
     spec = inputs.small_spec(seqs=[(5000, 1000), (901, 0)], num_q_heads=32, num_kv_heads=1, page_size=32, dtype=dtype,
                              config_id=160 + first_loud)
     spec.alpha = 0.2
@@ -686,6 +686,69 @@ def test_scores_far_above_those_of_the_first_rows(first_loud, dtype):
     dc.select()
     dc.status()
     check_lists(dc, wl)
+
+
+# per row of a tile: by how much its logits (log2) stand above those of the first 16 rows
+LOUD = {
+    "from16": lambda j: 170.0 if j >= 16 else 0.0,          # first batch, all of it
+    "from40": lambda j: 170.0 if j >= 40 else 0.0,          # FP8: second batch of 32; BF16: first of 64
+    "from70": lambda j: 170.0 if j >= 70 else 0.0,          # FP8: third; BF16: second
+    "from100": lambda j: 170.0 if j >= 100 else 0.0,        # the last batch
+    "once": lambda j: 170.0 if j == 77 else 0.0,            # one row, the others behind it quiet again
+    "stairs": lambda j: 150.0 * (j // 32),                  # every batch of 32, or of 64, once more above the one before
+    "stairs64": lambda j: 170.0 * (j // 64) + (90.0 if j % 64 >= 32 else 0.0),   # rises that need a second pass, and rises that do not
+}
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("shape", list(LOUD))
+def test_scores_that_leave_the_reference_behind_in_a_given_batch(shape, dtype):
+    """The scorer goes through a tile's 128 rows in batches (64, FP8: 32) against the maximum of the first 16, and a batch that
+    comes out above 2^119 is done again against its own maximum, the sum so far scaled down.  Here one dimension of every key
+    holds a constant c and the queries' entry there sets a row's level, so which batches that happens in is known: asserted from
+    the oracle's logits.  A tile is 4 tokens x 32 heads; pairs, a single tile, and a last tile of 3 tokens.  No block is forced
+    into a list."""
+    spec = inputs.small_spec(seqs=[(5000, 4001), (902, 3)], num_q_heads=32, num_kv_heads=1, page_size=32, dtype=dtype,
+                             config_id=200, locality_a=0.5)
+    spec.alpha = 0.3
+
+    def levels(case):
+        c = 128.0 * float(case.k_scale[0]) if dtype == "fp8" else 2.0
+        case.k_cache[..., 0] = 0x70 if dtype == "fp8" else c
+        if dtype == "fp8":
+            q = case.q.view(torch.float8_e4m3fn).float() * case.q_scale[None, :, None]
+        else:
+            q = case.q.float()
+        cu = case.cu_seqlens_q.tolist()
+        for b in range(2):
+            r = torch.arange((cu[b + 1] - cu[b]) * 32)
+            lv = torch.tensor([LOUD[shape](int(j) % 128) for j in r])
+            q[cu[b]:cu[b + 1], :, 0] = (lv / (c * 128 ** -0.5 * np.log2(np.e))).view(-1, 32)
+        if dtype == "fp8":
+            case.q_scale[:] = q.abs().amax() / 448.0
+            case.q[:] = inputs.quantize_e4m3(q, case.q_scale[None, :, None])
+        else:
+            case.q[:] = q.to(torch.bfloat16)
+    case, dc, wl = make(spec, edit_case=levels, sink_tokens=0, window_tokens=0)
+    W = 32 if dtype == "fp8" else 64
+    redone = {}
+    for s in wl.segs:
+        x = O.tile_queries(wl.q_seq(s.b), wl.p, s) @ wl.kv(s.b, s.h)[2][:s.J_hi + 1].T * wl.p.scale * np.log2(np.e)
+        ref = x[:16].max(axis=0)                        # per block
+        for k in range(0, x.shape[0], W):
+            top = x[k:k + W].max(axis=0)
+            up = top - ref > 120.0
+            assert (up | (top - ref < 112.0)).all()     # 2^119.6 is the limit on a sum of up to 128: none is near it
+            redone.setdefault(k // W, []).append(up)
+            ref = np.where(up, np.maximum(top, ref), ref)
+    redone = {k: bool(np.concatenate(v).any()) for k, v in redone.items()}
+    want = {"from16": [0], "from40": [40 // W], "from70": [70 // W], "from100": [100 // W], "once": [77 // W],
+            "stairs": [1, 2, 3] if W == 32 else [0, 1], "stairs64": [2] if W == 32 else [1]}[shape]
+    assert [k for k in sorted(redone) if redone[k]] == list(want), redone
+    dc.select()
+    dc.status()
+    tot, _ = check_lists(dc, wl)
+    assert 0.1 < tot / dc.plan.idx_capacity < 0.9
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp8"])
