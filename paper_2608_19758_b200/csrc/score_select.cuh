@@ -39,51 +39,6 @@ constexpr int kScoreRawBytes = 20480;     // FP8: one raw e4m3 box of a query ti
 constexpr int kScoreSmemBytes = 1024 /*align*/ + kScoreQSlots * 32768 + kScoreStages * 32768 + kMaxBlocks * 4 + 2048 +
                                 (2 * kScoreRawBytes - 32768);   // the two raw boxes take the third Q slot and 8 KB more
 
-// Query tile -> shared memory in the K-major 128-byte-swizzled layout the UMMA descriptors expect:
-// BF16: two 64-column halves of [128 rows x 128 B]; FP8 is widened to BF16 on the way (exact).
-// Rows >= nrows are zero-filled.  Called by `nthr` threads with local index `t`.
-template <bool FP8, int BATCH = 8>
-__device__ __forceinline__ void load_q_tile_bf16(uint8_t* sQ, const uint8_t* q, const SegInfo& sg,
-                                                 const DevParams& P, int t, int nthr) {
-  const int g = P.group;
-  for (int i0 = t; i0 < kTileRows * 16; i0 += nthr * BATCH) {
-    uint4 v[BATCH];
-#pragma unroll
-    for (int u = 0; u < BATCH; ++u) {
-      const int i = i0 + u * nthr;
-      const int row = i >> 4, ch = i & 15;  // 16 chunks of 8 elements per row
-      v[u] = make_uint4(0, 0, 0, 0);
-      if (i < kTileRows * 16 && row < sg.nrows) {
-        const int r = sg.r0 + row;
-        const size_t tok = (size_t)sg.q_tok0 + r / g;
-        const size_t head = (size_t)sg.h * g + r % g;
-        const size_t e = (tok * P.num_q_heads + head) * kHeadDim + ch * 8;
-        if constexpr (!FP8) {
-          v[u] = __ldg(reinterpret_cast<const uint4*>(q + e * 2));
-        } else {
-          uint2 raw = __ldg(reinterpret_cast<const uint2*>(q + e));
-          const __nv_fp8x2_storage_t* p2 = reinterpret_cast<const __nv_fp8x2_storage_t*>(&raw);
-          uint32_t o[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            __half2_raw hh = __nv_cvt_fp8x2_to_halfraw2(p2[k], __NV_E4M3);
-            float2 f = __half22float2(*reinterpret_cast<__half2*>(&hh));
-            o[k] = pack_bf16x2(f.x, f.y);
-          }
-          v[u] = make_uint4(o[0], o[1], o[2], o[3]);
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < BATCH; ++u) {
-      const int i = i0 + u * nthr;
-      const int row = i >> 4, ch = i & 15;
-      if (i < kTileRows * 16)
-        *reinterpret_cast<uint4*>(sQ + (ch >> 3) * 16384 + sw128_offset(row, ch & 7)) = v[u];
-    }
-  }
-}
-
 // One raw FP8 tile (128 rows x 128 bytes, 128-byte swizzle as TMA wrote it) -> one F16 tile in the two-halves
 // layout of the K / V rings.  nthr threads (a multiple of 8); eight consecutive threads take one row, so every quarter-warp reads
 // one whole 128-byte row (conflict-free).  Element order inside a row is preserved, so the same routine
@@ -195,10 +150,10 @@ __device__ __forceinline__ void score_chunk(uint32_t lane_addr, float cs, const 
   sum_out = t0 + t1;
 }
 
-// BF16 query tile -> shared memory with cp.async: every 16-byte piece of the tile is in flight at once (the
-// register-staged variant above keeps only a few loads per thread in flight and was latency-bound at one tile
-// per ~12 us).  Same layout and zero fill as load_q_tile_bf16; with `wait` it returns after the copies have landed,
-// otherwise the caller closes a cp.async group and waits for it later.
+// BF16 query tile -> shared memory with cp.async, in the K-major 128-byte-swizzled layout the UMMA descriptors expect (two
+// 64-column halves of [128 rows x 128 bytes]; rows >= nrows are zeros): every 16-byte piece of the tile is in flight at once
+// (staged through registers, a few loads per thread at a time, it was latency-bound at one tile per ~12 us).  With `wait` it
+// returns after the copies have landed, otherwise the caller closes a cp.async group and waits for it later.
 template <int HALF = 16384>   // bytes from one 64-element half of the tile to the other
 __device__ __forceinline__ void load_q_tile_async(uint8_t* sQ, const uint8_t* q, const SegInfo& sg,
                                                   const DevParams& P, int t, int nthr, bool wait = true) {
