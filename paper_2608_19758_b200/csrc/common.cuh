@@ -42,7 +42,8 @@ struct DevParams {
   int32_t num_seqs, nseg, nblk_tot, total_q;
   int32_t fp8;
   int32_t q_box;     // 1: the boxes around one packed tile (q_box_tok tokens) and around two adjacent ones (q_box2_tok) fit the
-                     //    padding: attention kernel (both dtypes) and BF16 scorer fetch query tiles by TMA
+                     //    padding: attention kernel and paired scorer (both dtypes) fetch query tiles by TMA.  Not so for
+                     //    group sizes such as 11, 12 or 48, whose boxes reach further in front of a tile or behind it
   int32_t q_box_tok, q_box2_tok;   // 128 / g tokens where g divides 128, else floor((g - 1 + 127) / g) + 1; 256 rows likewise
   int32_t q_raw_tma; // 1: FP8 plans whose box fits the scorer's raw staging slot: the scorer fetches query tiles by TMA
   int32_t diag_mma;  // 1: a tile spans at most 32 positions (g >= 4), so the causal mask of a diagonal block can ride

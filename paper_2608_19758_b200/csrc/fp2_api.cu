@@ -38,7 +38,7 @@ struct fp2_plan {
   int32_t* d_blk_off;
   int32_t* d_carry;                 // [3 x num_seqs]: pooled rows carried over from a previous chunk (fp2_pool_carry)
   int32_t* d_lk;                    // [num_seqs]: KV lengths as given to fp2_plan_create
-  int2* d_units;                    // scorer work units of BF16 plans whose query tiles come by TMA: (segment, second segment or -1)
+  int2* d_units;                    // scorer work units of plans with DevParams::q_box: (segment, second segment or -1)
   int32_t nunits;
   std::vector<int32_t> h_blk_off, h_carry;
   bool carry_valid;
@@ -461,8 +461,8 @@ static fp2_status launch_pool(fp2_plan* pl, const void* k, const void* v, const 
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }
 
-// What an attention call runs before its kernel: the counting sort of the segments (KV-head-major, descending block count;
-// hist: class counts and cursors, 2 nb words), and for FP8 plans with a workspace V as F16 (v16, else NULL).
+// What an attention call runs before its kernel: the counting sort of the segments (see order_scatter_kernel; hist: class
+// counts and cursors, 2 nb words), and for FP8 plans with a workspace V as F16 (v16, else NULL).
 // cut: see order_scatter_kernel.  A launch that fails is reported before the attention kernel is launched on an order that was
 // not written.
 static fp2_status launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t* hist, int32_t* order, const CutLists& cut,

@@ -125,7 +125,7 @@ __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const 
     };
     if (j0 == 0) m = fmaxf(batch_max(kFirst), -3.402823466e38f);
     float sum = add_batch();
-    if (__any_sync(0xffffffffu, sum > 1e36f)) {   // (as one warp: the TMEM accesses are warp-wide)
+    if (__any_sync(0xffffffffu, sum > 1e36f)) {   // (as one warp: the next batch's TMEM loads want it whole)
       const float m_new = fmaxf(m, batch_max(W));
       s4[0] = f2_pack(total * ex2(m - m_new), 0.f);   // (total = 0 in the first batch, m is finite)
       s4[1] = s4[2] = s4[3] = 0ull;

@@ -2,8 +2,8 @@
 // persistent, warp-specialised, tcgen05 / TMEM / TMA.  The same kernel runs the dense path (implicit list
 // 0..J_hi, no correction).
 //
-// CTAs loop over work units (sequence, KV head, packed query tile) taken from a work order (KV-head-major,
-// heaviest first) through a global counter.  For a unit with selected list idx[0..T) the iteration sequence
+// CTAs loop over work units (sequence, KV head, packed query tile) taken from a work order (long ones of all heads
+// first, then KV-head-major, see order_scatter_kernel) through a global counter.  For a unit with selected list idx[0..T) the iteration sequence
 // is the list traversed backwards (Eq. 17) followed by the non-empty correction chunks: a correction chunk
 // stages 128 consecutive pooled (kbar, vbar) rows exactly like a KV block, its logits are shifted by log2(128)
 // (every corrected block is full) and masked by todo = fully-visible & ~selected.
