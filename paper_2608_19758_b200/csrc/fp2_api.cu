@@ -61,13 +61,16 @@ struct fp2_plan {
 // FP8 attention with V as F16 in the workspace, or widened by the kernel in every iteration?  The copy takes about 6 us and
 // 11 ns per block of a KV head (3 bytes per element at 4.5 TB/s); an iteration without the widening is 450 cycles of an SM
 // shorter (900 of one of its two CTAs), 1.6 ns over 148 SMs.  So it pays from 4000 + 7 blocks x heads iterations.  Measured
-// (whole calls, widened per iteration / copy): 700 tokens, 32 heads on 8 48.3 / 56.4 us, 2000 tokens, 28 on 4 78.8 / 81.1,
-// 8191 tokens 267 / 236, 131072 tokens 8985 / 7990, its last 8192 tokens 777 / 729, 16 sequences of 245000 tokens
-// 3824 / 3579, dense 16384 tokens 1782 / 1486.  A sparse call's lists are not known on the host: 20 blocks per tile (sink,
-// window and diagonal are 7 to 8 of them).
+// (whole calls, widened per iteration / copy): 700 tokens, 32 heads on 8 46.2 / 50.2 us, 2000 tokens, 28 on 4 70.4 / 75.0,
+// 8191 tokens 221.7 / 196.1, 131072 tokens 8706 / 7715, its last 8192 tokens 1139 / 1078, 16 sequences of 245000 tokens
+// 3611 / 3333, dense 16384 tokens 1723 / 1456.  A sparse call's lists are not known on the host: 20 blocks per tile (sink,
+// window and diagonal are 7 to 8 of them); short calls with longer lists, at low thresholds, go on widening.
 constexpr int kLikelyListLen = 20;
 constexpr int kCutSlots = 256;       // 16.7 MB of partial results
-constexpr int kCutMinCand = 512;     // longest candidate range (60160 tokens, 4 heads, nothing to cut: the launch costs 2 of 101 us)
+// Longest candidate range from which calls cut.  Not the quantity that decides (that is the longest list against a worker's share,
+// known on the device only): from 128 on the last 2040 tokens of 60000 went from 279 to 215 us, but the dense last 512 tokens of
+// 32768 from 362 to 429, and calls with nothing to cut lose up to 1 % to the launch.
+constexpr int kCutMinCand = 512;
 static inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 extern "C" const char* fp2_status_string(fp2_status s) {
@@ -168,7 +171,7 @@ extern "C" fp2_status fp2_plan_create(const fp2_params* p, const int32_t* h_cu, 
   // blocks, so they are scored together when the later one has at most kPairMaxCand candidates; heaviest first
   // (descending segment index, like the single-tile scorer's order).  Where every tile has an SM to itself a pair would only
   // lengthen the chain of its CTA: 768 tokens FP8, 48 tiles, select + sparse
-  // 38.0 us in pairs, 35.6 one by one.
+  // 35.2 us in pairs, 33.3 one by one.
   std::vector<int2> units;
   int cur_dev = -1, sms = 0;
   if (cudaGetDevice(&cur_dev) != cudaSuccess ||
@@ -345,8 +348,8 @@ extern "C" int32_t fp2_last_launch_count(const fp2_plan* pl) { return pl ? pl->l
 // helpers
 // ------------------------------------------------------------------------------------------------------
 // A kernel launch that may overlap the end of its predecessor on the stream (see pdl_wait: every kernel of this library
-// waits there before it touches global memory).  Select + sparse at 2048 tokens, 4 heads: 48 us with plain launches, two
-// memsets and a scan kernel in the sort, 35 us so.
+// waits there before it touches global memory).  Select + sparse at 2048 tokens, 4 heads: 48.4 us with plain launches, two
+// memsets and a scan kernel in the sort, 35.2 so; dense 839 tokens 42.9 / 25.2.
 template <typename... KArgs, typename... Args>
 static void launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchAttribute attr;

@@ -32,7 +32,7 @@ __device__ __forceinline__ int clamped_count(const SegInfo& sg, const int32_t* s
 // Offsets in two steps, in place (nothing but the caller's cu holds them).  csr_count_kernel: cu[g + 1] = tiles of the segments
 // of g's group of kCsrGroup up to g.  csr_offset_kernel, one CTA: adds the groups in front, whose totals are the last entries of
 // the groups.  (One CTA that scanned all counts tile by tile took 13 of the 32 us of an export of 16384 segments; index and
-// export of 65536 tokens 402 -> 374 us, of 22965 tokens 122 -> 119, of 98374 tokens 610 -> 589.)
+// export of 65536 tokens 391 -> 384 us, of 22965 tokens 112.5 -> 107.2, of 98374 tokens 713 -> 698.)
 constexpr int kCsrGroup = 256;
 
 // inclusive prefix sum over the CTA's threads (a multiple of 32, up to 1024); warp_tot: 32 words of shared memory

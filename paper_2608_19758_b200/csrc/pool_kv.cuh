@@ -357,7 +357,8 @@ __global__ void __launch_bounds__(256) attn_prepare_kernel(int32_t* __restrict__
 }
 
 // Where every segment has a worker of its own (nseg <= workers) all of them start at once: there is nothing to sort, the order
-// is the segments' own.  Select + sparse, 768 tokens FP8 35.1 -> 32.9 us, 2370 tokens 38.6 -> 36.9; dense, 839 tokens 21.5 -> 21.0.
+// is the segments' own.  Sorted / so: select + sparse, 768 tokens FP8 35.5 / 33.3 us, 2370 tokens 41.5 / 40.3, 2048 tokens 34.4 /
+// 32.9; dense, 839 tokens 22.9 / 22.1.
 __global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_t* count, int nseg, int workers,
                                   int32_t* __restrict__ hist) {
   pdl_trigger();
@@ -372,10 +373,9 @@ __global__ void order_hist_kernel(const SegInfo* __restrict__ segs, const int32_
 // head's long ones late.  So segments longer than 1 / kLongShare of a worker's share of all listed blocks come first, heads
 // mixed, longest first; the others follow KV-head-major (the K / V of one head stay in L2), in descending order too.  With
 // many segments per worker hardly any is that long and the order is KV-head-major; with few the heads run side by side
-// whatever the order is.  Whole calls, KV-head-major throughout / so: the last 8192 of 131072 tokens 1404 / 1142 us (longest
-// list 408 blocks, mean 41), 8191 tokens FP8 227 / 212, 15616 tokens, 32 heads on 4, 134 / 122, 32768 tokens 1576 / 1536,
-// 131072 tokens 8632 / 8634.  Shares of 1/4, 1/8, 1/16: 32768 tokens 1697 / 1639 / 1610, the last 8192 of 131072 tokens 1198 /
-// 1107 / 1120, 8191 tokens FP8 211 / 206 / 204, the others within 1 %.
+// whatever the order is.  Whole calls, KV-head-major throughout / shares of 1/4 / 1/8 / 1/16, in turn: the last 8192 of 131072
+// tokens 1514 / 1347 / 1375 / 1408 us, FP8 1204 / 1075 / 1084 / 1088, 32768 tokens 1778 / 1780 / 1731 / 1759, 8191 tokens FP8
+// 206.5 / 201.7 / 196.4 / 196.2; 131072 tokens, and 15616 tokens with 32 heads on 4, the same.
 // Every CTA of 256 threads adds the histogram up for itself (Hkv x 128 counts, in L2): column sums and their prefix give the
 // long segments' places, and the number of long segments per head (head_long, Hkv words of shared memory) the start of each
 // head.  Above kMaxLongHeads heads (32 KB; the launch's limit with the static arrays is 48) the order is KV-head-major

@@ -19,10 +19,9 @@
 // about 2700 at the clocks that the power limit leaves at 131072 tokens (without the exponentials 7 % less, without the MMAs
 // the same).  The items (chunk, tile) are dealt to THREE consumer warpgroups, so that one loads or waits while the others
 // exponentiate, and an item goes through in batches (see score_cols), which is what lets three of them fit into the registers.
-// Index stage, two warpgroups with a tile each and 128 columns in one piece / so: 131072 tokens 1099 / 1065 us, 65536 tokens
-// 376 / 365, 32768 tokens 150 / 141, 16 sequences of 245000 tokens 681 / 650, 24 short ones 48.5 / 45.3.  FP8 plans took one
-// tile per chunk in score_select_kernel before: 131072 tokens, 28 heads on 4, 1216 / 1012, 16 sequences 874 / 720, 8191 tokens
-// 53.3 / 48.6.
+// Whole calls, two warpgroups with a tile each and 128 columns in one piece / so: lists of 65536 tokens 398 / 390 us, of 22965
+// 115.0 / 112.5; attention included 131072 tokens 10828 / 10790.  FP8 plans took one tile per chunk in score_select_kernel before:
+// 131072 tokens, 28 heads on 4, 7935 / 7720, 16 sequences 3492 / 3357, 8191 tokens 204.7 / 200.6.
 //
 // FP8: the raw e4m3 box lands in the second half of a query buffer, where its 128-byte rows are as many as the F16 rows of a
 // half, and the set-up warp widens it in place: elements 0..63 of a row go to the first half, 64..127 over the raw row.  Every
@@ -35,8 +34,8 @@
 // columns.
 //
 // Group sizes that do not divide 128 (7 and the like) used to stage every tile with 2048 cp.async pieces of 16 bytes, each
-// with its own divisions: 24 sequences of 60 to 1500 tokens, 28 query heads on 4 KV heads, 202 us for the index stage then,
-// 53 us with the boxes (and the attention call 174 -> 131 us by the same change).
+// with its own divisions: select + sparse of 24 sequences of 60 to 1500 tokens, 28 query heads on 4 KV heads, 360 us then, 170
+// with the boxes in this kernel and the attention kernel.
 #pragma once
 #include "score_select.cuh"
 

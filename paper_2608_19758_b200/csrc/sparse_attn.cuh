@@ -39,7 +39,7 @@
 // output.  Correction chunks: the pooled keys come as an e4m3 hi + lo pair in raw units (two accumulating MMA groups, ~8
 // mantissa bits together), the pooled values as F16.  Tile memory: Q 16 KB, K 32 KB (one raw tile, or hi | lo of a
 // chunk), F16 V 32 KB (raw V 16 KB).
-// 16384 tokens dense, 28 heads on 4 KV heads: 1782 us widening per iteration, 1486 us with the copy (its 11 us included).
+// 16384 tokens dense, 28 heads on 4 KV heads: 1723 us widening per iteration, 1456 us with the copy (its 11 us included).
 #pragma once
 #include <cuda_bf16.h>
 #include "common.cuh"
@@ -102,9 +102,10 @@ struct AttnArgs {
 
 // P is handed to the issuer in column slices.  Each hand-over stalls the warp for its TMEM stores, and what follows the last one
 // (the slice's MMAs, then S = Q K^T) is what the warp waits for; so: a short first slice to get O += P V going, a long middle
-// one, a short last one.  In k-steps (of eight), us at the power limit: 32768 tokens dense BF16 4 x 2 8290, 4 + 4 7920, 2 + 5 + 1
-// 7600, 2 + 4 + 2 7360; 131072 tokens 8930 / 8620 / 8530 / 8330; dense 16384 tokens FP8 1492 / 1488 / 1411 / 1484, 16 sequences
-// FP8 3376 / 3270 / 3295 / 3321.  16 columns a store, except FP8, whose middle slice ends inside 16 (8 there: 1411, 16: 1465).
+// one, a short last one.  In k-steps (of eight), whole calls in us, in turn: 4 x 2 / 4 + 4 / 2 + 5 + 1 / 2 + 4 + 2: 32768 tokens
+// dense BF16 8090 / 8050 / 7786 / 7615, 32768 tokens 1794 / 1775 / 1739 / 1728, 131072 tokens 10980 / 10923 / 10722 / 10611, 16
+// sequences within 1 %; FP8 16384 tokens dense 1509 / 1506 / 1456 / 1518, 131072 tokens 7872 / 7882 / 7715 / 7898, 8191 tokens
+// 200.6 / 200.2 / 196.2 / 199.7, 16 sequences within 1 %.  16 columns a store, except FP8, whose middle slice ends inside 16.
 constexpr int kPParts = 3;
 template <bool FP8>
 struct PSlices {
@@ -320,8 +321,8 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     // A chain of dependent global loads (work counter -> order -> segment and count -> list -> page table), which at the start
     // of a call nothing hides: both warps load what they need themselves instead of passing it on, the page-table entries of
     // the list go to the L1 for the producer, the first unit is the CTA's own number, and its query tile is requested as soon
-    // as the segment is known.  2048 tokens: logits of the first block after 8000 cycles of the kernel (9100 before), whole call
-    // 38.6 -> 37.4 us; 16 sequences of 245000 tokens 3561 -> 3513, 60160 tokens with 4 heads 100.8 -> 96.1.
+    // as the segment is known.  2048 tokens: logits of the first block after 8000 cycles of the kernel (9100 before).  Whole calls,
+    // together with the issuer's look-ahead: 2048 tokens 35.8 -> 34.3 us, 2370 tokens 43.4 -> 41.2; long ones within 1 %.
     setmaxnreg_dec<AttnCfg<FP8>::kRegsService>();
     const int t64 = tid - 32 * 6;
     const bool corr = P.use_correction != 0;
@@ -608,8 +609,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     // =============================== UMMA issuer ===============================
     // The whole warp walks this loop and waits; one elected lane issues.  Outside the elected branches the loop is
     // warp-uniform, which shortens the instruction chain around every MMA: with the loop inside `if (lane == 0)` the
-    // issuing thread itself was what the tensor pipe waited for (32768 tokens, dense: 8.56 -> 7.99 ms; 131072 tokens at
-    // 95 % sparsity: 10.1 -> 9.6 ms, FP8 8.4 -> 8.0 ms).
+    // issuing thread itself was what the tensor pipe waited for (32768 tokens dense 8429 -> 7993 us, 131072 tokens at 95 %
+    // sparsity 11368 -> 10825, FP8 9320 -> 9035, 16 sequences 3702 -> 3556).  The waits' results stay out of it: with a flag per
+    // lane that an expired wait clears, `if (leader && live)`, every call was 5 to 10 % slower.
     setmaxnreg_dec<AttnCfg<FP8>::kRegsService>();
     const bool leader = elect_one();
     constexpr int kFmt = FP8 ? 0 : 1;   // kind::f16 operand format of O += P V: 0 = F16, 1 = BF16
@@ -647,9 +649,9 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
     // Look-ahead.  A shared-memory wait that follows a commit in this warp is held until the commit has been taken: from the last
     // slice of O += P V to S = Q K^T (G+1) it took some 500 cycles although K (G+1) had long landed.  So what S = Q K^T (G+1)
     // needs is looked at BEFORE the last slice of P (G) is waited for, across a unit boundary too, and where it is there its
-    // MMAs follow those of the last slice without a wait in between.  Without / with it (us): 32768 tokens dense 7900 / 7510,
-    // 16384 tokens dense FP8 1569 / 1428, 131072 tokens 8780 / 8350, FP8 6440 / 6120, 16 sequences FP8 3376 / 3296, 24 short ones
-    // 162.7 / 156.7, 16 sequences BF16 3562 / 3565.
+    // MMAs follow those of the last slice without a wait in between.  Without / with it (us): 32768 tokens dense 7760 / 7615,
+    // 16384 tokens dense FP8 1503 / 1456, 131072 tokens FP8 7849 / 7715, 8191 tokens FP8 199.3 / 196.2; 131072 and 32768 tokens BF16
+    // and 16 sequences within 1 %.  (With P in four slices it gave nothing.)
     uint32_t G = 0;
     bool qk_issued = false;   // S = Q K^T (G) is under way already
     for (int it = 0;; ++it) {
