@@ -350,8 +350,12 @@ extern "C" int32_t fp2_last_launch_count(const fp2_plan* pl) { return pl ? pl->l
 // A kernel launch that may overlap the end of its predecessor on the stream (see pdl_wait: every kernel of this library
 // waits there before it touches global memory).  Select + sparse at 2048 tokens, 4 heads: 48.4 us with plain launches, two
 // memsets and a scan kernel in the sort, 35.2 so; dense 839 tokens 42.9 / 25.2.
+// Not early: kernels that stream much memory from CTAs of which several fit on an SM.  Early ones fill the first SMs that the
+// predecessor leaves, and the rest of the chip, bandwidth with it, idles: pooling back to back 12000 tokens, 8 heads, 27.0 us
+// early / 12.3 behind its predecessor, 22965 tokens 31.1 / 20.6.
 template <typename... KArgs, typename... Args>
-static void launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args) {
+static void launch_at(bool early, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                      Args&&... args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -361,8 +365,12 @@ static void launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   (void)cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);   // the caller reads cudaGetLastError
+}
+template <typename... KArgs, typename... Args>
+static void launch(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args&&... args) {
+  launch_at(true, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 
 // 3-D map over [rows, heads, 128] elements, box = [box_rows, 1, 64 (bf16) | 128 (fp8)], 128-byte swizzle.
@@ -458,8 +466,13 @@ static fp2_status launch_pool(fp2_plan* pl, const void* k, const void* v, const 
   const unsigned grid = (unsigned)(pl->nblk_tot * (rows ? 1 : pl->prm.num_kv_heads) * 2);
   auto kernel = pl->dev.fp8 ? (rows ? pool_rows_kernel<true> : pool_kv_kernel<true>)
                             : (rows ? pool_rows_kernel<false> : pool_kv_kernel<false>);
-  launch(kernel, grid, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs, pl->dev, khi,
-         klo, vb, ws + pl->ws_k8hi, ws + pl->ws_k8lo, carry, status);
+  // Early (see launch_at) where little is read, or behind the small kernel that carries means over.  Select + sparse, early /
+  // not: 0.4 MB 33.3 / 35.7 us, 1 MB 32.7 / 33.5, 2.4 MB 40.4 / 40.9, 8.4 MB 190.3 / 185.3, 9.7 MB 86.4 / 70.2, 20 MB 130.8 / 116.5
+  // and, 16 heads, 122.3 / 85.9; with carried means 145.5 / 148.7.
+  constexpr int64_t kPoolEarlyBytes = 2 << 20;
+  const bool early = carry != nullptr || pl->nblk_tot * kBlock * row_chunks * 32 <= kPoolEarlyBytes;
+  launch_at(early, kernel, grid, 256, 0, st, (const uint8_t*)k, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, ks, vs, pl->dev,
+            khi, klo, vb, ws + pl->ws_k8hi, ws + pl->ws_k8lo, carry, status);
   pl->last_launches += 1;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }
@@ -473,8 +486,9 @@ static fp2_status launch_prepare(fp2_plan* pl, const int32_t* seg_count, int32_t
   const int nseg = (int)pl->nseg;
   const int nb = pl->prm.num_kv_heads * kCountBuckets;
   const unsigned blocks = (unsigned)((nseg + 255) / 256), n_clear = (unsigned)((2 * nb + 255) / 256);
-  launch(attn_prepare_kernel, n_clear + (v16 ? (unsigned)(pl->nblk_tot * (kBlock / kWidenTokens)) : 0u), 256, 0, st, hist, 2 * nb, counter, (int)n_clear,
-         (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, pl->dev, v16, status);
+  // (with V to widen not early, see launch_at: 8191 tokens 196.7 / 190.3 us, 12000 tokens 287.8 / 277.6)
+  launch_at(v16 == nullptr, attn_prepare_kernel, n_clear + (v16 ? (unsigned)(pl->nblk_tot * (kBlock / kWidenTokens)) : 0u), 256,
+            0, st, hist, 2 * nb, counter, (int)n_clear, (const uint8_t*)v, pt, pl->d_lk, pl->d_blk_off, pl->dev, v16, status);
   const int workers = pl->num_sms * AttnCfg<false>::kCtasPerSm;
   launch(order_hist_kernel, blocks, 256, 0, st, pl->d_segs, seg_count, nseg, cut.unit_split ? 0 : workers, hist);
   const int heads = pl->prm.num_kv_heads;
