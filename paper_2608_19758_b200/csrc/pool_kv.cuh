@@ -387,11 +387,12 @@ __device__ __forceinline__ int class_min_count(int c) {   // smallest block coun
   return v < 64 ? v : (8 + (v & 7)) << ((v - 64) / 8 + 3);
 }
 // Cutting (Eq. 18).  A segment longer than a worker's share outlasts the rest even when it starts first (the last 8192 of
-// 131072 tokens: one list of 408 blocks against a share of 349).  Calls that can have such segments (template parameter CUT, see
+// 131072 tokens: one list of 408 blocks against a share of 287).  Calls that can have such segments (template parameter CUT, see
 // fp2_plan_create) ask for units instead of segments: if the longest class exceeds kCutFrom shares, segments longer than half a
 // share become parts of about that length, longest classes first while their partial results fit into max_slots, and the
-// merge kernel of the split path puts them together.  That call 1279 -> 1056 us; where the longest list is three quarters of a
-// share cutting gained nothing (107371-token chunk 978 / 989).
+// merge kernel of the split path puts them together.  That call 1133 -> 1049 us, with a list of 466 blocks against a share of 382
+// 1380 -> 1328; where the longest list is below a share nothing is cut.  Against attention in 64 bits the parts' result is as
+// far off as the uncut one (rel 1.8059e-3 / 1.8066e-3, 100001 tokens 1.7861e-3 / 1.8029e-3, FP8 1.66254e-3 / 1.66258e-3).
 // unit_split[w]: see pack_split; *n_units: units; seg_split, split_list, *n_split: what the merge kernel reads.
 struct ClassScan {   // exclusive prefix over the classes, four per lane of a warp
   int before[4], total;
