@@ -897,7 +897,7 @@ extern "C" fp2_status fp2_page_table_from_token_map(fp2_plan* pl, const int32_t*
 // descriptor handed to a whole warp (the lanes of warp 1 run out at times of their own, those of warp 0 see its flag), then
 // the common way out.
 // ------------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(64, 1) bounded_wait_probe_kernel(int* status, long long budget_cycles) {
+__global__ void __launch_bounds__(64, 1) bounded_wait_probe_kernel(int* status, uint32_t budget_cycles) {
   __shared__ uint64_t never;       // nobody arrives here
   __shared__ uint64_t drain_bar;
   __shared__ uint32_t tmem_base_s;
@@ -919,7 +919,7 @@ __global__ void __launch_bounds__(64, 1) bounded_wait_probe_kernel(int* status, 
   tc_fence_after();
   WaitCtx ctx{status, &abort_flag, warp == 1 ? budget_cycles * (32 + lane) / 64 : budget_cycles};
   while (ready_warp(&never, 0, ctx, warp == 1 ? 901 : 902, &valid)) {}   // (ends with the first wait)
-  leave_cta(&abort_flag, &drain_bar, warp == 0);
+  leave_cta(ctx, &drain_bar, warp == 0);
   if (warp == 0) tmem_dealloc(tmem_base_s, 32);
 }
 
@@ -930,7 +930,7 @@ extern "C" fp2_status fp2_selftest_bounded_wait(fp2_plan* pl, void* workspace, f
   if (cudaGetDevice(&dev) != cudaSuccess) return FP2_ERR_CUDA;
   if (dev != pl->device) return FP2_ERR_INVALID_ARG;
   int* status = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(workspace) + pl->ws_status);
-  bounded_wait_probe_kernel<<<1, 64, 0, reinterpret_cast<cudaStream_t>(stream)>>>(status, 1000000ll);
+  bounded_wait_probe_kernel<<<1, 64, 0, reinterpret_cast<cudaStream_t>(stream)>>>(status, 1000000u);
   pl->last_launches = 1;
   return cudaGetLastError() == cudaSuccess ? FP2_OK : FP2_ERR_CUDA;
 }

@@ -17,15 +17,15 @@ namespace fp2 {
 // Layout of the device status block (int32 words) kept in the caller's workspace.
 enum : int { ST_TIMEOUT = 0, ST_WHERE = 1, ST_BAD_LIST = 2, ST_WORDS = 8 };
 
-// Cycle budget of one wait (about one second at 2 GHz).
+// Cycle budget of one wait (about one second at 2 GHz), below 2^32.
 #ifndef FP2_WAIT_CYCLES
-#define FP2_WAIT_CYCLES (2000000000ll)
+#define FP2_WAIT_CYCLES (2000000000u)
 #endif
 
 struct WaitCtx {
   int* status;           // global status block
-  volatile int* abort;   // CTA-shared flag: once set, every wait returns after at most 256 polls
-  long long budget = FP2_WAIT_CYCLES;   // cycles one wait may take
+  volatile int* abort;   // CTA-shared flag: once set (to the site of an expired wait), every wait returns after at most 256 polls
+  uint32_t budget = FP2_WAIT_CYCLES;    // cycles one wait may take
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -73,20 +73,21 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 }
 // Waits until the phase with the given parity has completed.  Bounded: on expiry the status
 // block records the site and the CTA-wide abort flag makes all later waits fall through.  False: the phase has not completed.
+// (Inlined at some forty places of a kernel, so what it does after an expiry is kept short: the abort flag holds the site until
+// leave_cta puts it into the status block.)
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtx& ctx, int where) {
   if (mbar_try_wait(bar, parity)) return true;
-  long long t0 = clock64();
-  int spins = 0;
+  const uint32_t t0 = clock();
+  uint32_t polls = 0;
   while (!mbar_try_wait(bar, parity)) {
-    if (((++spins) & 255) == 0) {
+    if (((++polls) & 255) == 0) {
       if (*ctx.abort) {
         // words 3..7: the wait each role (2xx .. 6xx) of an aborted CTA was found in (last writer wins)
         if (where >= 200 && where < 700) ctx.status[3 + (where / 100 - 2)] = where;
         return false;
       }
-      if (clock64() - t0 > ctx.budget) {
-        *ctx.abort = 1;
-        if (atomicCAS(ctx.status + ST_TIMEOUT, 0, 1) == 0) ctx.status[ST_WHERE] = where;
+      if ((uint32_t)clock() - t0 > ctx.budget) {
+        *ctx.abort = where;
         return false;
       }
     }
@@ -210,11 +211,12 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 // every MMA has completed.  After an abort MMAs and bulk copies may still be in flight: that thread waits (bounded) for its
 // MMAs and everyone gives the copies time, before tensor memory is released and the CTA's shared memory goes.  The flag is
 // read behind the CTA barrier: every wait is over then, so it is final and all threads read the same.
-__device__ __forceinline__ void leave_cta(const volatile int* abort_flag, uint64_t* drain_bar, bool issuer) {
+__device__ __forceinline__ void leave_cta(const WaitCtx& ctx, uint64_t* drain_bar, bool issuer) {
   tc_fence_before();
   __syncwarp();
   __syncthreads();
-  if (*abort_flag) {
+  if (*ctx.abort) {
+    if (threadIdx.x == 0 && atomicCAS(ctx.status + ST_TIMEOUT, 0, 1) == 0) ctx.status[ST_WHERE] = *ctx.abort;
     if (issuer && elect_one()) {
       umma_commit(drain_bar);
       mbar_wait_drain(drain_bar, 0, 200000000ll);

@@ -463,7 +463,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       gc0 += (uint32_t)nchunks;
     }
   }
-  leave_cta(&abort_flag, &drain_bar, warp == 4 * kPairGroups + 1);
+  leave_cta(ctx, &drain_bar, warp == 4 * kPairGroups + 1);
   if (warp == 4 * kPairGroups + 1) tmem_dealloc(tmem, 512);
 }
 

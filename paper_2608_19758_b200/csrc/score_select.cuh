@@ -508,7 +508,7 @@ score_select_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_co
       gc0 += (uint32_t)nchunks;
     }
   }
-  leave_cta(&abort_flag, &drain_bar, warp == 9);
+  leave_cta(ctx, &drain_bar, warp == 9);
   if (warp == 9) tmem_dealloc(tmem, 256);
 }
 
