@@ -406,11 +406,10 @@ static bool make_q_map(fp2_plan* pl, CUtensorMap* m, const void* q, int box_toke
 
 static fp2_status set_attrs(fp2_plan* pl) {
   if (pl->attrs_set) return FP2_OK;
-  if (cudaFuncSetAttribute(score_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(score_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(score_select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  for (auto kernel : {score_pair_kernel<false, 0>, score_pair_kernel<true, 0>, score_pair_kernel<true, 4>, score_pair_kernel<true, 7>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) != cudaSuccess)
+      return FP2_ERR_CUDA;
+  if (cudaFuncSetAttribute(score_select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kScoreSmemBytes) != cudaSuccess ||
       cudaFuncSetAttribute(score_select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kScoreSmemBytes) != cudaSuccess ||
@@ -529,7 +528,10 @@ extern "C" fp2_status fp2_select_blocks(fp2_plan* pl, const void* q, const void*
   int* status = reinterpret_cast<int*>(ws + pl->ws_status);
   if (pl->dev.q_box) {
     // pairs of adjacent tiles per pooled-key chunk, in pieces of 64 elements x 128 keys (the box of mhi / mlo)
-    launch(pl->dev.fp8 ? score_pair_kernel<true> : score_pair_kernel<false>,
+    const int g = pl->dev.group;
+    auto kernel = !pl->dev.fp8 ? score_pair_kernel<false, 0> : 8 % g == 0 ? score_pair_kernel<true, 4>
+                               : g == 7 ? score_pair_kernel<true, 7> : score_pair_kernel<true, 0>;
+    launch(kernel,
            (unsigned)(pl->nunits < pl->num_sms ? pl->nunits : pl->num_sms), kPairThreads, kPairSmemBytes, st, mhi, mlo, mq, mq2,
            pl->d_segs, pl->d_units, pl->nunits, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
   } else {

@@ -24,8 +24,11 @@
 // 131072 tokens, 28 heads on 4, 7935 / 7720, 16 sequences 3492 / 3357, 8191 tokens 204.7 / 200.6.
 //
 // FP8: the raw e4m3 box lands in the second half of a query buffer, where its 128-byte rows are as many as the F16 rows of a
-// half, and the set-up warp widens it in place: elements 0..63 of a row go to the first half, 64..127 over the raw row.  Every
-// row has a multiplier of its own (q_scale), kept per unit in sC.
+// half, and the consumer warps widen it in place, one unit ahead: elements 0..63 of a row go to the first half, 64..127 over the
+// raw row.  Every row has a multiplier of its own (q_scale), kept per unit in sC.  One warp that fetched and widened the tiles was
+// what the units waited for (8191 tokens, one chunk of keys per unit: 8900 cycles a unit, of which 5000 widening and 2100 the box).
+// Select call in us, widened by one warp / by the consumers: 8191 tokens, 28 heads on 4, 42.6 / 32.8, 12000 tokens, 32 on 8, 66.8 /
+// 48.8; lists of 12000 tokens with export 77.0 / 57.8; with attention 16 sequences 3222 / 3186, 131072 tokens the same.
 //
 // Roles: warps 0-11 consumers; warp 12 TMA producer of kbar pieces (16 KB: 128 keys x 64 elements, four per chunk: hi | lo x
 // the two halves of d); warp 13 UMMA issuer and TMEM owner; warp 14 unit set-up and query tiles by TMA (two units in flight);
@@ -68,9 +71,12 @@ struct PairInfo {
 // reference is kept finite: where the first 16 logits are all below the range of fp32 (-inf; queries of -3e38 will do) the
 // others count as ever.  A key whose logits are all -inf has no energy: NaN, which no threshold keeps.  The accumulator is
 // handed back once the last batch is in registers.
-template <bool FP8, bool PARTIAL>
+template <bool FP8, int NP, bool PARTIAL>
 __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const float* sC, int nrows, uint64_t* release) {
-  constexpr int W = FP8 ? 32 : 64;   // the multipliers take registers too: FP8 with 64 spills (131072 tokens 1010 -> 1590 us)
+  uint64_t period[NP > 0 ? NP : 1];
+#pragma unroll
+  for (int k = 0; k < NP; ++k) period[k] = reinterpret_cast<const uint64_t*>(sC)[k];
+  constexpr int W = FP8 && NP == 0 ? 32 : 64;   // multipliers from shared memory take registers too: with 64 columns they spill (131072 tokens 1010 -> 1590 us)
   constexpr int kFirst = 16;
   float m = -INFINITY, total = 0.f;
   uint64_t s4[4] = {0ull, 0ull, 0ull, 0ull};   // sums of 2^(x_j - m), four independent (lo, hi) accumulators
@@ -85,7 +91,11 @@ __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const 
       tc_fence_before();
       mbar_arrive(release);
     }
-    auto mult2 = [&](int j) { return FP8 ? *reinterpret_cast<const uint64_t*>(sC + j0 + j) : f2_pack(cs, cs); };
+    auto mult2 = [&](int j) {
+      if constexpr (!FP8) return f2_pack(cs, cs);
+      else if constexpr (NP > 0) return period[((j0 + j) >> 1) % NP];
+      else return *reinterpret_cast<const uint64_t*>(sC + j0 + j);
+    };
     auto batch_max = [&](int n) {   // of the first n scaled logits
       float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -136,33 +146,40 @@ __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const 
   return total > 0.f ? m + log2f(total) : __int_as_float(0x7fc00000);
 }
 
-// Raw e4m3 rows in the second half of a query buffer -> F16 rows in both halves, in place; one warp, `rows` a multiple of 32.
-// Eight lanes take a row; the rows of a batch are in registers before the first of them is overwritten.
-__device__ __forceinline__ void widen_pair_in_place(uint8_t* half0, uint8_t* half1, int rows, int lane) {
-  for (int i0 = lane; i0 < rows * 8; i0 += 256) {
-    uint4 v[8];
+// Raw e4m3 rows in the second half of a query buffer -> F16 rows in both halves, in place; by all consumer warps, four rows of
+// 128 bytes per warp and step.  Eight lanes take a row; a warp's rows are in registers before the first of them is overwritten.
+// The conversion runs at an eighth of the issue rate, on the pipe of the exponentials: spread over the schedulers it costs each an
+// eighth of what the exponentials of one chunk do.
+__device__ __forceinline__ void widen_pair_in_place(uint8_t* half0, uint8_t* half1, int rows, int warp, int lane) {
+  constexpr int kStep = 16 * kPairGroups;   // rows per step
+  const int c = lane & 7;
+  uint8_t* const half = c < 4 ? half0 : half1;
+#pragma unroll 1
+  for (int row0 = warp * 4 + (lane >> 3); row0 - (lane >> 3) < rows; row0 += 2 * kStep) {
+    uint4 v[2];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * 32;
-      v[u] = *reinterpret_cast<const uint4*>(half1 + sw128_offset(i >> 3, i & 7));
-    }
+    for (int u = 0; u < 2; ++u)
+      if (row0 + u * kStep < rows) v[u] = *reinterpret_cast<const uint4*>(half1 + sw128_offset(row0 + u * kStep, c));
     __syncwarp();
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * 32, row = i >> 3, c = i & 7;
-      uint8_t* half = c < 4 ? half0 : half1;
-      *reinterpret_cast<uint4*>(half + sw128_offset(row, (c & 3) * 2)) =
-          make_uint4(e4m3x2_to_f16x2(v[u].x), e4m3x2_to_f16x2(v[u].x >> 16), e4m3x2_to_f16x2(v[u].y),
-                     e4m3x2_to_f16x2(v[u].y >> 16));
-      *reinterpret_cast<uint4*>(half + sw128_offset(row, (c & 3) * 2 + 1)) =
-          make_uint4(e4m3x2_to_f16x2(v[u].z), e4m3x2_to_f16x2(v[u].z >> 16), e4m3x2_to_f16x2(v[u].w),
-                     e4m3x2_to_f16x2(v[u].w >> 16));
-    }
-    __syncwarp();
+    for (int u = 0; u < 2; ++u)
+      if (row0 + u * kStep < rows) {
+        const int row = row0 + u * kStep;
+        *reinterpret_cast<uint4*>(half + sw128_offset(row, (c & 3) * 2)) =
+            make_uint4(e4m3x2_to_f16x2(v[u].x), e4m3x2_to_f16x2(v[u].x >> 16), e4m3x2_to_f16x2(v[u].y),
+                       e4m3x2_to_f16x2(v[u].y >> 16));
+        *reinterpret_cast<uint4*>(half + sw128_offset(row, (c & 3) * 2 + 1)) =
+            make_uint4(e4m3x2_to_f16x2(v[u].z), e4m3x2_to_f16x2(v[u].z >> 16), e4m3x2_to_f16x2(v[u].w),
+                       e4m3x2_to_f16x2(v[u].w >> 16));
+      }
   }
 }
 
-template <bool FP8>
+// NP: FP8 plans whose row multipliers repeat every 2 NP rows of a tile (4: the group size divides 8, 7: it is 7) hold them in
+// registers, NP pairs; 0: read from shared memory (other group sizes, such as 5 or 16).  Read for every pair of columns they are a
+// load each, which waits behind the operands of the MMAs, and leave no room for batches of 64 columns.  Whole calls, from shared
+// memory / so: 12000 tokens, lists and export, 78.4 / 77.4 us, 8191 tokens 180.8 / 178.8, 16 sequences 3285 / 3260.
+template <bool FP8, int NP>
 __global__ void __launch_bounds__(kPairThreads, 1)
 score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_constant__ CUtensorMap map_klo,
                   const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_q2,
@@ -200,9 +217,9 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
       mbar_init(&info_empty[i], 2 + kPairConsumers + 1);   // producer, issuer, consumers, selection warp
     }
     for (int i = 0; i < kPairQBufs; ++i) {
-      mbar_init(&q_full[i], 1);
+      mbar_init(&q_full[i], FP8 ? 4 * kPairGroups : 1);   // FP8: the consumer warps, which widen the tiles
       mbar_init(&q_empty[i], 1);
-      mbar_init(&raw_full[i], 1);
+      mbar_init(&raw_full[i], 2);   // the box, and the unit's multipliers in sC
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&e_full[i], kPairConsumers);
@@ -271,11 +288,7 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
         for (int j = lane; j < nt * kTileRows; j += 32)   // (adjacent tiles: row j of the pair is packed row r0 + j)
           sC[slot][j] = P.scale_log2 * q_scale[sg.h * P.group + (sg.r0 + j) % P.group];
         __syncwarp();
-        live &= mbar_wait(&raw_full[qb], (k / kPairQBufs) & 1, ctx, 114);
-        widen_pair_in_place(buf, buf + kPairQHalf, nt * kTileRows, lane);
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&q_full[qb]);
+        if (lane == 0 && live) mbar_arrive(&raw_full[qb]);
       } else if (lane == 0 && live) {
         mbar_arrive_expect_tx(&q_full[qb], rows * 256u);
         tma_load_3d_hint(buf - lead * 128, mp, &q_full[qb], 0, sg.h * P.group, sg.q_tok0 + tok0, pol);
@@ -400,10 +413,25 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
     uint32_t gc0 = 0;  // chunks of all earlier units
     int turn = 0;      // warpgroup whose turn the next item (chunk, tile) is
     bool prev_big = false;
+    // FP8: the tiles of unit k from e4m3 to F16, for the MMAs.  Done one unit ahead, when the unit's raw box has had the time
+    // of a unit's last chunk to land.
+    auto widen_unit = [&](int k) {
+      const PairInfo& pk = info[k % kPairInfoSlots];
+      const int qb = k % kPairQBufs;
+      if (!ready_warp(&info_full[k % kPairInfoSlots], (k / kPairInfoSlots) & 1, ctx, 145, &pk.valid)) return;
+      mbar_wait(&raw_full[qb], (k / kPairQBufs) & 1, ctx, 114);
+      uint8_t* const buf = sQ + qb * kPairQBytes;
+      widen_pair_in_place(buf, buf + kPairQHalf, pk.nt * kTileRows, warp, lane);
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&q_full[qb]);
+    };
+    if constexpr (FP8) widen_unit(0);
     for (int it = 0;; ++it) {
       const int slot = it % kPairInfoSlots;
       const PairInfo& pi = info[slot];
       if (!ready_warp(&info_full[slot], (it / kPairInfoSlots) & 1, ctx, 141, &pi.valid)) break;
+      if constexpr (FP8) widen_unit(it + 1);
       const int nt = pi.nt;
       const int nchunks = unit_chunks(pi);
       const int ncand0 = pi.sg[0].J_hi + 1, ncand1 = nt > 1 ? pi.sg[1].J_hi + 1 : 0;
@@ -439,8 +467,8 @@ score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_cons
         const int nrows = tt ? nrows1 : nrows0;
         const uint32_t lane_addr = lane_base + a * 256 + tt * 128;
         const float* mult = &sC[FP8 ? slot : 0][FP8 ? tt * kTileRows : 0];
-        const float e = nrows == kTileRows ? score_cols<FP8, false>(lane_addr, cs, mult, kTileRows, &acc_empty[a])
-                                           : score_cols<FP8, true>(lane_addr, cs, mult, nrows, &acc_empty[a]);
+        const float e = nrows == kTileRows ? score_cols<FP8, NP, false>(lane_addr, cs, mult, kTileRows, &acc_empty[a])
+                                           : score_cols<FP8, NP, true>(lane_addr, cs, mult, nrows, &acc_empty[a]);
         if (J < (tt ? ncand1 : ncand0)) {
           (tt ? e1 : e0)[J] = e;
           if (tt) lmax1 = fmaxf(lmax1, e);

@@ -285,6 +285,26 @@ def test_fp8_query_scales_far_apart_within_a_group(g, hkv, seqs):
     full_pipeline(spec, edit_case=spread)
 
 
+@pytest.mark.parametrize("g,hkv", [(1, 4), (2, 4), (8, 3), (7, 5), (16, 1)])
+def test_fp8_row_multipliers_and_tiles_of_pairs(g, hkv):
+    """FP8 scorer: row multipliers in registers (group sizes that divide 8, and 7) or in shared memory (16), with scales of their own
+    for every head; query tiles widened one unit ahead, in pairs and singly, ragged last tiles.  The tiles outnumber the SMs,
+    so that a CTA takes several units and both query buffers come round."""
+    lq = 128 * (160 // hkv + 1) // g + 37                # more tiles than SMs, the last one ragged
+    spec = inputs.small_spec(seqs=[(lq + 200, 200), (61, 0), (1300, 1290)], num_q_heads=g * hkv, num_kv_heads=hkv, page_size=16,
+                             dtype="fp8", config_id=240 + g)
+    spec.alpha = 0.3
+
+    def spread(case):
+        case.q_scale[:] *= torch.linspace(0.5, 2.0, g * hkv)
+
+    case, dc, wl = make(spec, edit_case=spread)
+    assert dc.plan.num_segments > torch.cuda.get_device_properties(0).multi_processor_count
+    dc.select()
+    dc.status()
+    check_lists(dc, wl)
+
+
 def test_config4_relative_at_16k():
     spec = inputs.config_spec(4, scale_down=8)
     full_pipeline(spec)
