@@ -498,38 +498,48 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         }
         return pid;
       };
-      // hidden columns of a masked iteration -> sBias (see there); row j = lane * 4 + u gets 32 bytes of which the
-      // first nh(u) are -57344 (e5m2 0xfb).  The S = Q K^T that last read sBias has completed (wait 302).  One copy, and a loop,
-      // for the instruction cache: what the roles of a CTA run per iteration and unit does not fit into the SM's, and every
+      // hidden columns of a masked iteration -> sBias (see there); row j = lane * 4 + u gets 32 bytes of which those of the
+      // positions it is hidden from, the first ones, are -57344 (e5m2 0xfb).  The S = Q K^T that last read sBias has completed
+      // (wait 302).  In little code, for the instruction cache: what the roles of a CTA run per iteration and unit does not fit into the SM's, and every
       // kilobyte less tells where units are short.  This and the shorter waits (see mbar_wait), 7 KB of code: requests to the next
       // cache level 453 -> 323 thousand (8191 tokens FP8), whole calls 24 short sequences 156.7 / 151.6 us, 8191 tokens FP8
       // 185.2 / 180.3, 2048 tokens 32.9 / 32.4, 16 sequences 3552 / 3516, FP8 3251 / 3189; long and dense calls within 1 %.
-      auto write_bias = [&](auto nh) {
-#pragma unroll 1
-        for (int u = 0; u < 4; ++u) {
-          const int j = lane * 4 + u;
-          const int sh = 32 - 8 * nh(u);   // bits of word 0 that stay clear; of word k 32 k more
-          uint32_t w[8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) w[k] = __funnelshift_rc(0xfbfbfbfbu, 0u, (uint32_t)max(0, sh + 32 * k));
-          uint8_t* dst = sBias + (j >> 3) * 256 + (j & 7) * 16;
-          *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-          *reinterpret_cast<uint4*>(dst + 128) = make_uint4(w[4], w[5], w[6], w[7]);
-        }
-        fence_proxy_async();
-        __syncwarp();
+      auto bias_row = [&](int u, const uint32_t (&w)[8]) {
+        const int j = lane * 4 + u;
+        uint8_t* dst = sBias + (j >> 3) * 256 + (j & 7) * 16;
+        *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(dst + 128) = make_uint4(w[4], w[5], w[6], w[7]);
       };
       int pid_next = fetch_pid(ti.it_begin);
       for (int i = ti.it_begin; i < ti.it_end; ++i, ++G) {
         const int pid = pid_next;
         const int J_cur = J_fetched;
         if (G >= 1) live &= mbar_wait(&s_done, (G - 1) & 1, ctx, 302);   // K stage free
-        if (i >= T || (i < ti.ndiag && P.diag_mma)) {
-          // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c; correction chunk: from
-          // all positions unless block j is to be corrected
-          const uint32_t todo = i < T ? 0u : ti.todo[ti.chunk_id[i - T]][lane >> 3] >> ((lane * 4) & 31);
-          const int t0 = i < T ? sg.pre + sg.r0 / g - J_cur * kBlock : 0;
-          write_bias([&](int u) { return i < T ? max(0, min(32, lane * 4 + u - t0)) : (todo >> u) & 1u ? 0 : 32; });
+        const bool diag = i < ti.ndiag && P.diag_mma;
+        if (i >= T) {
+          // correction chunk: hidden from all positions unless block j is to be corrected.  Unrolled: the chunk's copies wait for
+          // it (as a loop / so, whole calls: 131072 tokens 10761 / 10746 us, FP8 7724 / 7685, 16 sequences 3609 / 3596)
+          const uint32_t todo = ti.todo[ti.chunk_id[i - T]][lane >> 3] >> ((lane * 4) & 31);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const uint32_t x = (todo >> u) & 1u ? 0u : 0xfbfbfbfbu;
+            bias_row(u, {x, x, x, x, x, x, x, x});
+          }
+        } else if (diag) {
+          // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c
+          const int t0 = sg.pre + sg.r0 / g - J_cur * kBlock;
+#pragma unroll 1
+          for (int u = 0; u < 4; ++u) {
+            const int sh = 32 - 8 * max(0, min(32, lane * 4 + u - t0));   // bits of word 0 that stay clear; of word k 32 k more
+            uint32_t w[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) w[k] = __funnelshift_rc(0xfbfbfbfbu, 0u, (uint32_t)max(0, sh + 32 * k));
+            bias_row(u, w);
+          }
+        }
+        if (i >= T || diag) {
+          fence_proxy_async();
+          __syncwarp();
         }
         if (i < T) {
           const int nvalid = __popc(__ballot_sync(0xffffffffu, pid >= 0));
