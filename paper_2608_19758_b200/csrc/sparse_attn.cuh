@@ -500,10 +500,12 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       };
       // hidden columns of a masked iteration -> sBias (see there); row j = lane * 4 + u gets 32 bytes of which those of the
       // positions it is hidden from, the first ones, are -57344 (e5m2 0xfb).  The S = Q K^T that last read sBias has completed
-      // (wait 302).  In little code, for the instruction cache: what the roles of a CTA run per iteration and unit does not fit into the SM's, and every
-      // kilobyte less tells where units are short.  This and the shorter waits (see mbar_wait), 7 KB of code: requests to the next
-      // cache level 453 -> 323 thousand (8191 tokens FP8), whole calls 24 short sequences 156.7 / 151.6 us, 8191 tokens FP8
-      // 185.2 / 180.3, 2048 tokens 32.9 / 32.4, 16 sequences 3552 / 3516, FP8 3251 / 3189; long and dense calls within 1 %.
+      // (wait 302).  Written behind the K tile's copies, which do not wait for it: k_full completes only with the arrival
+      // behind the mask, whatever has landed by then.  In front of the copies / behind them, whole calls in us, in turn (15 rounds):
+      // 131072 tokens 10593 / 10553, the last 8192 of them 1378 / 1370, 32768 tokens dense 7671 / 7644, the last 512 of them 362.5 /
+      // 354.2, 24 short sequences 153.1 / 152.1, 8191 tokens FP8 170.2 / 171.9, 16384 tokens dense FP8 1449 / 1452; other calls
+      // within 0.4 %.  As little code as that takes, for the instruction cache (with both masks unrolled, 16384 tokens dense FP8
+      // +1 %, 24 short sequences +1 %).
       auto bias_row = [&](int u, const uint32_t (&w)[8]) {
         const int j = lane * 4 + u;
         uint8_t* dst = sBias + (j >> 3) * 256 + (j & 7) * 16;
@@ -515,41 +517,30 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         const int pid = pid_next;
         const int J_cur = J_fetched;
         if (G >= 1) live &= mbar_wait(&s_done, (G - 1) & 1, ctx, 302);   // K stage free
-        const bool diag = i < ti.ndiag && P.diag_mma;
-        if (i >= T) {
-          // correction chunk: hidden from all positions unless block j is to be corrected.  Unrolled: the chunk's copies wait for
-          // it (as a loop / so, whole calls: 131072 tokens 10761 / 10746 us, FP8 7724 / 7685, 16 sequences 3609 / 3596)
-          const uint32_t todo = ti.todo[ti.chunk_id[i - T]][lane >> 3] >> ((lane * 4) & 31);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint32_t x = (todo >> u) & 1u ? 0u : 0xfbfbfbfbu;
-            bias_row(u, {x, x, x, x, x, x, x, x});
-          }
-        } else if (diag) {
-          // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c
-          const int t0 = sg.pre + sg.r0 / g - J_cur * kBlock;
-#pragma unroll 1
-          for (int u = 0; u < 4; ++u) {
-            const int sh = 32 - 8 * max(0, min(32, lane * 4 + u - t0));   // bits of word 0 that stay clear; of word k 32 k more
-            uint32_t w[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) w[k] = __funnelshift_rc(0xfbfbfbfbu, 0u, (uint32_t)max(0, sh + 32 * k));
-            bias_row(u, w);
-          }
-        }
-        if (i >= T || diag) {
-          fence_proxy_async();
-          __syncwarp();
-        }
         if (i < T) {
           const int nvalid = __popc(__ballot_sync(0xffffffffu, pid >= 0));
-          if constexpr (FP8) {
-            // raw e4m3 K tile, 128 bytes per token row, straight into the K stage (the MMA reads it as it lands)
-            const uint32_t bytes = (uint32_t)nvalid * psz * 128u;
-            if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, bytes);
+          const uint32_t bytes = (uint32_t)nvalid * psz * (FP8 ? 128u : 256u);
+          if (pid >= 0 && live) {   // (FP8: the raw e4m3 tile, which the MMA reads as it lands)
+            tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
+            if constexpr (!FP8) tma_load_3d_hint(sK + 16384 + lane * psz * 128, &map_k, &k_full, 64, sg.h, pid * psz, keep);
+          }
+          if (i < ti.ndiag && P.diag_mma) {
+            // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c
+            const int t0 = sg.pre + sg.r0 / g - J_cur * kBlock;
+#pragma unroll 1
+            for (int u = 0; u < 4; ++u) {
+              const int sh = 32 - 8 * max(0, min(32, lane * 4 + u - t0));   // bits of word 0 that stay clear; of word k 32 k more
+              uint32_t w[8];
+#pragma unroll
+              for (int k = 0; k < 8; ++k) w[k] = __funnelshift_rc(0xfbfbfbfbu, 0u, (uint32_t)max(0, sh + 32 * k));
+              bias_row(u, w);
+            }
+            fence_proxy_async();
             __syncwarp();
-            if (pid >= 0 && live) tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
-            pid_next = fetch_pid(i + 1);
+          }
+          if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, bytes);
+          pid_next = fetch_pid(i + 1);   // (it waits for the loads: behind the arrival)
+          if constexpr (FP8) {
             if constexpr (WIDEN) {
               if (rc >= 1) live &= mbar_wait(&vraw_empty, (rc - 1) & 1, ctx, 306);
               if (lane == 0 && live) mbar_arrive_expect_tx(&vraw_full, bytes);
@@ -567,14 +558,6 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
               __syncwarp();
             }
           } else {
-            const uint32_t bytes = (uint32_t)nvalid * psz * 256u;
-            if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, bytes);
-            __syncwarp();
-            if (pid >= 0 && live) {
-              tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
-              tma_load_3d_hint(sK + 16384 + lane * psz * 128, &map_k, &k_full, 64, sg.h, pid * psz, keep);
-            }
-            pid_next = fetch_pid(i + 1);
             if (G >= 1) live &= wait_pv(G - 1, 303);  // V stage free
             if (lane == 0 && live) mbar_arrive_expect_tx(&v_full, bytes);
             __syncwarp();
@@ -587,7 +570,6 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
           const int cid = ti.chunk_id[i - T];
           const int row0 = sg.blk_off + cid * 128;
           if (lane == 0 && live) {
-            mbar_arrive_expect_tx(&k_full, kTileBytes);
             if constexpr (FP8) {   // e4m3 hi | lo, 16 KB each
               tma_load_3d_hint(sK, &map_kbar, &k_full, 0, sg.h, row0, keep);
               tma_load_3d_hint(sK + 16384, &map_kbar_lo, &k_full, 0, sg.h, row0, keep);
@@ -596,6 +578,16 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
               tma_load_3d_hint(sK + 16384, &map_kbar, &k_full, 64, sg.h, row0, keep);
             }
           }
+          // hidden from all positions unless block j is to be corrected
+          const uint32_t todo = ti.todo[cid][lane >> 3] >> ((lane * 4) & 31);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const uint32_t x = (todo >> u) & 1u ? 0u : 0xfbfbfbfbu;
+            bias_row(u, {x, x, x, x, x, x, x, x});
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, kTileBytes);
           if (G >= 1) live &= wait_pv(G - 1, 305);    // V stage free
           if (lane == 0 && live) {
             if constexpr (WIDEN) mbar_arrive_n(&v_full, 3);
