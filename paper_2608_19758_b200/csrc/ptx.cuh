@@ -1,7 +1,7 @@
 // Thin inline-PTX wrappers for sm_100a: mbarrier, TMA (cp.async.bulk.tensor), tcgen05 (TMEM
 // allocation, UMMA issue/commit, TMEM load/store), shared-memory matrix descriptors.
-// Every wait is bounded: after a cycle budget it records a status word and lets the caller continue.  That bounds a kernel
-// only if what follows a failed wait is bounded too, so: no role reads a descriptor that it has not been handed (see
+// Every wait is bounded: after a cycle budget it leaves its site in the CTA's abort flag and lets the caller continue; the status
+// block says so once the CTA is on its way out (leave_cta).  That bounds a kernel only if what follows a failed wait is bounded too, so: no role reads a descriptor that it has not been handed (see
 // ready_warp), and nothing that waits for other threads without a bound (a full-mask vote, a CTA barrier) follows a decision
 // that those threads may take differently.
 #pragma once
@@ -17,10 +17,13 @@ namespace fp2 {
 // Layout of the device status block (int32 words) kept in the caller's workspace.
 enum : int { ST_TIMEOUT = 0, ST_WHERE = 1, ST_BAD_LIST = 2, ST_WORDS = 8 };
 
-// Cycle budget of one wait (about one second at 2 GHz), below 2^32.
+// Cycle budget of one wait (about one second at 2 GHz).  A wait reads the 32-bit clock every 256 polls and compares its
+// distance from the start, modulo 2^32: up to 2^31 the distance stays above an expired budget for another 2^31 cycles, a second and
+// more, in which one of the readings is sure to fall; a budget near 2^32 might never be seen to expire, a larger one would be cut.
 #ifndef FP2_WAIT_CYCLES
 #define FP2_WAIT_CYCLES (2000000000u)
 #endif
+static_assert((FP2_WAIT_CYCLES) > 0 && (FP2_WAIT_CYCLES) <= 0x80000000u, "FP2_WAIT_CYCLES: 1 to 2^31 cycles");
 
 struct WaitCtx {
   int* status;           // global status block
@@ -71,10 +74,10 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Waits until the phase with the given parity has completed.  Bounded: on expiry the status
-// block records the site and the CTA-wide abort flag makes all later waits fall through.  False: the phase has not completed.
-// (Inlined at some forty places of a kernel, so what it does after an expiry is kept short: the abort flag holds the site until
-// leave_cta puts it into the status block.)
+// Waits until the phase with the given parity has completed.  Bounded: on expiry the CTA-wide abort flag takes the site and makes
+// all later waits fall through.  False: the phase has not completed.
+// (Inlined at some forty places of a kernel, so what it does after an expiry is kept short: leave_cta puts the site into the
+// status block.  Of waits that run out together, between one's look at the flag and its write, the last one's site stays.)
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtx& ctx, int where) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint32_t t0 = clock();

@@ -3,6 +3,8 @@ the host, and its planner agrees with the oracle's geometry.  No kernel is launc
 import ctypes as C
 import os
 import re
+import shutil
+import subprocess
 
 import numpy as np
 import pytest
@@ -159,3 +161,18 @@ def test_pool_carry_count_is_host_only_and_counts_complete_blocks():
     assert binding.fp2_pool_carry_count(dst, src, [0, -1, 1, 2]) == [7, 0, 2, 1]
     with pytest.raises(binding.Fp2Error):
         binding.fp2_pool_carry_count(dst, src, [5, -1, 1, 2])          # no such source sequence
+
+
+@pytest.mark.parametrize("budget,ok", [("2000000000u", True), ("0x80000000u", True), ("1", True), ("0", False), ("-1", False),
+                                       ("0x80000001u", False), ("5000000000ll", False)])
+def test_budgets_of_a_wait_that_a_32_bit_clock_cannot_hold_do_not_compile(budget, ok, tmp_path):
+    """A wait compares 32-bit clock differences with its budget: values that would be cut, or whose expiry could be missed before
+    the difference wraps, are refused when the library is compiled."""
+    src = tmp_path / "wait.cu"
+    src.write_text('#include "ptx.cuh"\n')
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    r = subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", f"-DFP2_WAIT_CYCLES={budget}", "-I",
+                        os.path.join(ROOT, "paper_2608_19758_b200", "csrc"), "-c", "-o", str(tmp_path / "wait.o"), str(src)],
+                       capture_output=True, text=True)
+    assert (r.returncode == 0) == ok, r.stderr
+    assert ok or "FP2_WAIT_CYCLES" in r.stderr
