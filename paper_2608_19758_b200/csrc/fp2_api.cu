@@ -404,12 +404,22 @@ static bool make_q_map(fp2_plan* pl, CUtensorMap* m, const void* q, int box_toke
   return r == CUDA_SUCCESS;
 }
 
+// The paired scorer of a plan: FP8 by the number of row pairs after which the heads of a tile, and with them the rows' multipliers,
+// repeat (see score_pair_kernel).
+static auto pair_kernel(const DevParams& d) -> decltype(&score_pair_kernel<false, 0>) {
+  if (!d.fp8) return score_pair_kernel<false, 0>;
+  const int pairs = d.group % 2 ? d.group : d.group / 2;
+  if (4 % pairs == 0) return score_pair_kernel<true, 4>;
+  if (pairs == 3) return score_pair_kernel<true, 3>;
+  if (pairs == 5) return score_pair_kernel<true, 5>;
+  if (pairs == 7) return score_pair_kernel<true, 7>;
+  return score_pair_kernel<true, 0>;
+}
+
 static fp2_status set_attrs(fp2_plan* pl) {
   if (pl->attrs_set) return FP2_OK;
-  for (auto kernel : {score_pair_kernel<false, 0>, score_pair_kernel<true, 0>, score_pair_kernel<true, 4>, score_pair_kernel<true, 7>})
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) != cudaSuccess)
-      return FP2_ERR_CUDA;
-  if (cudaFuncSetAttribute(score_select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(pair_kernel(pl->dev), cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) != cudaSuccess ||
+      cudaFuncSetAttribute(score_select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kScoreSmemBytes) != cudaSuccess ||
       cudaFuncSetAttribute(score_select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kScoreSmemBytes) != cudaSuccess ||
@@ -528,10 +538,7 @@ extern "C" fp2_status fp2_select_blocks(fp2_plan* pl, const void* q, const void*
   int* status = reinterpret_cast<int*>(ws + pl->ws_status);
   if (pl->dev.q_box) {
     // pairs of adjacent tiles per pooled-key chunk, in pieces of 64 elements x 128 keys (the box of mhi / mlo)
-    const int g = pl->dev.group;
-    auto kernel = !pl->dev.fp8 ? score_pair_kernel<false, 0> : 8 % g == 0 ? score_pair_kernel<true, 4>
-                               : g == 7 ? score_pair_kernel<true, 7> : score_pair_kernel<true, 0>;
-    launch(kernel,
+    launch(pair_kernel(pl->dev),
            (unsigned)(pl->nunits < pl->num_sms ? pl->nunits : pl->num_sms), kPairThreads, kPairSmemBytes, st, mhi, mlo, mq, mq2,
            pl->d_segs, pl->d_units, pl->nunits, qs, pl->dev, seg_offset, seg_count, blk_idx, status);
   } else {

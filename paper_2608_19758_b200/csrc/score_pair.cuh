@@ -175,10 +175,14 @@ __device__ __forceinline__ void widen_pair_in_place(uint8_t* half0, uint8_t* hal
   }
 }
 
-// NP: FP8 plans whose row multipliers repeat every 2 NP rows of a tile (4: the group size divides 8, 7: it is 7) hold them in
-// registers, NP pairs; 0: read from shared memory (other group sizes, such as 5 or 16).  Read for every pair of columns they are a
-// load each, which waits behind the operands of the MMAs, and leave no room for batches of 64 columns.  Whole calls, from shared
-// memory / so: 12000 tokens, lists and export, 78.4 / 77.4 us, 8191 tokens 180.8 / 178.8, 16 sequences 3285 / 3260.
+// NP: FP8 plans whose heads repeat every NP pairs of rows of a tile hold the row multipliers in registers, NP pairs: 4 (group sizes
+// that divide 8), 3 (3, 6), 5 (5, 10), 7 (7); 0: read from shared memory (9, 16 and more; more pairs would take registers that the
+// columns need).  Read for every pair of columns they are a load each, which waits behind the operands of the MMAs, and leave no
+// room for batches of 64 columns.  The registers are full: NP 3 and 4 spill 4 and 12 bytes, 5 and 7 12 and 16; with batches of 32
+// nothing spills.  Lists and export of FP8 calls in us, in turn, from shared memory / registers and 32 columns / and 64: 12000
+// tokens, groups of 3, 4, 5, 6 and 7: 54.2 / 51.9 / 50.8, 63.0 / 60.6 / 57.9, 74.9 / 72.1 / 67.8, 49.7 / 48.1 / 47.3, 55.0 / 53.2 / 51.3; 65536
+// tokens 339 / 324 / 318, 435 / 417 / 406, 527 / 501 / 487, 314 / 301 / 296, 352 / 336 / 334.  Select + sparse of 16 sequences, groups of
+// 4, 3273 / 3233 / 3211, 131072 tokens, groups of 7, 7644 / 7611 / 7602, 8191 tokens 174.0 / 172.3 / 172.0.
 template <bool FP8, int NP>
 __global__ void __launch_bounds__(kPairThreads, 1)
 score_pair_kernel(const __grid_constant__ CUtensorMap map_khi, const __grid_constant__ CUtensorMap map_klo,
