@@ -285,21 +285,26 @@ def test_fp8_query_scales_far_apart_within_a_group(g, hkv, seqs):
     full_pipeline(spec, edit_case=spread)
 
 
-@pytest.mark.parametrize("g,hkv", [(1, 4), (2, 4), (8, 3), (7, 5), (16, 1)])
-def test_fp8_row_multipliers_and_tiles_of_pairs(g, hkv):
-    """FP8 scorer: row multipliers in registers (group sizes that divide 8, and 7) or in shared memory (16), with scales of their own
-    for every head; query tiles widened one unit ahead, in pairs and singly, ragged last tiles.  The tiles outnumber the SMs,
-    so that a CTA takes several units and both query buffers come round."""
-    lq = 128 * (160 // hkv + 1) // g + 37                # more tiles than SMs, the last one ragged
-    spec = inputs.small_spec(seqs=[(lq + 200, 200), (61, 0), (1300, 1290)], num_q_heads=g * hkv, num_kv_heads=hkv, page_size=16,
-                             dtype="fp8", config_id=240 + g)
+@pytest.mark.parametrize("g", [1, 2, 3, 5, 7, 8, 9, 10, 16])
+def test_fp8_row_multipliers_and_tiles_of_pairs(g):
+    """FP8 scorer: row multipliers in registers (group sizes that divide 8, and 3, 5, 7, 10) or in shared memory (9, 16), with scales
+    of their own for every head; query tiles widened one unit ahead, in pairs and singly, ragged last tiles.  There are five
+    units for every CTA, so that both query buffers, both phases of their barriers and all four descriptors come round."""
+    hkv, sms = 8, torch.cuda.get_device_properties(0).multi_processor_count
+    lq = 10 * sms // hkv * 128 // g + 37
+    while lq * g % 128 == 0 or -(-lq * g // 128) % 2 == 0:
+        lq += 1                                          # a ragged last tile, one tile without a partner
+    seqs = [(lq + 200, 200), (61, 0), (1300, 1290)]
+    spec = inputs.small_spec(seqs=seqs, num_q_heads=g * hkv, num_kv_heads=hkv, page_size=16, dtype="fp8", config_id=240 + g)
     spec.alpha = 0.3
 
     def spread(case):
         case.q_scale[:] *= torch.linspace(0.5, 2.0, g * hkv)
 
     case, dc, wl = make(spec, edit_case=spread)
-    assert dc.plan.num_segments > torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = [-(-(n - pre) * g // 128) for n, pre in seqs]
+    assert dc.plan.num_segments == hkv * sum(tiles) > sms                     # so tiles are paired (all lists are short)
+    assert hkv * sum(-(-t // 2) for t in tiles) >= 5 * sms
     dc.select()
     dc.status()
     check_lists(dc, wl)
@@ -739,8 +744,8 @@ def test_scores_far_above_those_of_the_first_rows(first_loud, dtype):
 # per row of a tile: by how much its logits (log2) stand above those of the first 16 rows
 LOUD = {
     "from16": lambda j: 170.0 if j >= 16 else 0.0,          # first batch, all of it
-    "from40": lambda j: 170.0 if j >= 40 else 0.0,          # FP8: second batch of 32; BF16: first of 64
-    "from70": lambda j: 170.0 if j >= 70 else 0.0,          # FP8: third; BF16: second
+    "from40": lambda j: 170.0 if j >= 40 else 0.0,          # second batch of 32, first of 64
+    "from70": lambda j: 170.0 if j >= 70 else 0.0,          # third, second
     "from100": lambda j: 170.0 if j >= 100 else 0.0,        # the last batch
     "once": lambda j: 170.0 if j == 77 else 0.0,            # one row, the others behind it quiet again
     "stairs": lambda j: 150.0 * (j // 32),                  # every batch of 32, or of 64, once more above the one before
@@ -748,15 +753,16 @@ LOUD = {
 }
 
 
-@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("dtype,g", [("bf16", 32), ("fp8", 32), ("fp8", 4), ("fp8", 7), ("fp8", 3), ("fp8", 5)])
 @pytest.mark.parametrize("shape", list(LOUD))
-def test_scores_that_leave_the_reference_behind_in_a_given_batch(shape, dtype):
-    """The scorer goes through a tile's 128 rows in batches (64, FP8: 32) against the maximum of the first 16, and a batch that
-    comes out above 2^119 is done again against its own maximum, the sum so far scaled down.  Here one dimension of every key
-    holds a constant c and the queries' entry there sets a row's level, so which batches that happens in is known: asserted from
-    the oracle's logits.  A tile is 4 tokens x 32 heads; pairs, a single tile, and a last tile of 3 tokens.  No block is forced
-    into a list."""
-    spec = inputs.small_spec(seqs=[(5000, 4001), (902, 3)], num_q_heads=32, num_kv_heads=1, page_size=32, dtype=dtype,
+def test_scores_that_leave_the_reference_behind_in_a_given_batch(shape, dtype, g):
+    """The scorer goes through a tile's 128 rows in batches (64; FP8 with row multipliers in shared memory, here groups of 32: 32)
+    against the maximum of the first 16, and a batch that comes out above 2^119 is done again against its own maximum, the sum so
+    far scaled down.  Here one dimension of every key holds a constant c and the queries' entry there sets a row's level, so which
+    batches that happens in is known: asserted from the oracle's logits.  Groups of 32: a tile is 4 tokens x 32 heads; pairs, a
+    single tile, and a last tile of 3 tokens.  Smaller groups: single tiles, a last one of a few rows.  No block is forced into a
+    list."""
+    spec = inputs.small_spec(seqs=[(5000, 4001), (902, 3)], num_q_heads=g, num_kv_heads=1, page_size=32, dtype=dtype,
                              config_id=200, locality_a=0.5)
     spec.alpha = 0.3
 
@@ -769,16 +775,16 @@ def test_scores_that_leave_the_reference_behind_in_a_given_batch(shape, dtype):
             q = case.q.float()
         cu = case.cu_seqlens_q.tolist()
         for b in range(2):
-            r = torch.arange((cu[b + 1] - cu[b]) * 32)
+            r = torch.arange((cu[b + 1] - cu[b]) * g)
             lv = torch.tensor([LOUD[shape](int(j) % 128) for j in r])
-            q[cu[b]:cu[b + 1], :, 0] = (lv / (c * 128 ** -0.5 * np.log2(np.e))).view(-1, 32)
+            q[cu[b]:cu[b + 1], :, 0] = (lv / (c * 128 ** -0.5 * np.log2(np.e))).view(-1, g)
         if dtype == "fp8":
             case.q_scale[:] = q.abs().amax() / 448.0
             case.q[:] = inputs.quantize_e4m3(q, case.q_scale[None, :, None])
         else:
             case.q[:] = q.to(torch.bfloat16)
     case, dc, wl = make(spec, edit_case=levels, sink_tokens=0, window_tokens=0)
-    W = 32 if dtype == "fp8" else 64
+    W = 32 if dtype == "fp8" and g == 32 else 64
     redone = {}
     for s in wl.segs:
         x = O.tile_queries(wl.q_seq(s.b), wl.p, s) @ wl.kv(s.b, s.h)[2][:s.J_hi + 1].T * wl.p.scale * np.log2(np.e)
