@@ -500,17 +500,24 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
       };
       // hidden columns of a masked iteration -> sBias (see there); row j = lane * 4 + u gets 32 bytes of which those of the
       // positions it is hidden from, the first ones, are -57344 (e5m2 0xfb).  The S = Q K^T that last read sBias has completed
-      // (wait 302).  Written behind the K tile's copies, which do not wait for it: k_full completes only with the arrival
-      // behind the mask, whatever has landed by then.  In front of the copies / behind them, whole calls in us, in turn (15 rounds):
-      // 131072 tokens 10593 / 10553, the last 8192 of them 1378 / 1370, 32768 tokens dense 7671 / 7644, the last 512 of them 362.5 /
-      // 354.2, 24 short sequences 153.1 / 152.1, 8191 tokens FP8 170.2 / 171.9, 16384 tokens dense FP8 1449 / 1452; other calls
-      // within 0.4 %.  As little code as that takes, for the instruction cache (with both masks unrolled, 16384 tokens dense FP8
-      // +1 %, 24 short sequences +1 %).
+      // (wait 302).  As little code as that takes, for the instruction cache.
       auto bias_row = [&](int u, const uint32_t (&w)[8]) {
         const int j = lane * 4 + u;
         uint8_t* dst = sBias + (j >> 3) * 256 + (j & 7) * 16;
         *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
         *reinterpret_cast<uint4*>(dst + 128) = make_uint4(w[4], w[5], w[6], w[7]);
+      };
+      // The K tile of an iteration and its mask.  BF16: the copies go out first and do not wait for the mask; the phase of k_full
+      // completes only with the arrival behind it, whatever has landed by then.  FP8, whose tile
+      // is half as large: the mask first; the other way round dense calls are slower.  Whole calls in us, in turn, mask first /
+      // copies first: 131072 tokens 10398 / 10361, last 8192 of them 1313 / 1305, 32768 tokens dense 7584 / 7562, the last 512 of
+      // them 361.2 / 354.5, 16 sequences 3455 / 3444, 24 short sequences 151.5 / 151.1; FP8 dense 16384 tokens 1440.1 / 1447.2, 1500
+      // tokens 39.6 / 40.6, 8191 tokens 170.7 / 172.5, 131072 tokens within 0.2 %.
+      auto request_k = [&](uint32_t bytes, auto copies, auto mask) {
+        if constexpr (!FP8) copies();
+        mask();
+        if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, bytes);
+        if constexpr (FP8) copies();
       };
       int pid_next = fetch_pid(ti.it_begin);
       for (int i = ti.it_begin; i < ti.it_end; ++i, ++G) {
@@ -520,25 +527,28 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         if (i < T) {
           const int nvalid = __popc(__ballot_sync(0xffffffffu, pid >= 0));
           const uint32_t bytes = (uint32_t)nvalid * psz * (FP8 ? 128u : 256u);
-          if (pid >= 0 && live) {   // (FP8: the raw e4m3 tile, which the MMA reads as it lands)
-            tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
-            if constexpr (!FP8) tma_load_3d_hint(sK + 16384 + lane * psz * 128, &map_k, &k_full, 64, sg.h, pid * psz, keep);
-          }
-          if (i < ti.ndiag && P.diag_mma) {
-            // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c
-            const int t0 = sg.pre + sg.r0 / g - J_cur * kBlock;
-#pragma unroll 1
-            for (int u = 0; u < 4; ++u) {
-              const int sh = 32 - 8 * max(0, min(32, lane * 4 + u - t0));   // bits of word 0 that stay clear; of word k 32 k more
-              uint32_t w[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) w[k] = __funnelshift_rc(0xfbfbfbfbu, 0u, (uint32_t)max(0, sh + 32 * k));
-              bias_row(u, w);
+          request_k(bytes, [&]() {
+            if constexpr (FP8) __syncwarp();
+            if (pid >= 0 && live) {   // (FP8: the raw e4m3 tile, which the MMA reads as it lands)
+              tma_load_3d_hint(sK + lane * psz * 128, &map_k, &k_full, 0, sg.h, pid * psz, keep);
+              if constexpr (!FP8) tma_load_3d_hint(sK + 16384 + lane * psz * 128, &map_k, &k_full, 64, sg.h, pid * psz, keep);
             }
-            fence_proxy_async();
-            __syncwarp();
-          }
-          if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, bytes);
+          }, [&]() {
+            if (i < ti.ndiag && P.diag_mma) {
+              // diagonal block: column j is hidden from the tile's position c iff J * 128 + j > pre + r0 / g + c
+              const int t0 = sg.pre + sg.r0 / g - J_cur * kBlock;
+#pragma unroll 1
+              for (int u = 0; u < 4; ++u) {
+                const int sh = 32 - 8 * max(0, min(32, lane * 4 + u - t0));   // bits of word 0 that stay clear; of word k 32 k more
+                uint32_t w[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) w[k] = __funnelshift_rc(0xfbfbfbfbu, 0u, (uint32_t)max(0, sh + 32 * k));
+                bias_row(u, w);
+              }
+              fence_proxy_async();
+              __syncwarp();
+            }
+          });
           pid_next = fetch_pid(i + 1);   // (it waits for the loads: behind the arrival)
           if constexpr (FP8) {
             if constexpr (WIDEN) {
@@ -569,25 +579,26 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         } else {
           const int cid = ti.chunk_id[i - T];
           const int row0 = sg.blk_off + cid * 128;
-          if (lane == 0 && live) {
-            if constexpr (FP8) {   // e4m3 hi | lo, 16 KB each
-              tma_load_3d_hint(sK, &map_kbar, &k_full, 0, sg.h, row0, keep);
-              tma_load_3d_hint(sK + 16384, &map_kbar_lo, &k_full, 0, sg.h, row0, keep);
-            } else {
-              tma_load_3d_hint(sK, &map_kbar, &k_full, 0, sg.h, row0, keep);
-              tma_load_3d_hint(sK + 16384, &map_kbar, &k_full, 64, sg.h, row0, keep);
+          request_k(kTileBytes, [&]() {
+            if (lane == 0 && live) {
+              if constexpr (FP8) {   // e4m3 hi | lo, 16 KB each
+                tma_load_3d_hint(sK, &map_kbar, &k_full, 0, sg.h, row0, keep);
+                tma_load_3d_hint(sK + 16384, &map_kbar_lo, &k_full, 0, sg.h, row0, keep);
+              } else {
+                tma_load_3d_hint(sK, &map_kbar, &k_full, 0, sg.h, row0, keep);
+                tma_load_3d_hint(sK + 16384, &map_kbar, &k_full, 64, sg.h, row0, keep);
+              }
             }
-          }
-          // hidden from all positions unless block j is to be corrected
-          const uint32_t todo = ti.todo[cid][lane >> 3] >> ((lane * 4) & 31);
+          }, [&]() {   // hidden from all positions unless block j is to be corrected
+            const uint32_t todo = ti.todo[cid][lane >> 3] >> ((lane * 4) & 31);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint32_t x = (todo >> u) & 1u ? 0u : 0xfbfbfbfbu;
-            bias_row(u, {x, x, x, x, x, x, x, x});
-          }
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0 && live) mbar_arrive_expect_tx(&k_full, kTileBytes);
+            for (int u = 0; u < 4; ++u) {
+              const uint32_t x = (todo >> u) & 1u ? 0u : 0xfbfbfbfbu;
+              bias_row(u, {x, x, x, x, x, x, x, x});
+            }
+            fence_proxy_async();
+            __syncwarp();
+          });
           if (G >= 1) live &= wait_pv(G - 1, 305);    // V stage free
           if (lane == 0 && live) {
             if constexpr (WIDEN) mbar_arrive_n(&v_full, 3);
