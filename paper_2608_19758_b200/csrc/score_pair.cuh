@@ -28,7 +28,8 @@
 // raw row.  Every row has a multiplier of its own (q_scale), kept per unit in sC.  One warp that fetched and widened the tiles was
 // what the units waited for (8191 tokens, one chunk of keys per unit: 8900 cycles a unit, of which 5000 widening and 2100 the box).
 // Select call in us, widened by one warp / by the consumers: 8191 tokens, 28 heads on 4, 42.6 / 32.8, 12000 tokens, 32 on 8, 66.8 /
-// 48.8; lists of 12000 tokens with export 77.0 / 57.8; with attention 16 sequences 3222 / 3186, 131072 tokens the same.
+// 48.8; lists of 12000 tokens with export 77.0 / 57.8 (row multipliers in registers on both sides); with attention 16 sequences
+// 3222 / 3186, 131072 tokens the same.
 //
 // Roles: warps 0-11 consumers; warp 12 TMA producer of kbar pieces (16 KB: 128 keys x 64 elements, four per chunk: hi | lo x
 // the two halves of d); warp 13 UMMA issuer and TMEM owner; warp 14 unit set-up and query tiles by TMA (two units in flight);
@@ -148,8 +149,9 @@ __device__ __forceinline__ float score_cols(uint32_t lane_addr, float cs, const 
 
 // Raw e4m3 rows in the second half of a query buffer -> F16 rows in both halves, in place; by all consumer warps, four rows of
 // 128 bytes per warp and step.  Eight lanes take a row; a warp's rows are in registers before the first of them is overwritten.
-// The conversion runs at an eighth of the issue rate, on the pipe of the exponentials: spread over the schedulers it costs each an
-// eighth of what the exponentials of one chunk do.
+// The conversion runs at an eighth of the issue rate, on the pipe of the exponentials: 512 warp instructions for a pair, 1024
+// cycles of each scheduler's, half of what the exponentials of one chunk take, once per unit.  Where a unit has one chunk or two that
+// is a good part of it.
 __device__ __forceinline__ void widen_pair_in_place(uint8_t* half0, uint8_t* half1, int rows, int warp, int lane) {
   constexpr int kStep = 16 * kPairGroups;   // rows per step
   const int c = lane & 7;
