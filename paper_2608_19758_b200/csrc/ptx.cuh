@@ -1,9 +1,9 @@
 // Thin inline-PTX wrappers for sm_100a: mbarrier, TMA (cp.async.bulk.tensor), tcgen05 (TMEM
 // allocation, UMMA issue/commit, TMEM load/store), shared-memory matrix descriptors.
 // Every wait is bounded: after a cycle budget it leaves its site in the CTA's abort flag and lets the caller continue; the status
-// block says so once the CTA is on its way out (leave_cta).  That bounds a kernel only if what follows a failed wait is bounded too, so: no role reads a descriptor that it has not been handed (see
-// ready_warp), and nothing that waits for other threads without a bound (a full-mask vote, a CTA barrier) follows a decision
-// that those threads may take differently.
+// block says so once the CTA is on its way out (leave_cta).  That bounds a kernel only if what follows a failed wait is bounded
+// too, so: no role reads a descriptor that it has not been handed (see ready_warp), and nothing that waits for other threads
+// without a bound (a full-mask vote, a CTA barrier) follows a decision that those threads may take differently.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -77,8 +77,9 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 // Waits until the phase with the given parity has completed.  Bounded: on expiry the CTA-wide abort flag takes the site and makes
 // all later waits fall through.  False: the phase has not completed.
 // (Inlined at some forty places of a kernel, so what it does after an expiry is kept short: leave_cta puts the site into the
-// status block.  With a 64-bit clock and the status block written here, 2.5 KB more in the attention kernel, whole calls in us, so /
-// short: 32768 tokens dense 7489 / 7458, 8191 tokens FP8 170.2 / 169.0, others within 0.3 %.  Of waits that run out together, between one's look at the flag and its write, the last one's site stays.)
+// status block.  With a 64-bit clock and the status block written here, 2.5 KB more in the attention kernel, whole calls in us,
+// so / short: 32768 tokens dense 7489 / 7458, 8191 tokens FP8 170.2 / 169.0, others within 0.3 %.  Of waits that run out
+// together, between one's look at the flag and its write, the last one's site stays.)
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtx& ctx, int where) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint32_t t0 = clock();

@@ -508,11 +508,11 @@ sparse_attn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_const
         *reinterpret_cast<uint4*>(dst + 128) = make_uint4(w[4], w[5], w[6], w[7]);
       };
       // The K tile of an iteration and its mask.  BF16: the copies go out first and do not wait for the mask; the phase of k_full
-      // completes only with the arrival behind it, whatever has landed by then.  FP8, whose tile
-      // is half as large: the mask first; the other way round dense calls are slower.  Whole calls in us, in turn, mask first /
-      // copies first: 131072 tokens 10398 / 10361, last 8192 of them 1313 / 1305, 32768 tokens dense 7584 / 7562, the last 512 of
-      // them 361.2 / 354.5, 16 sequences 3455 / 3444, 24 short sequences 151.5 / 151.1; FP8 dense 16384 tokens 1440.1 / 1447.2, 1500
-      // tokens 39.6 / 40.6, 8191 tokens 170.7 / 172.5, 131072 tokens within 0.2 %.
+      // completes only with the arrival behind it, whatever has landed by then.  FP8, whose tile is half as large: the mask first;
+      // the other way round dense calls are slower.  Whole calls in us, in turn, mask first / copies first: 131072 tokens 10398 /
+      // 10361, last 8192 of them 1313 / 1305, 32768 tokens dense 7584 / 7562, the last 512 of them 361.2 / 354.5, 16 sequences
+      // 3455 / 3444, 24 short sequences 151.5 / 151.1; FP8 dense 16384 tokens 1440.1 / 1447.2, 1500 tokens 39.6 / 40.6, 8191 tokens
+      // 170.7 / 172.5, 131072 tokens within 0.2 %.
       auto request_k = [&](uint32_t bytes, auto copies, auto mask) {
         if constexpr (!FP8) copies();
         mask();
